@@ -1,10 +1,11 @@
-"""ctypes binding of libb2blas.so: argument marshalling only.
+"""Python binding of libb2blas.so: argument marshalling only.
 
 Every routine of ``include/b2blas.h`` is exposed twice:
 
-* ``lib().b2_saxpy`` etc. -- the raw C symbols with their prototypes set;
-* ``axpy``, ``scal``, ... -- thin wrappers that pick the s/d symbol from the tensor dtype, pass
-  ``tensor.data_ptr()`` and raise :class:`B2Error` on a non-zero status.
+* ``lib().b2_saxpy`` etc. -- the raw C symbols through ctypes, with their prototypes set;
+* ``axpy``, ``scal``, ... -- callables of the compiled module ``_binding`` that pick the s/d symbol
+  from the tensor dtype, pass the tensors' addresses and torch's current stream, and raise
+  :class:`B2Error` on a non-zero status.
 
 PyTorch is used for device memory and streams only.  There is no CPU path: if the compiled
 CUDA library is missing the import of the symbols fails loudly.
@@ -15,6 +16,11 @@ import ctypes
 import os
 
 import torch
+
+try:
+    from . import _binding as _native  # (built with the library; its absence is reported at the first call)
+except ImportError:
+    _native = None
 
 ROW_MAJOR, COL_MAJOR = 101, 102
 NO_TRANS, TRANS = 111, 112
@@ -120,13 +126,14 @@ def exported_symbols():
                                        "b2_debug_bounds_report", "b2_debug_bounds_shrink"]
 
 
-class Context:
-    """Owns the workspace and status word (torch tensors) and builds the b2_ctx per call from
+class Context(_native.ContextBase if _native else object):
+    """Owns the workspace and status word (torch tensors); the calls build the b2_ctx from it and from
     torch's current stream."""
 
     def __init__(self, device="cuda", workspace_bytes: int | None = None, wait_limit: int = 0):
         h = lib()
         self.device = torch.device(device)
+        self._device_index = -1 if self.device.index is None else self.device.index  # -1: the current device
         nbytes = int(workspace_bytes if workspace_bytes is not None else h.b2_workspace_bytes())
         self.workspace = torch.zeros(nbytes + 256, dtype=torch.uint8, device=self.device)
         off = (-self.workspace.data_ptr()) % 256
@@ -159,135 +166,61 @@ def _p(t):
     return t.data_ptr()
 
 
-def _prefix(t) -> str:
-    if t.dtype == torch.float32:
-        return "s"
-    if t.dtype == torch.float64:
-        return "d"
-    raise TypeError(f"b2blas supports float32/float64, got {t.dtype}")
+def _missing(name):
+    def call(*args, **kwargs):
+        lib()
+        raise ImportError("the compiled module paper_2411_07211_b200._binding is missing: build it with "
+                          "`python -m paper_2411_07211_b200.build`")
+    call.__name__ = name
+    return call
 
 
-_recording = None  # list of (function, ctx struct, args) while prepare() runs a thunk
-
-
-def _call(name, ctx: Context, *args, check=True):
-    c = ctx.struct()
-    fn = getattr(lib(), name)
-    st = fn(ctypes.byref(c), *args)
-    if _recording is not None:
-        _recording.append((fn, c, args))
-    if check and st != 0:
-        raise B2Error(name, st)
-    return st
+_NAMES = ("axpy", "scal", "copy", "swap", "rot", "rotm", "dot", "dsdot", "sdsdot", "asum", "nrm2", "iamax",
+          "gemv", "ger", "syr", "syr2", "symv", "trmv", "trsv")
+_routines = _native.routines(LIB_PATH, B2Error, lib) if _native else {name: _missing(name) for name in _NAMES}
 
 
 def prepare(thunk):
     """Runs `thunk` (calls of this module) once and returns a callable that repeats exactly those
-    library calls with the arguments marshalled then -- same stream, same pointers -- without the
-    per-call Python work of the wrappers (about 10 us a call, more than a small kernel takes).
-    For timing loops over small problems; the returned callable returns the last status."""
-    global _recording
-    _recording = rec = []
-    try:
-        thunk()
-    finally:
-        _recording = None
-    calls = [(fn, ctypes.byref(c), args, c) for fn, c, args in rec]
-
-    def replay():
-        st = 0
-        for fn, ref, args, _keep in calls:
-            st = fn(ref, *args)
-        return st
-    return replay
+    library calls with the arguments marshalled then -- same stream, same pointers -- without
+    going through the interpreter for each of them.  For timing loops over small problems; the
+    returned callable returns the last status."""
+    return _native.record(thunk)
 
 
+# Every routine ends with `check=True`: raise B2Error on a non-zero status instead of returning it.
 # ---- level 1 ----------------------------------------------------------------------------
-def axpy(ctx, n, alpha, x, incx, y, incy, check=True):
-    return _call(f"b2_{_prefix(x)}axpy", ctx, n, alpha, _p(x), incx, _p(y), incy, check=check)
-
-
-def scal(ctx, n, alpha, x, incx, check=True):
-    return _call(f"b2_{_prefix(x)}scal", ctx, n, alpha, _p(x), incx, check=check)
-
-
-def copy(ctx, n, x, incx, y, incy, check=True):
-    return _call(f"b2_{_prefix(x)}copy", ctx, n, _p(x), incx, _p(y), incy, check=check)
-
-
-def swap(ctx, n, x, incx, y, incy, check=True):
-    return _call(f"b2_{_prefix(x)}swap", ctx, n, _p(x), incx, _p(y), incy, check=check)
-
-
-def rot(ctx, n, x, incx, y, incy, c, s, check=True):
-    return _call(f"b2_{_prefix(x)}rot", ctx, n, _p(x), incx, _p(y), incy, c, s, check=check)
+axpy = _routines["axpy"]      # (ctx, n, alpha, x, incx, y, incy, check=True)
+scal = _routines["scal"]      # (ctx, n, alpha, x, incx, check=True)
+copy = _routines["copy"]      # (ctx, n, x, incx, y, incy, check=True)
+swap = _routines["swap"]      # (ctx, n, x, incx, y, incy, check=True)
+rot = _routines["rot"]        # (ctx, n, x, incx, y, incy, c, s, check=True)
+dsdot = _routines["dsdot"]    # (ctx, n, x, incx, y, incy, result, check=True): float32 vectors, float64 device result
+sdsdot = _routines["sdsdot"]  # (ctx, n, sb, x, incx, y, incy, result, check=True)
+dot = _routines["dot"]        # (ctx, n, x, incx, y, incy, result, check=True)
+asum = _routines["asum"]      # (ctx, n, x, incx, result, check=True)
+nrm2 = _routines["nrm2"]      # (ctx, n, x, incx, result, check=True)
+iamax = _routines["iamax"]    # (ctx, n, x, incx, result, check=True)
 
 
 def rotm(ctx, n, x, incx, y, incy, param, check=True):
     """param: 5 host values [flag, h11, h21, h12, h22] (any sequence); None passes a NULL pointer."""
     if param is None:
-        hp = None
-    else:
-        ctype = ctypes.c_float if x.dtype == torch.float32 else ctypes.c_double
-        hp = ctypes.cast((ctype * 5)(*[float(v) for v in param]), _vp)
-    return _call(f"b2_{_prefix(x)}rotm", ctx, n, _p(x), incx, _p(y), incy, hp, check=check)
-
-
-def dsdot(ctx, n, x, incx, y, incy, result, check=True):
-    """float32 vectors, float64 device result."""
-    return _call("b2_dsdot", ctx, n, _p(x), incx, _p(y), incy, _p(result), check=check)
-
-
-def sdsdot(ctx, n, sb, x, incx, y, incy, result, check=True):
-    return _call("b2_sdsdot", ctx, n, sb, _p(x), incx, _p(y), incy, _p(result), check=check)
-
-
-def dot(ctx, n, x, incx, y, incy, result, check=True):
-    return _call(f"b2_{_prefix(x)}dot", ctx, n, _p(x), incx, _p(y), incy, _p(result), check=check)
-
-
-def asum(ctx, n, x, incx, result, check=True):
-    return _call(f"b2_{_prefix(x)}asum", ctx, n, _p(x), incx, _p(result), check=check)
-
-
-def nrm2(ctx, n, x, incx, result, check=True):
-    return _call(f"b2_{_prefix(x)}nrm2", ctx, n, _p(x), incx, _p(result), check=check)
-
-
-def iamax(ctx, n, x, incx, result, check=True):
-    return _call(f"b2_i{_prefix(x)}amax", ctx, n, _p(x), incx, _p(result), check=check)
+        return _routines["rotm"](ctx, n, x, incx, y, incy, None, check)
+    ctype = ctypes.c_float if x.dtype == torch.float32 else ctypes.c_double
+    host = (ctype * 5)(*[float(v) for v in param])
+    _native.keep(host)
+    return _routines["rotm"](ctx, n, x, incx, y, incy, ctypes.addressof(host), check)
 
 
 # ---- level 2 ----------------------------------------------------------------------------
-def gemv(ctx, order, trans, m, n, alpha, a, lda, x, incx, beta, y, incy, check=True):
-    return _call(f"b2_{_prefix(a)}gemv", ctx, order, trans, m, n, alpha, _p(a), lda, _p(x), incx, beta, _p(y),
-                 incy, check=check)
-
-
-def ger(ctx, order, m, n, alpha, x, incx, y, incy, a, lda, check=True):
-    return _call(f"b2_{_prefix(a)}ger", ctx, order, m, n, alpha, _p(x), incx, _p(y), incy, _p(a), lda, check=check)
-
-
-def syr(ctx, order, uplo, n, alpha, x, incx, a, lda, check=True):
-    return _call(f"b2_{_prefix(a)}syr", ctx, order, uplo, n, alpha, _p(x), incx, _p(a), lda, check=check)
-
-
-def syr2(ctx, order, uplo, n, alpha, x, incx, y, incy, a, lda, check=True):
-    return _call(f"b2_{_prefix(a)}syr2", ctx, order, uplo, n, alpha, _p(x), incx, _p(y), incy, _p(a), lda,
-                 check=check)
-
-
-def symv(ctx, order, uplo, n, alpha, a, lda, x, incx, beta, y, incy, check=True):
-    return _call(f"b2_{_prefix(a)}symv", ctx, order, uplo, n, alpha, _p(a), lda, _p(x), incx, beta, _p(y), incy,
-                 check=check)
-
-
-def trmv(ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True):
-    return _call(f"b2_{_prefix(a)}trmv", ctx, order, uplo, trans, diag, n, _p(a), lda, _p(x), incx, check=check)
-
-
-def trsv(ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True):
-    return _call(f"b2_{_prefix(a)}trsv", ctx, order, uplo, trans, diag, n, _p(a), lda, _p(x), incx, check=check)
+gemv = _routines["gemv"]      # (ctx, order, trans, m, n, alpha, a, lda, x, incx, beta, y, incy, check=True)
+ger = _routines["ger"]        # (ctx, order, m, n, alpha, x, incx, y, incy, a, lda, check=True)
+syr = _routines["syr"]        # (ctx, order, uplo, n, alpha, x, incx, a, lda, check=True)
+syr2 = _routines["syr2"]      # (ctx, order, uplo, n, alpha, x, incx, y, incy, a, lda, check=True)
+symv = _routines["symv"]      # (ctx, order, uplo, n, alpha, a, lda, x, incx, beta, y, incy, check=True)
+trmv = _routines["trmv"]      # (ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True)
+trsv = _routines["trsv"]      # (ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True)
 
 
 def set_tuning(knob: int, value: int):

@@ -1,11 +1,13 @@
 """In-tree build of libb2blas.so with nvcc for sm_100a (no torch extension machinery: the
-library has a plain C ABI and links only the CUDA runtime)."""
+library has a plain C ABI and links only the CUDA runtime) and, with the host compiler, of the
+Python module _binding.so that calls it."""
 from __future__ import annotations
 
 import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +17,8 @@ INCLUDE = os.path.join(ROOT, "include")
 OBJ_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(PKG, "libb2blas.so")
 DEBUG_LIB_PATH = os.path.join(PKG, "libb2blas_dbg.so")  # the bounds-checking build (-DB2_DEBUG_BOUNDS)
+
+BINDING_PATH = os.path.join(PKG, "_binding.so")  # Python entry points (torch and CPython headers, no CUDA code)
 
 SOURCES = ["api_common.cu", "level1.cu", "gemv.cu", "ger.cu", "tri_f32.cu", "tri_f64.cu", "trsv.cu", "trsv_front.cu", "syr.cu"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
@@ -39,15 +43,32 @@ def _digest() -> str:
     return h.hexdigest()
 
 
+def _compile_binding() -> None:
+    """The Python module: its symbols of torch resolve against the libraries `import torch` has loaded."""
+    from torch.utils.cpp_extension import include_paths, library_paths
+    incs = [a for d in [INCLUDE, sysconfig.get_paths()["include"], *include_paths(),
+                        os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")] for a in ("-I", d)]
+    tmp = BINDING_PATH + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", *incs,
+           os.path.join(CSRC, "binding_native.cpp"), "-o", tmp, *[a for d in library_paths() for a in ("-L", d)],
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-ldl"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"compiling the Python module failed:\n{res.stdout}\n{res.stderr}")
+    os.replace(tmp, BINDING_PATH)
+
+
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
-    """Compile every .cu under csrc/ and link libb2blas.so; a no-op when sources are unchanged.
-    debug_bounds=True builds the bounds-checking variant (libb2blas_dbg.so) instead."""
+    """Compile every .cu under csrc/, link libb2blas.so and build the Python module; a no-op when
+    sources are unchanged.  debug_bounds=True builds the bounds-checking variant (libb2blas_dbg.so)
+    of the library instead."""
     lib_path = DEBUG_LIB_PATH if debug_bounds else LIB_PATH
     obj_dir = os.path.join(OBJ_DIR, "dbg") if debug_bounds else OBJ_DIR
     extra = ["-DB2_DEBUG_BOUNDS"] if debug_bounds else []
     stamp = os.path.join(obj_dir, "stamp.txt")
     digest = _digest()
-    if not force and os.path.exists(lib_path) and os.path.exists(stamp) and open(stamp).read() == digest:
+    have = os.path.exists(lib_path) and (debug_bounds or os.path.exists(BINDING_PATH))
+    if not force and have and os.path.exists(stamp) and open(stamp).read() == digest:
         return lib_path
     os.makedirs(obj_dir, exist_ok=True)
     nvcc = _nvcc()
@@ -64,8 +85,11 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
             sys.stderr.write(res.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=min(8, len(SOURCES))) as pool:
+    with ThreadPoolExecutor(max_workers=min(8, len(SOURCES) + 1)) as pool:
+        binding = None if debug_bounds else pool.submit(_compile_binding)
         objs = list(pool.map(compile_one, SOURCES))
+        if binding is not None:
+            binding.result()
     tmp = lib_path + f".tmp{os.getpid()}"
     res = subprocess.run([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"],
                          capture_output=True, text=True)
