@@ -20,7 +20,7 @@ DEBUG_LIB_PATH = os.path.join(PKG, "libb2blas_dbg.so")  # the bounds-checking bu
 
 BINDING_PATH = os.path.join(PKG, "_binding.so")  # Python entry points (torch and CPython headers, no CUDA code)
 
-SOURCES = ["api_common.cu", "level1.cu", "gemv.cu", "ger.cu", "tri_f32.cu", "tri_f64.cu", "trsv.cu", "trsv_front.cu", "syr.cu"]
+SOURCES = ["api_common.cu", "level1.cu", "gemv.cu", "ger.cu", "tri_f32.cu", "tri_f64.cu", "trsv.cu", "trsv_front.cu", "trsv_cluster.cu", "syr.cu"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

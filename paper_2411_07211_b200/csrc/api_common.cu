@@ -13,13 +13,14 @@ static int64_t g_knobs[kKnobCount] = {
     /* kKnobTrsvDebugSkip   */ -1,
     /* kKnobTriWide         */ 0,
     /* kKnobTrsvPrefetchBytes */ 12 << 20,
-    /* kKnobTrsvFront       */ 2,
+    /* kKnobTrsvFront       */ 3,
     /* kKnobTrsvCluster     */ 0,
     /* kKnobTrsvPmFrom      */ -1,
     /* kKnobTriTile         */ 1,
     /* kKnobTriTileUnit     */ 0,
     /* kKnobNarrowBlock     */ 1,
     /* kKnobTriBulk         */ 0,
+    /* kKnobTrsvStreams     */ -1,
 };
 
 unsigned long long g_launch_count = 0;

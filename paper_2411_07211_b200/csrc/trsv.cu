@@ -587,6 +587,13 @@ static int trsv_impl(const b2_ctx* ctx, int order, int uplo, int trans, int diag
   const unsigned tag = next_tag();
   {
     bool handled = false;
+    // The cluster kernel is the fastest one at every size and alignment measured (n = 64 .. 16384); the other two
+    // serve what it declines: workspaces too small for its inverses, devices without clusters of its size,
+    // more unknowns than its streaming blocks can hold sums for (about 43,000).
+    if (knob(kKnobTrsvFront) >= 3) {
+      const int st = trsv_cluster_try<T>(l, coltype, !eff_lower, unit, n, a, lda, vec_base(x, n, incx), incx, tag, &handled);
+      if (handled) return st;
+    }
     const int st = trsv_front_try<T>(l, coltype, !eff_lower, unit, n, a, lda, vec_base(x, n, incx), incx, tag, &handled);
     if (handled) return st;
   }

@@ -12,4 +12,9 @@ template <typename T>
 int trsv_front_try(const Launch& l, bool coltype, bool backward, bool unit, int64_t n, const T* a, int64_t lda,
                    T* xbase, int64_t incx, unsigned tag, bool* handled);
 
+// The cluster kernel (trsv_cluster.cu), the same way; it takes every alignment.
+template <typename T>
+int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, int64_t n, const T* a, int64_t lda,
+                     T* xbase, int64_t incx, unsigned tag, bool* handled);
+
 }  // namespace b2

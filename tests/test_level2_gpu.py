@@ -257,6 +257,36 @@ def test_trsv_every_kernel_choice(b2, ctx, dtype, front, cluster, pm_from):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("streams", [-1, 1, 0])
+def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
+    """The cluster kernel at its edges: one unknown more and less than a block row, than the rows the solving
+    cluster multiplies itself, than one turn of the cluster; more strips than streaming blocks; with all
+    streaming clusters, with one, and with none (the solving cluster then does their work)."""
+    nb, near, cs = (128, 4, 16) if dtype == np.float32 else (64, 6, 16)
+    sizes = [1, nb, nb + 1, (near + 1) * nb, (near + 1) * nb + 1, cs * nb - 1, cs * nb + 3]
+    if streams != 0:
+        sizes += [(cs + near + 2) * nb + 5] if streams == 1 else [(2 * cs + 7) * nb + 5, 70 * nb]
+    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
+    try:
+        for n, pad in itertools.product(sizes, (0, 1)):
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                diag = orc.UNIT if n % 2 else orc.NON_UNIT
+                a = tri_buf(22, n, n + pad, dtype, orc.ROW_MAJOR, uplo, diag)
+                hx = place(synth.vector_np(9, n, n, dtype), -2 if pad else 1)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, diag, n, ga.t, n + pad, gx.t, -2 if pad else 1)
+                assert ctx.device_status() == 0
+                rx = gx.host()
+                gx.check_guards()
+                inc = -2 if pad else 1
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, diag, n, a, n + pad, hx, inc, rx, inc)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 def test_small_integer_level2_is_bit_exact(b2, ctx, dtype):
     rng = np.random.default_rng(2)
     m, n = 300, 1100
