@@ -21,6 +21,7 @@ static int64_t g_knobs[kKnobCount] = {
     /* kKnobNarrowBlock     */ 1,
     /* kKnobTriBulk         */ 0,
     /* kKnobTrsvStreams     */ -1,
+    /* kKnobGather          */ 1,
 };
 
 unsigned long long g_launch_count = 0;

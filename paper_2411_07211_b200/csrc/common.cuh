@@ -68,11 +68,13 @@ constexpr int kWarps = kThreads / 32;
 //   word 16     : ticket counter of trsv (next block-row to hand out)
 //   word 17     : trsv "blocks finished" counter
 //   word 19     : sub-block trsv: abort flag (stays up after a timeout until the workspace is reset)
+//   words 64 .. : counters and flags of in-place products (gather.cuh)
 // Scratch (partials, trsv flags) starts at kCtlBytes.
 constexpr size_t kCtlBytes = 4096;
 constexpr int kCtlReduceTicket = 0;
 constexpr int kCtlTrsvTicket = 16;
 constexpr int kCtlTrsvDone = 17;
+constexpr int kCtlGather = 64;
 constexpr int kCtlTrsvAbort = 19;  // sub-block trsv: raised when a bounded wait ran out
 
 // ---------------------------------------------------------------------------------------
@@ -348,7 +350,8 @@ enum Knob {
   kKnobNarrowBlock = 14,       // gemv on unpadded narrow matrices: 1 = block-wide kernels, 0 = warp-wide / general ones
   kKnobTriBulk = 15,           // tile kernel with the shared-memory ring: 1 = a tile arrives as one tiled TMA copy (measured equal to the 16-byte copies; off by default)
   kKnobTrsvStreams = 16,       // streaming clusters of the cluster trsv kernel at most (-1: as many as fit)
-  kKnobCount = 17
+  kKnobGather = 17,            // gemv / symv / trmv by one cluster per 32 outputs: 0 never, 1 where it is the faster kernel, 2 wherever it can, 3 the same with trmv's late outputs forced
+  kKnobCount = 18
 };
 int64_t knob(int id);
 

@@ -1,0 +1,378 @@
+// Small and middle-sized gemv, symv and trmv in one launch (Section 6.2.2): every output is gathered by one cluster.
+//
+// What bounds such a call is latency: launches, passes over partial sums, barriers.  A cluster of 1 .. 8 blocks
+// owns 32 outputs and reads everything they depend on -- 32 rows of the canonical row-major view (row part), 32
+// columns of it (column part), or, for symv, the 32 rows of the stored triangle up to the diagonal and the 32
+// columns beyond it.  symv so reads each element twice, the second time from L2 where matrices of this size stay;
+// in exchange no sum leaves the cluster: its blocks take the chunks of the contraction in turn and hand their 32
+// sums to rank 0 through distributed shared memory, which writes y.  One launch, no workspace, no second pass.
+//   row part:    a warp holds 4 rows, 64 packs of each in flight per chunk; rows are dealt to the warps modulo 8, so
+//                that all rows of a warp start the same number of elements past a 16-byte boundary (8 lda is a
+//                multiple of the pack length) and packs can be read aligned, the columns shifted by that number.
+//   column part: a lane per column, so an instruction reads one 128-byte (256-byte) run of a row whatever its
+//                alignment.  (Packs, several rows per instruction: a third slower at n = 3000 in double.)
+//
+// trmv overwrites x while other clusters still need it: every block first copies the part of x that it reads into
+// shared memory and counts itself in the control block.  A cluster that finds all blocks counted writes its outputs;
+// one that does not (a block has not even started) leaves them in the workspace under a flag, and the last block to
+// be counted writes them at its end.  Nobody waits.
+#pragma once
+
+#include <algorithm>
+
+#include "level2.cuh"
+
+namespace b2 {
+namespace ga {
+
+constexpr int R = 32;             // outputs per cluster
+constexpr int RPW = R / kWarps;   // rows of a warp in the row part
+constexpr int kMaxGroups = 896;   // flags in the control block
+constexpr int kMaxCluster = 8;
+constexpr int CL = 16;            // loads of a thread in flight in the column part
+constexpr int CB = CL * kWarps;   // rows of a batch there
+constexpr int64_t kMaxBytesPerBlock = 128 * 1024;  // matrix bytes a block may be given: four chunks of latency
+
+template <typename T>
+struct Args {
+  const T* a;
+  int64_t lda;
+  const T* x;  // base per vec_base()
+  int64_t incx;
+  T* y;
+  int64_t incy;
+  T alpha, beta;
+  T* late;        // [groups * R] outputs that could not be written yet (in-place kinds)
+  unsigned* ctl;  // counters, flags (in-place kinds)
+  int defer;      // tests: take the late way first
+  int rows, cols;
+};
+
+template <typename T>
+__device__ __forceinline__ T ld_x(const T* p) { return B2_GUARD(p, sizeof(T)) ? *p : T(0); }
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_rank0(float* local, float v) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_rank0(double* local, double v) {
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+// ROWOUT / COLOUT of the kind: row part / column part.  Triangular kinds that are not symmetric work in place.
+template <typename T, bool AL, class K>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kernel(const Args<T> p) {
+  constexpr int V = VecLen<T>::value, SH = AL ? 0 : V - 1;
+  constexpr int CH = 2 * 32 * V;                              // columns of a row-part chunk
+  constexpr bool INPLACE = K::TRI != TRI_FULL && !K::SYM;
+  using P = Pack<T, V>;
+  __shared__ T s_row[R], s_col[kWarps][R], s_sum[kMaxCluster][R];
+  __shared__ int s_last;
+  __shared__ unsigned s_mine[INPLACE ? kThreads : 1];
+  extern __shared__ __align__(16) unsigned char gather_smem[];
+  const int tid = (int)threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_rank(), nr = (int)cluster_size();
+  const int g = (int)blockIdx.x / nr, o0 = g * R;
+  const unsigned long long a_el = (unsigned long long)p.a / sizeof(T);
+  // columns of the row part, rows of the column part
+  const int rlo = K::TRI == TRI_UPPER ? o0 : 0, rhi = K::TRI == TRI_LOWER ? min(p.cols, o0 + R) : p.cols;
+  const int clo = K::TRI == TRI_LOWER ? o0 : 0, chi = K::TRI == TRI_UPPER ? min(p.rows, o0 + R) : p.rows;
+  const int k0 = rlo / CH, nrow = K::ROWOUT ? (rhi + SH - 1) / CH + 1 - k0 : 0;
+  const int nbat = K::COLOUT ? (chi - clo + CB - 1) / CB : 0;
+  if (nr > 1) cluster_arrive();  // (completed below: every block of the cluster is running)
+  grid_dep_wait();
+  grid_dep_launch();
+
+  const T* xp = p.x;
+  int64_t xi = p.incx;
+  bool last_reader = false;
+  if (INPLACE) {
+    T* xs = reinterpret_cast<T*>(gather_smem);
+    const int lo = K::ROWOUT ? rlo : clo, hi = K::ROWOUT ? rhi : chi;
+    for (int t0 = lo + tid; t0 < hi; t0 += 8 * kThreads) {  // eight loads in flight
+      T v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = t0 + u * kThreads < hi ? ld_x(p.x + (int64_t)(t0 + u * kThreads) * p.incx) : T(0);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (t0 + u * kThreads < hi) xs[t0 + u * kThreads - lo] = v[u];
+    }
+    xp = xs - lo;
+    xi = 1;
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      s_last = atomicAdd(p.ctl, 1u) == gridDim.x - 1;
+    }
+  }
+  // (x of an in-place kind lies in shared memory, where the checking build's extents do not reach)
+  auto x_at = [&](int j) { return INPLACE ? xp[j] : ld_x(xp + (int64_t)j * xi); };
+
+  T rsum[RPW], csum = T(0);
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) rsum[u] = T(0);
+
+  if (K::ROWOUT) {
+    const int s = AL ? 0 : (int)((a_el + (unsigned long long)warp * (unsigned long long)p.lda) % V);
+    const T* const a0 = p.a + (int64_t)(o0 + warp) * p.lda + (lane * V - s);
+    const int64_t rstride = (int64_t)kWarps * p.lda;
+    const bool all_rows = o0 + R <= p.rows;
+#pragma unroll 1
+    for (int t = rank; t < nrow; t += nr) {
+      const int c0 = (k0 + t) * CH;
+      const bool fast = all_rows && c0 >= SH && c0 + CH <= p.cols &&
+                        (K::TRI == TRI_FULL || (K::TRI == TRI_LOWER ? c0 + CH - 1 < o0 : c0 - SH > o0 + R - 1));
+      P av[RPW][2];
+      T xv[2][V];
+      if (fast) {
+#pragma unroll
+        for (int u = 0; u < RPW; ++u)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) av[u][h] = ld_nc<T, V>(a0 + u * rstride + c0 + h * 32 * V);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int e = 0; e < V; ++e) xv[h][e] = x_at(c0 + h * 32 * V + lane * V - s + e);
+#pragma unroll
+        for (int u = 0; u < RPW; ++u)
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int e = 0; e < V; ++e) rsum[u] = av[u][h].v[e] * xv[h][e] + rsum[u];
+      } else {
+        // packs that exist go out together, each under its predicate; those the matrix edge cuts element by element
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int c = c0 + h * 32 * V + lane * V - s;
+          const bool whole = c >= 0 && c + V <= p.cols;
+#pragma unroll
+          for (int u = 0; u < RPW; ++u) {
+            const int i = o0 + u * kWarps + warp;
+            const bool in = i < p.rows && (K::TRI == TRI_FULL || (K::TRI == TRI_LOWER ? c <= i : c + V - 1 >= i));
+            av[u][h] = ld_nc_if<T, V>(a0 + u * rstride + c0 + h * 32 * V, whole && in);
+          }
+#pragma unroll
+          for (int e = 0; e < V; ++e) xv[h][e] = c + e >= rlo && c + e < rhi ? x_at(c + e) : T(0);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int c = c0 + h * 32 * V + lane * V - s;
+          if (!(c >= 0 && c + V <= p.cols) && c + V > 0 && c < p.cols) {
+#pragma unroll
+            for (int u = 0; u < RPW; ++u)
+#pragma unroll
+              for (int e = 0; e < V; ++e)
+                if (o0 + u * kWarps + warp < p.rows && c + e >= 0 && c + e < p.cols)
+                  av[u][h].v[e] = __ldg(a0 + u * rstride + c0 + h * 32 * V + e);
+          }
+#pragma unroll
+          for (int u = 0; u < RPW; ++u) {
+            const int i = o0 + u * kWarps + warp;
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+              const int j = c + e;
+              bool in = i < p.rows && j >= 0 && j < p.cols;
+              if (K::TRI == TRI_LOWER) in = in && j <= i;
+              if (K::TRI == TRI_UPPER) in = in && j >= i;
+              const T v = (K::UNIT && j == i) ? T(1) : av[u][h].v[e];
+              rsum[u] = in ? v * xv[h][e] + rsum[u] : rsum[u];  // (a select: what is not referenced may be anything)
+            }
+          }
+        }
+      }
+    }
+    const T v = multi_group_sum<32, RPW>(rsum, lane);
+    constexpr int LPV = 32 / RPW;
+    if (lane % LPV == 0) s_row[lane / LPV * kWarps + warp] = v;
+  }
+  if (K::COLOUT) {
+    const int j = o0 + lane;
+    const bool all_cols = o0 + R <= p.cols;
+    const int64_t rstride = (int64_t)kWarps * p.lda;
+    int t = rank - nrow % nr;  // (the row part's chunks come first in the blocks' turns)
+    if (t < 0) t += nr;
+#pragma unroll 1
+    for (; t < nbat; t += nr) {
+      const int r0 = clo + t * CB;
+      const bool fast = all_cols && r0 + CB <= chi && (K::TRI == TRI_FULL || (K::TRI == TRI_LOWER ? r0 > o0 + R - 1 : r0 + CB - 1 < o0));
+      T av[CL], xv[CL];
+      const T* at = p.a + (int64_t)(r0 + warp) * p.lda + j;
+      if (fast) {
+#pragma unroll
+        for (int u = 0; u < CL; ++u) av[u] = __ldg(at + u * rstride);
+#pragma unroll
+        for (int u = 0; u < CL; ++u) xv[u] = x_at(r0 + warp + u * kWarps);
+#pragma unroll
+        for (int u = 0; u < CL; ++u) csum = av[u] * xv[u] + csum;
+      } else {
+#pragma unroll
+        for (int u = 0; u < CL; ++u) {
+          const int i = r0 + warp + u * kWarps;
+          bool in = i < chi && j < p.cols;
+          if (K::TRI == TRI_LOWER) in = in && (K::SYM ? j < i : j <= i);
+          if (K::TRI == TRI_UPPER) in = in && (K::SYM ? j > i : j >= i);
+          av[u] = T(0), xv[u] = T(0);
+          if (in) av[u] = (K::UNIT && j == i) ? T(1) : __ldg(at + u * rstride);
+          if (in) xv[u] = x_at(i);  // (not what a zero would meet: x may hold infinities where the triangle ends)
+        }
+#pragma unroll
+        for (int u = 0; u < CL; ++u) csum = av[u] * xv[u] + csum;
+      }
+    }
+    s_col[warp][lane] = csum;
+  }
+  __syncthreads();
+  if (INPLACE) last_reader = s_last != 0;
+  if (nr > 1) cluster_wait();
+  if (warp == 0) {
+    T v = K::ROWOUT ? s_row[lane] : T(0);
+    if (K::COLOUT) {
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) v += s_col[w][lane];
+    }
+    if (rank == 0) s_sum[0][lane] = v;
+    else st_rank0(&s_sum[rank][lane], v);
+  }
+  if (nr > 1) {
+    cluster_arrive();
+    cluster_wait();
+  }
+  const int nout = K::ROWOUT ? p.rows : p.cols;
+  auto write = [&](int i, T v) {
+    T* yp = p.y + (int64_t)i * p.incy;
+    B2_STORE(yp, p.beta != T(0) ? p.alpha * v + p.beta * *yp : p.alpha * v);
+  };
+  if (rank == 0 && warp == 0) {
+    T v = s_sum[0][lane];
+    for (int c = 1; c < nr; ++c) v += s_sum[c][lane];
+    if (!INPLACE) {
+      if (o0 + lane < nout) write(o0 + lane, v);
+    } else {
+      volatile unsigned* const readers = p.ctl;
+      unsigned* const flag = p.ctl + 2 + g;
+      bool now = false;
+      if (lane == 0) now = !p.defer && *readers == gridDim.x;
+      now = __shfl_sync(0xffffffffu, (int)now, 0) != 0;
+      if (!now) {  // some block has not read its x yet
+        p.late[o0 + lane] = v;
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) {
+          atomicExch(flag, 1u);
+          __threadfence();
+          if (*readers == gridDim.x) now = atomicCAS(flag, 1u, 0u) == 1u;  // all have by now: nobody may come for it
+        }
+        now = __shfl_sync(0xffffffffu, (int)now, 0) != 0;
+      }
+      if (now) {
+        __threadfence();
+        if (o0 + lane < nout) write(o0 + lane, v);
+      }
+    }
+  }
+  if (INPLACE) {
+    if (last_reader) {  // outputs left behind before this block had read its x
+      const int ngroups = (int)gridDim.x / nr;
+      __threadfence();
+      for (int q0 = 0; q0 < ngroups; q0 += kThreads) {
+        if (q0 + tid < ngroups) s_mine[tid] = atomicCAS(p.ctl + 2 + q0 + tid, 1u, 0u);
+        __syncthreads();
+        __threadfence();
+        const int n = min(kThreads, ngroups - q0) * R;
+#pragma unroll 4
+        for (int t = tid; t < n; t += kThreads) {
+          const int i = q0 * R + t;
+          if (s_mine[t / R] == 1u && i < nout) write(i, __ldcg(p.late + i));
+        }
+        __syncthreads();
+      }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      __threadfence();
+      if (atomicAdd(p.ctl + 1, 1u) == gridDim.x - 1) p.ctl[0] = p.ctl[1] = 0u;  // the last block leaves the counters clean
+    }
+  }
+}
+
+// Launches the kernel; *handled is false (nothing launched) where the sizes do not allow it.
+template <typename T, bool AL, class K>
+static int launch(const Launch& l, const L2Args<T>& q, bool* handled) {
+  constexpr int V = VecLen<T>::value, CH = 2 * 32 * V;
+  constexpr bool INPLACE = K::TRI != TRI_FULL && !K::SYM;
+  const int64_t nout = K::ROWOUT ? q.rows : q.cols, len = K::ROWOUT ? q.cols : q.rows;
+  const int64_t groups = (nout + R - 1) / R;
+  if (groups > kMaxGroups || len > (1 << 24)) return B2_STATUS_OK;
+  const size_t smem = INPLACE ? (size_t)len * sizeof(T) : 0;
+  if (smem > 40 * 1024 || (INPLACE && (size_t)groups * R * sizeof(T) > l.scratch_bytes)) return B2_STATUS_OK;
+  // blocks per cluster: no more than there are chunks, and one resident wave in all
+  const int64_t items = (K::ROWOUT ? (len + CH - 1) / CH : 0) + (K::COLOUT ? (len + CB - 1) / CB : 0);
+  const int64_t wave = (int64_t)sm_count() * (sizeof(T) == 8 ? 3 : 4);
+  int nr = 1;
+  while (nr < kMaxCluster && 2 * nr <= items && groups * nr * (INPLACE ? 2 : 1) <= wave) nr *= 2;
+  const int64_t bytes = q.rows * q.cols * (int64_t)sizeof(T) / (INPLACE ? 2 : 1);
+  if (knob(kKnobGather) < 2 && bytes > kMaxBytesPerBlock * groups * nr) return B2_STATUS_OK;
+  Args<T> p = {};
+  p.a = q.a;
+  p.lda = q.lda;
+  p.x = K::ROWOUT ? q.xc : q.xr;
+  p.incx = K::ROWOUT ? q.incxc : q.incxr;
+  p.y = q.y;
+  p.incy = q.incy;
+  p.alpha = q.alpha;
+  p.beta = q.beta;
+  p.late = reinterpret_cast<T*>(l.scratch);
+  p.ctl = l.ctl + kCtlGather;
+  p.defer = knob(kKnobGather) == 3;
+  p.rows = (int)q.rows;
+  p.cols = (int)q.cols;
+  *handled = true;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)nr;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)(groups * nr));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = l.stream;
+  cfg.attrs = at;
+  cfg.numAttrs = knob(kKnobUsePdl) ? 2 : 1;
+  (void)cudaLaunchKernelEx(&cfg, gather_kernel<T, AL, K>, p);
+  return check_launch();
+}
+// Where one launch by clusters is the faster way (total matrix bytes; measured with three matrices in turn, against
+// the tile kernels and their finalize pass): gemv up to 20 MB (n = 1500 double 16.1 -> 10.0 us for two calls, 2000
+// float 13.1 -> 11.1), off 16-byte boundaries up to 34 MB (2001 double 22.1 -> 19.9); trmv up to 36 MB (2000 double
+// 20 -> 17.7 us with its copy, 3000 float 20.2 -> 19.3), unaligned up to 72 MB (3001 double 40 -> 26.6); symv, which
+// reads its elements twice, up to 6 MB (1000 float 11.8 -> 8.4), unaligned up to 72 MB (1001 float 21.7 -> 9,
+// 3001 float 40 -> 29).
+template <typename T, class K>
+static int run(const Launch& l, const L2Args<T>& q, bool* handled) {
+  *handled = false;
+  if (knob(kKnobGather) == 0) return B2_STATUS_OK;
+  const bool al = aligned_to(q.a, 16) && q.lda % VecLen<T>::value == 0;
+  const int64_t mb = K::TRI == TRI_FULL ? (al ? 20 : 34) : K::SYM ? (al ? 6 : 72) : (al ? 36 : 73);
+  if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)mb * 1e6) return B2_STATUS_OK;
+  return al ? launch<T, true, K>(l, q, handled) : launch<T, false, K>(l, q, handled);
+}
+
+}  // namespace ga
+}  // namespace b2

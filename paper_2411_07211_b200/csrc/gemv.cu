@@ -3,6 +3,7 @@
 // the transposed row-major problem (A^T stored row-major), so N and T swap kinds.
 #include "level2.cuh"
 #include "skinny.cuh"
+#include "gather.cuh"
 
 namespace b2 {
 
@@ -46,6 +47,11 @@ static int gemv_impl(const b2_ctx* ctx, int order, int trans, int64_t m, int64_t
   if (rowdot) {
     args.xc = vec_base(x, lenx, incx);
     args.incxc = incx;
+    {
+      bool handled = false;
+      const int st = ga::run<T, GemvRow>(l, args, &handled);
+      if (handled) return st;
+    }
     if (knob(kKnobNarrowBlock) && block_narrow_applies(a, lda, args.rows, args.cols))
       return block_rowdot<T>(l, a, args.rows, args.cols, args.xc, incx, alpha, beta, args.y, incy);
     if (skinny_applies(a, lda, args.rows, args.cols, true))
@@ -54,6 +60,11 @@ static int gemv_impl(const b2_ctx* ctx, int order, int trans, int64_t m, int64_t
   }
   args.xr = vec_base(x, lenx, incx);
   args.incxr = incx;
+  {
+    bool handled = false;
+    const int st = ga::run<T, GemvCol>(l, args, &handled);
+    if (handled) return st;
+  }
   if (knob(kKnobNarrowBlock) && wide_applies<T>(args.rows, args.cols)) {
     const int64_t want = (args.cols + kThreads - 1) / kThreads, cap = (int64_t)sm_count() * 8;
     launch_chained(wide_colsum_kernel<T>, dim3((unsigned)(want < cap ? want : cap)), dim3(kThreads), 0, l.stream, a, lda, (int)args.rows, args.cols, args.xr,

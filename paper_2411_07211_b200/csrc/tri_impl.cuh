@@ -7,6 +7,7 @@
 //          written over x by the finalize kernel, after every block has finished reading x.
 #pragma once
 #include "level2.cuh"
+#include "gather.cuh"
 #include "tri_tile.cuh"
 
 namespace b2 {
@@ -61,6 +62,12 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
   args.incy = incy;
   // the stored triangle as it sits in the row-major view of the buffer
   const bool upper = (order == B2_ROW_MAJOR) == (uplo == B2_UPPER);
+  if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {  // (a forced tile kernel stays forced)
+    bool handled = false;
+    const int st = upper ? ga::run<T, Kind<true, true, TRI_UPPER, false, true>>(l, args, &handled)
+                         : ga::run<T, Kind<true, true, TRI_LOWER, false, true>>(l, args, &handled);
+    if (handled) return st;
+  }
   // The tile kernel with the shared-memory ring (16-byte aligned matrices) is the faster one while
   // the triangle is small (n = 4096: 13 us against 19 us in float); from about 64 MiB of triangle
   // on the general tile kernel streams faster (n = 32768 float: 320 us against 357 us).  Knob value
@@ -84,6 +91,11 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
 
 template <typename T, bool ROW, int TRI>
 static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
+  if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {
+    bool handled = false;
+    const int st = unit ? ga::run<T, Kind<ROW, !ROW, TRI, true, false>>(l, args, &handled) : ga::run<T, Kind<ROW, !ROW, TRI, false, false>>(l, args, &handled);
+    if (handled) return st;
+  }
   // The tile kernel with the shared-memory ring serves trmv where it measured faster than the
   // general tile kernel: float row sums with a strided x (knob value 2: always, for the tests).
   const bool ring = knob(kKnobTriTile) == 2 || (knob(kKnobTriTile) == 1 && sizeof(T) == 4 && ROW && args.incxc != 1);

@@ -257,6 +257,52 @@ def test_trsv_every_kernel_choice(b2, ctx, dtype, front, cluster, pm_from):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("mode", [0, 2, 3])
+def test_cluster_gather_kernel(b2, ctx, dtype, mode):
+    """The one-launch kernel at its edges: one output more and less than a cluster owns, one element more and less
+    than a chunk of the row part (256 / 128 columns) and a batch of the column part (128 rows), every residue of the
+    rows' starts; mode 3 sends every output of trmv through the workspace first, mode 0 keeps these sizes on the tile
+    kernels."""
+    old = b2.get_tuning(b2.KNOB_GATHER)
+    b2.set_tuning(b2.KNOB_GATHER, mode)
+    try:
+        for n, pad, off in ((1, 0, 0), (31, 0, 0), (32, 1, 0), (33, 0, 1), (127, 2, 0), (129, 0, 0), (255, 0, 0), (257, 3, 1), (512, 0, 0), (1030, 1, 0)):
+            lda, inc = n + pad, -2 if pad else 1
+            x, y = synth.vector_np(7, n, n, dtype), synth.vector_np(8, n, n, dtype)
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                diag = orc.UNIT if n % 2 else orc.NON_UNIT
+                a = tri_buf(12, n, lda, dtype, orc.ROW_MAJOR, uplo, diag)
+                ga, gx = Guarded(a, off), Guarded(place(x, inc))
+                b2.trmv(ctx, orc.ROW_MAJOR, uplo, trans, diag, n, ga.t, lda, gx.t, inc)
+                ox = place(x, inc)
+                absterms = orc.trmv(orc.ROW_MAJOR, uplo, trans, diag, n, a, lda, ox, inc)
+                assert_close(pick(gx.host(), n, inc), pick(ox, n, inc), absterms, dtype, f"trmv {n} {pad} {uplo} {trans}")
+                gx.check_guards()
+            if mode == 3:
+                continue
+            for uplo in UPLOS:
+                a = tri_buf(9, n, lda, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+                ga, gx, gy = Guarded(a, off), Guarded(place(x, inc)), Guarded(place(y, 1))
+                b2.symv(ctx, orc.ROW_MAJOR, uplo, n, 1.25, ga.t, lda, gx.t, inc, 0.5, gy.t, 1)
+                oy = y.copy()
+                absterms = orc.symv(orc.ROW_MAJOR, uplo, n, dtype(1.25), a, lda, place(x, inc), inc, dtype(0.5), oy, 1)
+                assert_close(gy.host(), oy, absterms, dtype, f"symv {n} {pad} {uplo}")
+                gy.check_guards()
+            for m, trans in itertools.product((n + 1, 200), TRANSES):
+                a = synth.matrix_np(3, m, m, n, lda, dtype).ravel()
+                lx, ly = (n, m) if trans == orc.NO_TRANS else (m, n)
+                vx, vy = synth.vector_np(5, lx, lx, dtype), np.full(ly, np.nan, dtype=dtype)
+                ga, gx, gy = Guarded(a, off), Guarded(place(vx, inc)), Guarded(vy)
+                b2.gemv(ctx, orc.ROW_MAJOR, trans, m, n, 1.25, ga.t, lda, gx.t, inc, 0.0, gy.t, 1)
+                oy = vy.copy()
+                absterms = orc.gemv(orc.ROW_MAJOR, trans, m, n, dtype(1.25), a, lda, place(vx, inc), inc, dtype(0.0), oy, 1)
+                assert_close(gy.host(), oy, absterms, dtype, f"gemv {m} {n} {pad} {trans}")
+                gy.check_guards()
+    finally:
+        b2.set_tuning(b2.KNOB_GATHER, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("streams", [-1, 1, 0])
 def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
     """The cluster kernel at its edges: one unknown more and less than a block row, than the rows the solving
