@@ -162,6 +162,26 @@ __device__ __forceinline__ Pack<T, N> ld_nc_if(const T* p, bool pred) {
   return r;
 }
 
+// One element under a predicate, zero otherwise, without a branch: for the few packs at a matrix edge that are read
+// element by element, all loads in flight together.  (The element-wise tiles stay with ld_nc_if: measured 10 % faster.)
+template <typename T>
+__device__ __forceinline__ T ld_el_if(const T* p, bool pred) {
+  if (pred && !B2_GUARD(p, sizeof(T))) pred = false;
+  if constexpr (sizeof(T) == 4) {
+    unsigned t;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.global.nc.u32 %0, [%1];\n\t}"
+                 : "=&r"(t)
+                 : "l"(p), "r"((unsigned)pred));
+    return *reinterpret_cast<T*>(&t);
+  } else {
+    unsigned long long t;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u64 %0, 0;\n\t@q ld.global.nc.u64 %0, [%1];\n\t}"
+                 : "=&l"(t)
+                 : "l"(p), "r"((unsigned)pred));
+    return *reinterpret_cast<T*>(&t);
+  }
+}
+
 // Read-only load of reused data (the x vectors): cached in L1.
 template <typename T, int N>
 __device__ __forceinline__ Pack<T, N> ld_ro(const T* p) {

@@ -167,7 +167,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
             av[u][h] = ld_nc_if<T, V>(a0 + u * rstride + c0 + h * 32 * V, whole && in);
           }
 #pragma unroll
-          for (int e = 0; e < V; ++e) xv[h][e] = c + e >= rlo && c + e < rhi ? x_at(c + e) : T(0);
+          for (int e = 0; e < V; ++e) {
+            const bool in = c + e >= rlo && c + e < rhi;
+            if constexpr (INPLACE) xv[h][e] = in ? x_at(c + e) : T(0);
+            else xv[h][e] = ld_el_if<T>(xp + (int64_t)(c + e) * xi, in);
+          }
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -177,8 +181,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
             for (int u = 0; u < RPW; ++u)
 #pragma unroll
               for (int e = 0; e < V; ++e)
-                if (o0 + u * kWarps + warp < p.rows && c + e >= 0 && c + e < p.cols)
-                  av[u][h].v[e] = __ldg(a0 + u * rstride + c0 + h * 32 * V + e);
+                av[u][h].v[e] = ld_el_if<T>(a0 + u * rstride + c0 + h * 32 * V + e, o0 + u * kWarps + warp < p.rows && c + e >= 0 && c + e < p.cols);
           }
 #pragma unroll
           for (int u = 0; u < RPW; ++u) {
@@ -226,9 +229,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
           bool in = i < chi && j < p.cols;
           if (K::TRI == TRI_LOWER) in = in && (K::SYM ? j < i : j <= i);
           if (K::TRI == TRI_UPPER) in = in && (K::SYM ? j > i : j >= i);
-          av[u] = T(0), xv[u] = T(0);
-          if (in) av[u] = (K::UNIT && j == i) ? T(1) : __ldg(at + u * rstride);
-          if (in) xv[u] = x_at(i);  // (not what a zero would meet: x may hold infinities where the triangle ends)
+          av[u] = ld_el_if<T>(at + u * rstride, in && !(K::UNIT && j == i));
+          if (K::UNIT && in && j == i) av[u] = T(1);
+          // (zero where the element is masked: x may hold infinities where the triangle ends)
+          if constexpr (INPLACE) xv[u] = in ? x_at(i) : T(0);
+          else xv[u] = ld_el_if<T>(xp + (int64_t)i * xi, in);
         }
 #pragma unroll
         for (int u = 0; u < CL; ++u) csum = av[u] * xv[u] + csum;
@@ -369,7 +374,7 @@ static int run(const Launch& l, const L2Args<T>& q, bool* handled) {
   *handled = false;
   if (knob(kKnobGather) == 0) return B2_STATUS_OK;
   const bool al = aligned_to(q.a, 16) && q.lda % VecLen<T>::value == 0;
-  const int64_t mb = K::TRI == TRI_FULL ? (al ? 20 : 34) : K::SYM ? (al ? 6 : 72) : (al ? 36 : 73);
+  const int64_t mb = K::TRI == TRI_FULL ? (al ? 20 : 34) : K::SYM ? (al ? 6 : 73) : (al ? 36 : 73);
   if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)mb * 1e6) return B2_STATUS_OK;
   return al ? launch<T, true, K>(l, q, handled) : launch<T, false, K>(l, q, handled);
 }

@@ -56,6 +56,7 @@ struct L2Args {
   int64_t incxr;
   T* rowpart;  // [ncs][rows]
   T* colpart;  // [nrs][cols]
+  T* colspill; // [nrs][nct][V - 1]: column sums left of a block's own columns (SHIFT)
   int64_t rows_per_cta;
   int ctiles_per_cta, nct, nrs, ncs;
   int direct;  // 1: blocks write alpha*acc + beta*y straight to y
@@ -81,10 +82,17 @@ __device__ __forceinline__ bool region_strictly_inside(int64_t r0, int64_t r1, i
   return true;
 }
 
-template <typename T, int V, class K, class S>
+// SHIFT: rows that start off 16-byte boundaries, read in aligned packs all the same.  A warp's rows are congruent
+// modulo 8 and 8 * lda is a multiple of V, so they all start the same number s of elements past a boundary; the warp
+// takes its packs from s elements before the row on, and its column q of a tile is column q - s of the matrix.  Row
+// sums do not mind; column sums of a tile cover its TC columns and the V - 1 before them, which go to colspill.  Only
+// packs that the matrix edge cuts are read element by element.  (Element loads everywhere, four times the load
+// instructions: float n = 8191 symv 60 us, trmv 34, gemv 54; aligned 28, 24, 43.)
+template <typename T, int V, class K, class S, bool SHIFT>
 __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args<T> p) {
   constexpr int LPR = S::LPR, CU = S::CU, RU = S::RU, G = S::G, RB = S::RB;
-  constexpr int TC = LPR * V * CU;
+  constexpr int TC = LPR * V * CU, SH = SHIFT ? V - 1 : 0;
+  static_assert(!SHIFT || (G == 1 && S::NCT == 1), "a warp's rows are congruent modulo kWarps");
   constexpr int NCT = K::COLOUT ? S::NCT : 1;
   using P = Pack<T, V>;
   grid_dep_wait();
@@ -105,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
   const int ct_begin = cs * p.ctiles_per_cta;
   const int ct_end = min(p.nct, ct_begin + p.ctiles_per_cta);
   const int64_t c_lo = (int64_t)ct_begin * TC, c_hi = min(p.cols, (int64_t)ct_end * TC);
-  if (!region_active<K::TRI>(r_begin, r_end, c_lo, c_hi)) return;
+  if (!region_active<K::TRI>(r_begin, r_end, c_lo - SH, c_hi)) return;
 
   T colacc[NCT][CU][V];
   T xcv[NCT][CU][V];
@@ -124,11 +132,12 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
   const int lrow0 = warp * G + g;                            // first local row of this thread
   const int64_t rstride = (int64_t)kWarps * G * p.lda;       // elements between a thread's rows
   const int64_t xstride = (int64_t)kWarps * G * p.incxr;
-  const T* a_cta = p.a + (r_begin + lrow0) * p.lda + q * V;  // row r_begin + lrow0, column q*V
+  const int s = SHIFT ? (int)(((unsigned long long)p.a / sizeof(T) + (unsigned long long)lrow0 * (unsigned long long)p.lda) % V) : 0;
+  const T* a_cta = p.a + (r_begin + lrow0) * p.lda + (q * V - s);  // row r_begin + lrow0, column q*V (- s)
 
   for (int64_t rb = r_begin; rb < r_end; rb += RB) {
     const int64_t rb_end = min(rb + RB, r_end);
-    if (!region_active<K::TRI>(rb, rb_end, c_lo, c_hi)) continue;
+    if (!region_active<K::TRI>(rb, rb_end, c_lo - SH, c_hi)) continue;
     const int nr = (int)(rb_end - rb);  // rows of this batch
     const T* a_rb = a_cta + (rb - r_begin) * p.lda;
     T rowacc[RU], xrv[RU];
@@ -151,10 +160,24 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
     const int ct_hi = K::COLOUT ? min(ct_lo + 1, ct_end) : ct_end;
     for (int ct = ct_lo; ct < ct_hi; ++ct) {
       const int64_t c0 = (int64_t)ct * TC, c1 = min(p.cols, c0 + TC);
-      if (!region_active<K::TRI>(rb, rb_end, c0, c1)) continue;
+      if (!region_active<K::TRI>(rb, rb_end, c0 - SH, c1)) continue;
       if (K::ROWOUT && xcv_ct[c] != ct) {
         xcv_ct[c] = ct;
-        if (V > 1 && p.xc_vec == 1 && c0 + TC <= p.cols) {
+        if (SHIFT && c0 > 0 && c0 + TC <= p.cols) {
+          const T* xp = p.xc + (c0 + q * V - s) * p.incxc;
+#pragma unroll
+          for (int u = 0; u < CU; ++u)
+#pragma unroll
+            for (int e = 0; e < V; ++e) xcv[c][u][e] = __ldg(xp + (u * LPR * V + e) * p.incxc);
+        } else if (SHIFT) {
+#pragma unroll
+          for (int u = 0; u < CU; ++u)
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+              const int64_t j = c0 + (u * LPR + q) * V + e - s;
+              xcv[c][u][e] = j >= 0 && j < p.cols ? __ldg(p.xc + j * p.incxc) : T(0);
+            }
+        } else if (V > 1 && p.xc_vec == 1 && c0 + TC <= p.cols) {
 #pragma unroll
           for (int u = 0; u < CU; ++u) {
             const P xv = ld_ro<T, V>(p.xc + c0 + (u * LPR + q) * V);
@@ -181,8 +204,8 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
             }
         }
       }
-      const bool fast = (rb + RB <= r_end) && (c0 + TC <= p.cols) &&
-                        region_strictly_inside<K::TRI>(rb, rb + RB, c0, c0 + TC);
+      const bool fast = (rb + RB <= r_end) && (c0 + TC <= p.cols) && (!SHIFT || c0 > 0) &&
+                        region_strictly_inside<K::TRI>(rb, rb + RB, c0 - SH, c0 + TC);
       if (fast) {
         P av[RU][CU];
         const T* at = a_rb + c0;
@@ -199,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
               if (K::ROWOUT) rowacc[ru] = av[ru][u].v[e] * xcv[c][u][e] + rowacc[ru];
               if (K::COLOUT) colacc[c][u][e] = av[ru][u].v[e] * xrv[ru] + colacc[c][u][e];
             }
-      } else if (K::TRI == TRI_FULL && (V == 1 || (c1 - c0) % V == 0)) {
+      } else if (!SHIFT && K::TRI == TRI_FULL && (V == 1 || (c1 - c0) % V == 0)) {
         // gemv: a tile that the matrix edge cuts (fewer rows than RB, or a row that ends on a
         // pack boundary before the tile does): the loads still go out together, each under its
         // own row / pack predicate.  Narrow matrices (fewer columns than one tile) and short
@@ -235,7 +258,8 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
         // issued one by one between the branches made such a tile last several memory latencies.
         const int64_t d64 = c0 - rb;
         const int d = (int)(d64 > (1 << 24) ? (1 << 24) : d64 < -(1 << 24) ? -(1 << 24) : d64);
-        const int nc = (int)(c1 - c0);
+        const int nc = (int)(p.cols - c0 < TC + SH ? p.cols - c0 : TC + SH);  // local columns that exist (of those before the tile: SHIFT)
+        const int lo = SHIFT && c0 == 0 ? 0 : -SH;                            // first local column that exists
         const T* at = a_rb + c0;
         P av[RU][CU];
 #pragma unroll
@@ -243,27 +267,28 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
           const int li = lrow0 + ru * kWarps * G;
 #pragma unroll
           for (int u = 0; u < CU; ++u) {
-            const int lc = (u * LPR + q) * V;
+            const int lc = (u * LPR + q) * V - s;
             bool use = li < nr && lc < nc;
             if (K::TRI == TRI_UPPER) use = use && d + lc + V - 1 >= li;
             if (K::TRI == TRI_LOWER) use = use && d + lc <= li;
-            av[ru][u] = ld_nc_if<T, V>(at + ru * rstride + u * (LPR * V), use && (V == 1 || lc + V <= nc));
+            av[ru][u] = ld_nc_if<T, V>(at + ru * rstride + u * (LPR * V), use && (V == 1 || (lc + V <= nc && (!SHIFT || lc >= lo))));
           }
         }
-        if (V > 1 && nc % V != 0) {  // the rows end inside a pack: that pack element by element
+        if (V > 1 && (SHIFT || nc % V != 0)) {  // the rows start or end inside a pack: that pack element by element
 #pragma unroll
-          for (int ru = 0; ru < RU; ++ru) {
-            const int li = lrow0 + ru * kWarps * G;
+          for (int u = 0; u < CU; ++u) {
+            const int lc = (u * LPR + q) * V - s;
+            if (lc < nc && (lc + V > nc || (SHIFT && lc < lo))) {  // (one branch; the loads below are predicated, not branched)
 #pragma unroll
-            for (int u = 0; u < CU; ++u) {
-              const int lc = (u * LPR + q) * V;
-              bool use = li < nr && lc < nc && lc + V > nc;
-              if (K::TRI == TRI_UPPER) use = use && d + lc + V - 1 >= li;
-              if (K::TRI == TRI_LOWER) use = use && d + lc <= li;
-              const T* ap = at + ru * rstride + u * (LPR * V);
+              for (int ru = 0; ru < RU; ++ru) {
+                const int li = lrow0 + ru * kWarps * G;
+                bool use = li < nr;
+                if (K::TRI == TRI_UPPER) use = use && d + lc + V - 1 >= li;
+                if (K::TRI == TRI_LOWER) use = use && d + lc <= li;
+                const T* ap = at + ru * rstride + u * (LPR * V);
 #pragma unroll
-              for (int e = 0; e < V; ++e)
-                if (use && lc + e < nc) av[ru][u].v[e] = __ldg(ap + e);
+                for (int e = 0; e < V; ++e) av[ru][u].v[e] = ld_el_if<T>(ap + e, use && lc + e < nc && (!SHIFT || lc + e >= lo));
+              }
             }
           }
         }
@@ -272,11 +297,11 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
           const int li = lrow0 + ru * kWarps * G;
 #pragma unroll
           for (int u = 0; u < CU; ++u) {
-            const int lc = (u * LPR + q) * V;
+            const int lc = (u * LPR + q) * V - s;
 #pragma unroll
             for (int e = 0; e < V; ++e) {
               const int lj = lc + e;
-              bool in = li < nr && lj < nc;
+              bool in = li < nr && lj < nc && (!SHIFT || lj >= lo);
               if (K::TRI == TRI_UPPER) in = in && d + lj >= li;
               if (K::TRI == TRI_LOWER) in = in && d + lj <= li;
               const bool dg = (K::TRI != TRI_FULL) && (d + lj == li);
@@ -292,38 +317,41 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
     }  // slot c
     if (K::ROWOUT) {  // all RU row sums in one transposing butterfly
       constexpr int LPV = LPR / RU;  // lanes left per row after the reduction
-      const T s = multi_group_sum<LPR, RU>(rowacc, lane);
+      const T sum = multi_group_sum<LPR, RU>(rowacc, lane);
       const int64_t i = rb + ((q / LPV) * kWarps + warp) * G + g;
       if (q % LPV == 0 && i < r_end) {
         if (p.direct) {
           T* yp = p.y + i * p.incy;
-          B2_STORE(yp, p.beta != T(0) ? p.alpha * s + p.beta * *yp : p.alpha * s);
+          B2_STORE(yp, p.beta != T(0) ? p.alpha * sum + p.beta * *yp : p.alpha * sum);
         } else {
-          p.rowpart[(int64_t)cs * p.rows + i] = s;
+          p.rowpart[(int64_t)cs * p.rows + i] = sum;
         }
       }
     }
   }
 
   if constexpr (K::COLOUT) {  // NCT column tiles per block for these kinds
-    __shared__ T sm[kWarps][NCT * TC];
+    __shared__ T sm[kWarps][NCT * TC + SH];  // SHIFT: entry t is column c_lo - SH + t
+    if (SHIFT && lane < SH) sm[warp][lane < SH - s ? lane : TC + lane] = T(0);
 #pragma unroll
     for (int c = 0; c < NCT; ++c)
 #pragma unroll
       for (int u = 0; u < CU; ++u)
 #pragma unroll
         for (int e = 0; e < V; ++e) {
-          const T s = cross_group_sum<LPR>(colacc[c][u][e]);
-          if (g == 0) sm[warp][c * TC + (u * LPR + q) * V + e] = s;
+          const T sum = cross_group_sum<LPR>(colacc[c][u][e]);
+          if (g == 0) sm[warp][c * TC + (u * LPR + q) * V + e + SH - s] = sum;
         }
     __syncthreads();
-    for (int t = threadIdx.x; t < NCT * TC; t += kThreads) {
-      const int64_t j = c_lo + t;
+    for (int t = threadIdx.x; t < NCT * TC + SH; t += kThreads) {
+      const int64_t j = c_lo - SH + t;
       if (j >= p.cols) break;
       T s = sm[0][t];
 #pragma unroll
       for (int w = 1; w < kWarps; ++w) s += sm[w][t];
-      if (p.direct) {
+      if (SHIFT && t < SH) {
+        p.colspill[(rs * p.nct + cs) * SH + t] = s;
+      } else if (p.direct) {
         T* yp = p.y + j * p.incy;
         B2_STORE(yp, p.beta != T(0) ? p.alpha * s + p.beta * *yp : p.alpha * s);
       } else {
@@ -337,8 +365,9 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
 // A block handles 256/SLICES consecutive outputs; SLICES threads share one output and split
 // its list of partials (slice k takes partials k, k+SLICES, ...), then combine through shared
 // memory in slice order.  Launched as a programmatic dependent of the tile kernel.
+// SH: columns before its own that a tile of the first pass covers (SHIFT: V - 1, else 0).
 template <typename T, class K, int SLICES>
-__global__ void __launch_bounds__(kThreads) l2_finalize(const L2Args<T> p, int RB, int TC) {
+__global__ void __launch_bounds__(kThreads) l2_finalize(const L2Args<T> p, int RB, int TC, int SH) {
   constexpr int OUTB = kThreads / SLICES;
   __shared__ T sm[SLICES][OUTB];
   grid_dep_wait();
@@ -366,7 +395,7 @@ __global__ void __launch_bounds__(kThreads) l2_finalize(const L2Args<T> p, int R
           const int cs = cs0 + k * SLICES;
           const int64_t c_lo = (int64_t)cs * p.ctiles_per_cta * TC;
           const int64_t c_hi = min(p.cols, c_lo + (int64_t)p.ctiles_per_cta * TC);
-          act[k] = cs < p.ncs && region_active<K::TRI>(rb, rb_end, c_lo, c_hi);
+          act[k] = cs < p.ncs && region_active<K::TRI>(rb, rb_end, c_lo - SH, c_hi);
           v[k] = act[k] ? __ldcg(p.rowpart + (int64_t)cs * p.rows + i) : T(0);
         }
 #pragma unroll
@@ -387,12 +416,19 @@ __global__ void __launch_bounds__(kThreads) l2_finalize(const L2Args<T> p, int R
         for (int k = 0; k < 4; ++k) {
           const int64_t rs = rs0 + k * SLICES;
           const int64_t r_begin = rs * p.rows_per_cta, r_end = min(p.rows, r_begin + p.rows_per_cta);
-          act[k] = rs < p.nrs && region_active<K::TRI>(r_begin, r_end, c_lo, c_hi);
+          act[k] = rs < p.nrs && region_active<K::TRI>(r_begin, r_end, c_lo - SH, c_hi);
           v[k] = act[k] ? __ldcg(p.colpart + rs * p.cols + i) : T(0);
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           if (act[k]) s += v[k];
+      }
+      if (SH > 0 && i - c_lo >= span - SH && i / span + 1 < p.nct) {  // the next tile's share of the last columns
+        const int64_t n_lo = c_lo + span, n_hi = min(p.cols, n_lo + span);
+        const T* sp = p.colspill + (i / span + 1) * SH + (i - c_lo - (span - SH));
+        for (int64_t rs = slice; rs < p.nrs; rs += SLICES)
+          if (region_active<K::TRI>(rs * p.rows_per_cta, min(p.rows, (rs + 1) * p.rows_per_cta), n_lo - SH, n_hi))
+            s += __ldcg(sp + rs * p.nct * SH);
       }
     }
   }
@@ -426,7 +462,7 @@ struct L2Plan {
 };
 
 template <typename T, class K, int SLICES>
-static void launch_finalize(const Launch& l, const L2Args<T>& args, int RB, int TC, int64_t nout) {
+static void launch_finalize(const Launch& l, const L2Args<T>& args, int RB, int TC, int64_t nout, int SH = 0) {
   constexpr int OUTB = kThreads / SLICES;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((nout + OUTB - 1) / OUTB));
@@ -437,17 +473,17 @@ static void launch_finalize(const Launch& l, const L2Args<T>& args, int RB, int 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = knob(kKnobUsePdl) ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, l2_finalize<T, K, SLICES>, args, RB, TC);
+  cudaLaunchKernelEx(&cfg, l2_finalize<T, K, SLICES>, args, RB, TC, SH);
 }
 
 // Launches the tile kernel (+ finalize when partials are needed) for one shape.
-template <typename T, int V, class K, class S>
+template <typename T, int V, class K, class S, bool SHIFT = false>
 static int l2_launch_shape(const Launch& l, L2Args<T> args, int64_t rows_per_cta, int ctiles_per_cta,
                            bool allow_direct) {
   constexpr int TC = S::template tc<V>();
-  constexpr int RB = S::RB;
-  args.nct = (int)((args.cols + TC - 1) / TC);
-  args.xc_vec = (K::ROWOUT && V > 1 && aligned_to(args.xc, 16)) ? (args.incxc == 1 ? 1 : args.incxc == 2 ? 2 : 0) : 0;
+  constexpr int RB = S::RB, SH = SHIFT ? V - 1 : 0;
+  args.nct = (int)((args.cols + SH + TC - 1) / TC);
+  args.xc_vec = (!SHIFT && K::ROWOUT && V > 1 && aligned_to(args.xc, 16)) ? (args.incxc == 1 ? 1 : args.incxc == 2 ? 2 : 0) : 0;
   if (K::COLOUT) ctiles_per_cta = S::NCT;
   if (ctiles_per_cta < 1) ctiles_per_cta = 1;
   if (ctiles_per_cta > args.nct) ctiles_per_cta = args.nct;
@@ -458,16 +494,18 @@ static int l2_launch_shape(const Launch& l, L2Args<T> args, int64_t rows_per_cta
     args.ctiles_per_cta = ctiles_per_cta;
     args.nrs = (int)((args.rows + rows_per_cta - 1) / rows_per_cta);
     args.ncs = (args.nct + ctiles_per_cta - 1) / ctiles_per_cta;
-    const bool single = (!K::ROWOUT || args.ncs == 1) && (!K::COLOUT || args.nrs == 1) && !(K::ROWOUT && K::COLOUT);
+    const bool single = (!K::ROWOUT || args.ncs == 1) && (!K::COLOUT || (args.nrs == 1 && !SHIFT)) && !(K::ROWOUT && K::COLOUT);
     args.direct = allow_direct && single;
     if (args.direct) break;
     size_t need = 0;
     if (K::ROWOUT) need += (size_t)args.ncs * args.rows * sizeof(T);
     const size_t row_bytes = (need + 255) / 256 * 256;
-    if (K::COLOUT) need = row_bytes + (size_t)args.nrs * args.cols * sizeof(T);
+    const size_t col_bytes = ((K::COLOUT ? (size_t)args.nrs * args.cols * sizeof(T) : 0) + 255) / 256 * 256;
+    if (K::COLOUT) need = row_bytes + (SHIFT ? col_bytes + (size_t)args.nrs * args.nct * SH * sizeof(T) : (size_t)args.nrs * args.cols * sizeof(T));
     if (need <= l.scratch_bytes) {
       args.rowpart = reinterpret_cast<T*>(l.scratch);
       args.colpart = reinterpret_cast<T*>(l.scratch + row_bytes);
+      args.colspill = reinterpret_cast<T*>(l.scratch + row_bytes + col_bytes);
       break;
     }
     // (a block of a column-sum kind walks exactly S::NCT column tiles -- their sums sit in its
@@ -480,14 +518,14 @@ static int l2_launch_shape(const Launch& l, L2Args<T> args, int64_t rows_per_cta
   }
   const int64_t nblocks = (int64_t)args.nrs * args.ncs;
   if (nblocks > 0x7fffffff) return B2_STATUS_NOT_IMPLEMENTED;
-  launch_chained(l2_tile_kernel<T, V, K, S>, dim3((unsigned)nblocks), dim3(kThreads), 0, l.stream, args);
+  launch_chained(l2_tile_kernel<T, V, K, S, SHIFT>, dim3((unsigned)nblocks), dim3(kThreads), 0, l.stream, args);
   if (int st = check_launch()) return st;
   if (!args.direct) {
     const int64_t nout = K::ROWOUT ? args.rows : args.cols;
     const int nparts = (K::ROWOUT ? args.ncs : 0) + (K::COLOUT ? args.nrs : 0);
-    if (nparts >= 512) launch_finalize<T, K, 32>(l, args, RB, TC, nout);
-    else if (nparts >= 12) launch_finalize<T, K, 8>(l, args, RB, TC, nout);
-    else launch_finalize<T, K, 1>(l, args, RB, TC, nout);
+    if (nparts >= 512) launch_finalize<T, K, 32>(l, args, RB, TC, nout, SH);
+    else if (nparts >= 12) launch_finalize<T, K, 8>(l, args, RB, TC, nout, SH);
+    else launch_finalize<T, K, 1>(l, args, RB, TC, nout, SH);
     if (int st = check_launch()) return st;
   }
   return B2_STATUS_OK;
@@ -531,11 +569,26 @@ static int l2_launch(const Launch& l, const L2Args<T>& args, const L2Plan& plan,
   return l2_launch_shape<T, V, K, ShapeMid>(l, args, plan.rows_per_cta, plan.ctiles_per_cta, allow_direct);
 }
 
+// Rows off 16-byte boundaries in shifted packs: where a row has more packs than the narrow shapes give it lanes and
+// there is a whole step of rows.  In double, where element loads are only twice as many, they stay ahead for the
+// kinds with one sum per element (gemv 8193 x 8191 175 us against 193, trmv n = 8191 95 against 112) and lose for
+// symv (142 against 120).  Float: symv n = 8191 120 -> 72 us a pair, 11519 210 -> 115, trmv 8191 67 -> 58 with its
+// copy, 11519 124 -> 100, gemv 8193 x 8191 108 -> 94.
+template <typename T>
+static bool l2_shift(const L2Args<T>& a, bool sym) {
+  constexpr int V = VecLen<T>::value;
+  return (sizeof(T) == 4 || sym) && !(aligned_to(a.a, 16) && a.lda % V == 0) && a.cols > 16 * V && a.rows >= ShapeMid::RB;
+}
+
 // Picks the pack width: 16-byte packs need a 16-byte aligned base and row stride.
 template <typename T, class K, bool NARROW>
 static int l2_dispatch(const Launch& l, const L2Args<T>& args, const L2Plan& plan, bool allow_direct) {
   constexpr int V = VecLen<T>::value;
   if (aligned_to(args.a, 16) && args.lda % V == 0) return l2_launch<T, V, K, NARROW>(l, args, plan, allow_direct);
+  if (l2_shift(args, K::SYM) && plan.shape == SHAPE_MID) {
+    const int st = l2_launch_shape<T, V, K, ShapeMid, true>(l, args, plan.rows_per_cta, plan.ctiles_per_cta, allow_direct);
+    if (st != B2_STATUS_WORKSPACE_TOO_SMALL) return st;
+  }
   return l2_launch<T, 1, K, NARROW>(l, args, plan, allow_direct);
 }
 
@@ -543,10 +596,11 @@ static int l2_dispatch(const Launch& l, const L2Args<T>& args, const L2Plan& pla
 // block streams about `tile_bytes`; the remaining column splits become partials.
 template <typename T>
 static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) ? VecLen<T>::value : 1;
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, false) ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
-  p.shape = nv >= 128 ? SHAPE_WIDE : (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
+  // (shifted packs: short segments, 4 x values for 8 packs instead of 16)
+  p.shape = nv >= 128 && !l2_shift(a, false) ? SHAPE_WIDE : (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
   const int64_t tile_bytes = (int64_t)shape_rb(p.shape) * shape_packs_per_row(p.shape) * V * sizeof(T);
   int64_t cpc = knob(kKnobGemvNTileBytes) / tile_bytes;
   if (cpc < 1) cpc = 1;
@@ -566,7 +620,7 @@ static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok) {
 // COLOUT kinds: one column tile per block, tall row bands; the bands become partials.
 template <typename T>
 static L2Plan plan_colout(const L2Args<T>& a, bool narrow_ok, int64_t rows_per_cta) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) ? VecLen<T>::value : 1;
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, false) ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
   p.shape = (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;

@@ -24,10 +24,10 @@ static int check_square(int order, int64_t n, const T* a, int64_t lda, int arg_o
 
 template <typename T>
 static L2Plan plan_tri(const L2Args<T>& a) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) ? VecLen<T>::value : 1;
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, true) ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
-  p.shape = (nv >= 512 && knob(kKnobTriWide)) ? SHAPE_WIDE : SHAPE_MID;
+  p.shape = (nv >= 512 && !l2_shift(a, true) && knob(kKnobTriWide)) ? SHAPE_WIDE : SHAPE_MID;
   p.ctiles_per_cta = 1;
   p.rows_per_cta = knob(kKnobTriRows);
   return p;
