@@ -182,6 +182,40 @@ __device__ __forceinline__ T ld_el_if(const T* p, bool pred) {
   }
 }
 
+// The same for data that this kernel writes back (L2 only): a pack, an element.
+template <typename T, int N>
+__device__ __forceinline__ Pack<T, N> ld_cg_if(const T* p, bool pred) {
+  if (pred && !B2_GUARD(p, sizeof(T) * N)) pred = false;
+  Pack<T, N> r;
+  if constexpr (sizeof(T) * N == 16) {
+    uint4 t;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\tmov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\tmov.u32 %3, 0;\n\t"
+        "@q ld.global.cg.v4.u32 {%0,%1,%2,%3}, [%4];\n\t}"
+        : "=&r"(t.x), "=&r"(t.y), "=&r"(t.z), "=&r"(t.w)
+        : "l"(p), "r"((unsigned)pred)
+        : "memory");
+    r = *reinterpret_cast<Pack<T, N>*>(&t);
+  } else if constexpr (sizeof(T) == 4) {
+    static_assert(N == 1, "packs are 16 bytes or one element");
+    unsigned t;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u32 %0, 0;\n\t@q ld.global.cg.u32 %0, [%1];\n\t}"
+                 : "=&r"(t)
+                 : "l"(p), "r"((unsigned)pred)
+                 : "memory");
+    r.v[0] = *reinterpret_cast<T*>(&t);
+  } else {
+    static_assert(N == 1, "packs are 16 bytes or one element");
+    unsigned long long t;
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\tmov.u64 %0, 0;\n\t@q ld.global.cg.u64 %0, [%1];\n\t}"
+                 : "=&l"(t)
+                 : "l"(p), "r"((unsigned)pred)
+                 : "memory");
+    r.v[0] = *reinterpret_cast<T*>(&t);
+  }
+  return r;
+}
+
 // Read-only load of reused data (the x vectors): cached in L1.
 template <typename T, int N>
 __device__ __forceinline__ Pack<T, N> ld_ro(const T* p) {

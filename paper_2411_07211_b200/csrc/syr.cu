@@ -51,8 +51,13 @@ __device__ __forceinline__ void syr_tile_of_block(unsigned b, int m, int nct, bo
 }
 
 // Canonical row-major view: `lower` means the stored triangle has column <= row there.
+// Resident blocks the registers are cut for: element-wise tiles are small, so many of them must be in flight.
 template <typename T, int V, bool TWO>
-__global__ void __launch_bounds__(kThreads, TWO ? 3 : 4) syr_kernel(T* __restrict__ a, int64_t lda, int64_t n,
+constexpr int syr_blocks() {
+  return V > 1 ? (TWO ? 3 : 4) : TWO ? 5 : sizeof(T) == 4 ? 8 : 6;
+}
+template <typename T, int V, bool TWO>
+__global__ void __launch_bounds__(kThreads, (syr_blocks<T, V, TWO>())) syr_kernel(T* __restrict__ a, int64_t lda, int64_t n,
                                                        const T* __restrict__ x, int64_t incx,
                                                        const T* __restrict__ y, int64_t incy, T alpha, bool lower,
                                                        int nct) {
@@ -128,36 +133,55 @@ __global__ void __launch_bounds__(kThreads, TWO ? 3 : 4) syr_kernel(T* __restric
     }
     return;
   }
-  // a tile that the diagonal or the matrix edge cuts: row by row; a pack that lies inside whole
-  // is still moved as one, a pack that is cut goes element by element.  Columns are counted
-  // from c0 here: jr in [0, TC), the matrix ends at ncols, row i has its diagonal at jd.
+  // a tile that the diagonal or the matrix edge cuts: a pack that lies inside whole is still moved as one, a pack
+  // that is cut goes element by element; all loads of the tile go out together, each under its predicate (one by
+  // one, each behind the store before it, such a tile lasted a dozen memory latencies: n = 500 5.8 -> 3.3 us).
+  // Columns are counted from c0 here: jr in [0, TC), the matrix ends at ncols, row i has its diagonal at jd.
   const int ncols = (int)min((int64_t)TC, n - c0);
-  for (int rr = warp; rr < kSyrRows; rr += kWarps) {
-    const int64_t i = r0 + rr;
-    if (i >= n) break;
+  int lo[kSyrRU], hi[kSyrRU];  // columns [lo, hi) of the row are inside
+#pragma unroll
+  for (int ru = 0; ru < kSyrRU; ++ru) {
+    const int64_t i = r0 + ru * kWarps + warp;
     const int jd = (int)max((int64_t)-1, min((int64_t)TC, i - c0));
-    const int lo = lower ? 0 : jd, hi = lower ? min(jd + 1, ncols) : ncols;  // columns [lo, hi) are inside
-    const T xi = sxi[rr];
-    const T yi = TWO ? syi[rr] : T(0);
-    T* arow = a + i * lda + c0;
+    lo[ru] = lower ? 0 : jd;
+    hi[ru] = i < n ? (lower ? min(jd + 1, ncols) : ncols) : 0;
+    ap[ru] = a + i * lda + c0 + lane * V;
 #pragma unroll
     for (int u = 0; u < kSyrCU; ++u) {
       const int jr = (u * 32 + lane) * V;
-      if (V > 1 && jr >= lo && jr + V <= hi) {
-        P av = ld_cg<T, V>(arow + jr);
+      av[ru][u] = ld_cg_if<T, V>(ap[ru] + u * 32 * V, jr >= lo[ru] && jr + V <= hi[ru]);
+    }
+  }
+  if (V > 1) {
 #pragma unroll
-        for (int e = 0; e < V; ++e) {
-          if (TWO) av.v[e] = yi * xj[u][e] + (xi * yj[u][e] + av.v[e]);
-          else av.v[e] = xi * xj[u][e] + av.v[e];
+    for (int ru = 0; ru < kSyrRU; ++ru)
+#pragma unroll
+      for (int u = 0; u < kSyrCU; ++u) {
+        const int jr = (u * 32 + lane) * V;
+        if (jr < hi[ru] && jr + V > lo[ru] && !(jr >= lo[ru] && jr + V <= hi[ru])) {
+#pragma unroll
+          for (int e = 0; e < V; ++e) av[ru][u].v[e] = ld_cg_if<T, 1>(ap[ru] + u * 32 * V + e, jr + e >= lo[ru] && jr + e < hi[ru]).v[0];
         }
-        st_cs<T, V>(arow + jr, av);
-      } else {
+      }
+  }
+#pragma unroll
+  for (int ru = 0; ru < kSyrRU; ++ru) {
+    const T xi = sxi[ru * kWarps + warp];
+    const T yi = TWO ? syi[ru * kWarps + warp] : T(0);
+#pragma unroll
+    for (int u = 0; u < kSyrCU; ++u) {
+      const int jr = (u * 32 + lane) * V;
+#pragma unroll
+      for (int e = 0; e < V; ++e) {
+        if (TWO) av[ru][u].v[e] = yi * xj[u][e] + (xi * yj[u][e] + av[ru][u].v[e]);
+        else av[ru][u].v[e] = xi * xj[u][e] + av[ru][u].v[e];
+      }
+      if (jr >= lo[ru] && jr + V <= hi[ru]) {
+        st_cs<T, V>(ap[ru] + u * 32 * V, av[ru][u]);
+      } else if (V > 1) {
 #pragma unroll
         for (int e = 0; e < V; ++e)
-          if (jr + e >= lo && jr + e < hi) {
-            if (TWO) arow[jr + e] = yi * xj[u][e] + (xi * yj[u][e] + arow[jr + e]);
-            else arow[jr + e] = xi * xj[u][e] + arow[jr + e];
-          }
+          if (jr + e >= lo[ru] && jr + e < hi[ru]) B2_STORE(ap[ru] + u * 32 * V + e, av[ru][u].v[e]);
       }
     }
   }

@@ -257,6 +257,21 @@ def test_trsv_every_kernel_choice(b2, ctx, dtype, front, cluster, pm_from):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("m,n", [(1, 5), (3, 1), (7, 3), (257, 31), (1025, 1), (2, 4099), (4100, 3), (1024, 5)])
+def test_ger_unpadded_odd_widths(b2, ctx, dtype, m, n):
+    """Matrices that are one contiguous run with rows off 16-byte boundaries: elements before the first and after the
+    last pack, packs that hold several rows, one row per element, rows longer than a chunk."""
+    for off, incx, incy in ((0, 1, 1), (1, 2, -1), (3, -1, 3)):
+        a, x, y = synth.matrix_np(3, m, m, n, n, dtype).ravel(), synth.vector_np(5, m, m, dtype), synth.vector_np(6, n, n, dtype)
+        ga, gx, gy = Guarded(a, off), Guarded(place(x, incx)), Guarded(place(y, incy))
+        b2.ger(ctx, orc.ROW_MAJOR, m, n, 0.75, gx.t, incx, gy.t, incy, ga.t, n)
+        oa = a.copy()
+        absterms = orc.ger(orc.ROW_MAJOR, m, n, dtype(0.75), place(x, incx), incx, place(y, incy), incy, oa, n)
+        assert_close(ga.host(), oa, np.asarray(absterms).ravel(), dtype, f"ger off={off}")
+        ga.check_guards()
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("mode", [0, 2, 3])
 def test_cluster_gather_kernel(b2, ctx, dtype, mode):
     """The one-launch kernel at its edges: one output more and less than a cluster owns, one element more and less
