@@ -7,6 +7,7 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "b2blas.h"
 
@@ -291,6 +292,30 @@ __device__ __forceinline__ T cross_group_sum(T v) {
   return v;
 }
 
+// Thread-block cluster: rank, size, the two halves of its barrier, a value into rank 0's shared memory.
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+template <typename A>
+__device__ __forceinline__ void st_rank0(A* local, const A& v) {
+  static_assert(sizeof(A) % 4 == 0, "whole words");
+  unsigned r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)));
+  unsigned w[sizeof(A) / 4];
+  memcpy(w, &v, sizeof(A));
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(A) / 4); ++i) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r + 4 * i), "r"(w[i]) : "memory");
+}
+
 // Programmatic dependent launch (PDL): a dependent kernel may start while its predecessor
 // drains; it must call grid_dep_wait() before touching the predecessor's outputs.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -429,6 +454,23 @@ inline void launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);  // (a failure is picked up by check_launch())
 }
 
+// The same as ONE cluster of grid.x blocks.
+template <typename... KArgs, typename... Args>
+inline void launch_one_cluster(void (*kernel)(KArgs...), unsigned blocks, dim3 block, cudaStream_t stream, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = block;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = blocks;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = knob(kKnobUsePdl) ? 2 : 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
 
 // Base pointer such that logical element i lives at base[i*inc] for either sign of inc.
 template <typename T>

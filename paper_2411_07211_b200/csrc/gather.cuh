@@ -51,29 +51,6 @@ struct Args {
 template <typename T>
 __device__ __forceinline__ T ld_x(const T* p) { return B2_GUARD(p, sizeof(T)) ? *p : T(0); }
 
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ unsigned cluster_size() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void st_rank0(float* local, float v) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_rank0(double* local, double v) {
-  unsigned r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(local)));
-  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
-}
-
 // ROWOUT / COLOUT of the kind: row part / column part.  Triangular kinds that are not symmetric work in place.
 template <typename T, bool AL, class K>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kernel(const Args<T> p) {

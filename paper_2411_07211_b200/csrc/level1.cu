@@ -305,15 +305,43 @@ __device__ __forceinline__ typename Op::Acc block_combine(typename Op::Acc a) {
   return a;
 }
 
+// Reductions of few chunks run as one cluster: handing 8 sums to rank 0 through distributed shared memory takes 0.4 us,
+// the fence, ticket and second pass through L2 1.5 us (n = 65536 in float: dot 3.9 -> 2.9 us, asum 4.0 -> 2.6).
+constexpr int kReduceCluster = 8;
+constexpr int64_t kClusterChunks = 16;  // (two chunks per block cost less than the ticket)
+__device__ __forceinline__ void cluster_begin() {
+  if (cluster_size() > 1) cluster_arrive();
+}
+
 // Second pass: each block stores its partial, takes a ticket, and the block that draws the
 // last ticket combines all partials in index order and writes the result.  It also puts the
 // ticket counter back to zero for the next call.
-template <class Op>
+// (CLUSTER: the kernel may be launched as one cluster.  The strided kernel is not: its float dot product comes out with
+// its loads one after the other as soon as anything is added to it, 73 -> 143 us at 20 million elements.)
+template <class Op, bool CLUSTER>
 __device__ __forceinline__ void reduce_finish(typename Op::Acc acc, typename Op::Acc* partials, unsigned* ticket,
                                               typename Op::Out* result) {
   using Acc = typename Op::Acc;
   __shared__ bool is_last;
   acc = block_combine<Op>(acc);
+  const unsigned nr = CLUSTER ? cluster_size() : 0u;
+  if (CLUSTER && nr == gridDim.x) {  // a single block, or a grid that is one cluster: sums meet in rank 0's shared memory
+    __shared__ __align__(16) unsigned char raw[kReduceCluster * sizeof(Acc)];
+    Acc* const ranks = reinterpret_cast<Acc*>(raw);
+    if (nr > 1) {
+      __syncwarp();
+      cluster_wait();  // (begun by cluster_begin: every block is running)
+      if (threadIdx.x == 0 && blockIdx.x != 0) st_rank0(&ranks[blockIdx.x], acc);
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      for (unsigned b = 1; b < nr; ++b) acc = Op::combine(acc, ranks[b]);
+      *result = Op::finalize(acc);
+    }
+    return;
+  }
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = acc;
     __threadfence();
@@ -344,6 +372,7 @@ __global__ void __launch_bounds__(kThreads) l1_reduce_unit(const T* __restrict__
                                                            int64_t head, int64_t nvec, int64_t nchunks,
                                                            typename Op::Acc* partials, unsigned* ticket,
                                                            typename Op::Out* result) {
+  cluster_begin();
   grid_dep_wait();
   grid_dep_launch();
   constexpr int V = VecLen<T>::value;
@@ -448,7 +477,7 @@ __global__ void __launch_bounds__(kThreads) l1_reduce_unit(const T* __restrict__
       a = Op::combine(a, e);
     }
   }
-  reduce_finish<Op>(a, partials, ticket, result);
+  reduce_finish<Op, true>(a, partials, ticket, result);
 }
 
 template <typename T, class Op, int NE>
@@ -508,7 +537,7 @@ __global__ void __launch_bounds__(kThreads) l1_reduce_strided(const T* __restric
 #pragma unroll
     for (int k = 0; k < NE; ++k) r = Op::combine(r, Op::slot_to_acc(acc[k], 0, 0));
   }
-  reduce_finish<Op>(r, partials, ticket, result);
+  reduce_finish<Op, false>(r, partials, ticket, result);
 }
 
 // sdsdot's last step: result = (float)(sb + the double-accumulated dot), rounded once.
@@ -582,6 +611,8 @@ static int run_map(const b2_ctx* ctx, Op op, int64_t n, T* x, int64_t incx, T* y
   return check_launch();
 }
 
+static unsigned cluster_blocks(int64_t nchunks) { return nchunks < kReduceCluster ? (unsigned)nchunks : (unsigned)kReduceCluster; }
+
 template <typename T, class Op>
 static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, const T* y, int64_t incy,
                       typename Op::Out* result) {
@@ -608,6 +639,11 @@ static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, co
     if (head > n) head = n;
     const int64_t nvec = (n - head) / V;
     const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV);
+    if (nchunks > 1 && nchunks <= kClusterChunks) {
+      launch_one_cluster(l1_reduce_unit<T, Op, NV>, cluster_blocks(nchunks), dim3(kThreads), l.stream, x, Op::RY ? y : x, n, head, nvec, nchunks, partials,
+                         ticket, result);
+      return check_launch();
+    }
     static WaveCache wc;
     const int wave = one_wave(l1_reduce_unit<T, Op, NV>, cap, wc);
     const int64_t grid = nchunks < 1 ? 1 : (nchunks > wave ? wave : nchunks);
@@ -620,6 +656,11 @@ static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, co
     if (head > span) head = span;
     const int64_t nvec = (span - head) / V;
     const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV);
+    if (nchunks > 1 && nchunks <= kClusterChunks) {
+      launch_one_cluster(l1_reduce_unit<T, Op, NV, 2>, cluster_blocks(nchunks), dim3(kThreads), l.stream, x, Op::RY ? y : x, span, head, nvec, nchunks,
+                         partials, ticket, result);
+      return check_launch();
+    }
     static WaveCache wc;
     const int wave = one_wave(l1_reduce_unit<T, Op, NV, 2>, cap, wc);
     const int64_t grid = nchunks < 1 ? 1 : (nchunks > wave ? wave : nchunks);
