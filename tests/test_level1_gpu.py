@@ -171,6 +171,35 @@ def test_small_integer_reductions_are_bit_exact(b2, ctx, dtype):
         assert got[1] == orc.asum(n, x, 1)[0] == float(np.abs(x).sum())
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("inc", [1, 2])
+@pytest.mark.parametrize("chunks", [1, 2, 8, 9, 16, 17])
+def test_reductions_at_the_cluster_edges(b2, ctx, dtype, inc, chunks):
+    """One block, a cluster of up to eight (one or two chunks of 16 or 32 KB each) and the ticketed grid:
+    whole numbers, so every result is exact, and one largest element at either end for iamax."""
+    rng = np.random.default_rng(chunks)
+    tdt = torch.float32 if dtype == np.float32 else torch.float64
+    for chunk_bytes in (16384, 32768):
+        edge = chunks * chunk_bytes // np.dtype(dtype).itemsize // inc
+        for n in (edge - 1, edge, edge + 1):
+            x = rng.integers(-2, 3, size=n).astype(dtype)
+            y = rng.integers(-2, 3, size=n).astype(dtype)
+            x[-1 if n % 2 else 0] = -3
+            gx, gy = Guarded(place(x, inc), n % 2), Guarded(place(y, inc), n % 2)
+            res = torch.zeros(3, dtype=tdt, device="cuda")
+            ires = torch.full((1,), -7, dtype=torch.int64, device="cuda")
+            b2.dot(ctx, n, gx.t, inc, gy.t, inc, res[0:1])
+            b2.asum(ctx, n, gx.t, inc, res[1:2])
+            b2.nrm2(ctx, n, gx.t, inc, res[2:3])
+            b2.iamax(ctx, n, gx.t, inc, ires)
+            got = res.cpu().numpy()
+            xi = x.astype(np.int64)
+            assert got[0] == np.dot(xi, y.astype(np.int64)) and got[1] == np.abs(xi).sum()
+            nrm = np.sqrt(float(np.dot(xi, xi)))
+            assert_close(got[2], nrm, nrm, dtype, "nrm2")
+            assert int(ires.item()) == (n - 1 if n % 2 else 0)
+
+
 def test_sdot_config1_matches_golden(b2, ctx):
     """n = 1,048,576 f32, seed 0: the device generator feeds the kernel, the stored oracle value
     (tests/golden) is the reference."""
