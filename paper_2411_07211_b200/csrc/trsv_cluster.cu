@@ -239,7 +239,8 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
   int pj = 0, plo = 0, ps = 0, pslot = 0;
   const T* const at = p.a + (COLTYPE ? (int64_t)(b.warp * (NB / kCW) + b.lane / ST::LPR) * p.lda + (b.lane % ST::LPR) * V
                                      : (int64_t)(b.warp * kTilePacks) * p.lda + b.lane * V);
-  const int64_t step_a = COLTYPE ? ST::GR * p.lda : p.lda;
+  const T* const uat = p.a + (COLTYPE ? (int64_t)(b.warp * (NB / kCW)) * p.lda : (int64_t)(b.warp * kTilePacks) * p.lda) + b.lane;
+  const int64_t step_a = COLTYPE ? ST::GR * p.lda : p.lda, step_e = COLTYPE ? p.lda : 32;  // (step_e: see copy_warp)
   const int64_t jstep = (COLTYPE ? p.lda : 1) * (p.backward ? -NB : NB);  // from a block column to the next in solve order
   const int64_t j0off = (COLTYPE ? p.lda : 1) * (int64_t)mem_block(p, 0) * NB;
   auto produce = [&]() {
@@ -248,13 +249,24 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
       const bool both = pj < s_last[ps];
       const bool whole = ragged < 0 || (p.backward ? pj > 0 : (q0 + ps * H) / SPB != ragged);
       if (whole) {
-        const T* src = at + s_base[ps] + j0off + pj * jstep;
+        const int64_t tile = s_base[ps] + j0off + pj * jstep;
+        if constexpr (AL) {
+          const T* src = at + tile;
 #pragma unroll
-        for (int r = 0; r < kTilePacks; ++r) copy_pack_full<T, AL>(dst + (size_t)r * kCT * V, src + r * step_a);
-        if (both) {
+          for (int r = 0; r < kTilePacks; ++r) cp_async16_full(dst + (size_t)r * kCT * V, src + r * step_a);
+          if (both) {
 #pragma unroll
-          for (int r = 0; r < kTilePacks; ++r)
-            copy_pack_full<T, AL>(dst + (size_t)(kTilePacks + r) * kCT * V, src + jstep + r * step_a);
+            for (int r = 0; r < kTilePacks; ++r) cp_async16_full(dst + (size_t)(kTilePacks + r) * kCT * V, src + jstep + r * step_a);
+          }
+        } else {
+          const T* src = uat + tile;
+          dst -= b.lane * (V - 1);
+#pragma unroll
+          for (int r = 0; r < kTilePacks; ++r) copy_warp(dst + (size_t)r * kCT * V, src + r * step_a, step_e);
+          if (both) {
+#pragma unroll
+            for (int r = 0; r < kTilePacks; ++r) copy_warp(dst + (size_t)(kTilePacks + r) * kCT * V, src + jstep + r * step_a, step_e);
+          }
         }
       } else {
         const int q = q0 + ps * H;
@@ -340,11 +352,13 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
     while (lo < S - 1 && s_last[lo] < j) ++lo;
 #pragma unroll 1
     for (int s = lo; s < S; ++s) {
+      if (!AL) __syncwarp();  // (a warp's copies are spread over its lanes: the slot's readers are done)
       produce();
       const int last_j = s_last[s];
       const T* src = b.big + ((size_t)(slot * 2 * kTilePacks) * kCT + b.tid) * V;
       slot = slot + 1 == kDepth ? 0 : slot + 1;
       cp_async_wait<kDepth - 1>();
+      if (!AL) __syncwarp();
       Pack<T, V> m[2][kTilePacks];
 #pragma unroll
       for (int r = 0; r < 2 * kTilePacks; ++r)
@@ -435,12 +449,25 @@ __device__ __forceinline__ void solve_block(const Args<T>& p, Block<T>& b, int r
       const int I = mem_block(p, nk + nw), J = mem_block(p, nk);
       const int li = block_len(p, I), lj = block_len(p, J);
       T* dst = b.big + (size_t)nslot * NB * NB + (size_t)b.tid * V;
+      if (!AL && li == NB && lj == NB) {
+        const int ru = COLTYPE ? b.warp * JT : 2 * b.warp * RS;  // a warp's packs: one stored row, or halves of two
+        const T* src = p.a + ((int64_t)(COLTYPE ? J : I) * NB + ru) * p.lda + (int64_t)(COLTYPE ? I : J) * NB + b.lane;
+        dst -= b.lane * (V - 1);
+        __syncwarp();
+#pragma unroll
+        for (int m = 0; m < NPK; ++m)
+#pragma unroll
+          for (int e = 0; e < V; ++e) {
+            const int r = COLTYPE ? m : e * 32 / H * RS + m / CP, c = COLTYPE ? e * 32 : (m % CP) * H + e * 32 % H;
+            cp_async_elem<sizeof(T)>(dst + (size_t)m * kCT * V + e * 32, src + r * p.lda + c, true);
+          }
+      } else
 #pragma unroll
       for (int m = 0; m < NPK; ++m) {
         const int r = COLTYPE ? b.warp * JT + m : rg * RS + m / CP, c = COLTYPE ? b.lane * V : (m % CP) * H + cg * V;
         const int rows = COLTYPE ? lj : li, cols = COLTYPE ? li : lj;
         const T* src = p.a + ((int64_t)(COLTYPE ? J : I) * NB + r) * p.lda + (int64_t)(COLTYPE ? I : J) * NB + c;
-        if (li == NB && lj == NB) copy_pack_full<T, AL>(dst + (size_t)m * kCT * V, src);
+        if (AL && li == NB && lj == NB) cp_async16_full(dst + (size_t)m * kCT * V, src);
         else copy_pack<T, AL>(dst + (size_t)m * kCT * V, src, r < rows ? min(V, max(0, cols - c)) : 0, p.a);
       }
       ++nw;
@@ -585,6 +612,7 @@ __device__ __forceinline__ void solve_block(const Args<T>& p, Block<T>& b, int r
 #pragma unroll 1
     for (int w = 2; w <= wn; ++w) {
       cp_async_wait<NEAR - 1>();
+      if (!AL) __syncwarp();
       const T* src = b.big + (size_t)rslot * NB * NB + (size_t)b.tid * V;
 #pragma unroll
       for (int m = 0; m < NPK; ++m) cur[m] = *reinterpret_cast<const P*>(src + (size_t)m * kCT * V);

@@ -172,15 +172,13 @@ __device__ __forceinline__ void copy_pack(T* dst, const T* src, int valid, const
     for (int e = 0; e < V; ++e) cp_async_elem<sizeof(T)>(dst + e, e < valid ? src + e : safe, e < valid);
   }
 }
-template <typename T, bool AL>
-__device__ __forceinline__ void copy_pack_full(T* dst, const T* src) {
-  constexpr int V = 16 / (int)sizeof(T);
-  if constexpr (AL) {
-    cp_async16_full(dst, src);
-  } else {
+// The whole packs of a warp off 16-byte boundaries, element by element: consecutive lanes take consecutive elements
+// (dst, src: this lane's first one; the next 32 of the warp's 32 V elements lie `step` further on in global memory), so
+// that a copy instruction touches one or two lines instead of the four or five of packs.  Readers wait for the warp.
+template <typename T>
+__device__ __forceinline__ void copy_warp(T* dst, const T* src, int64_t step) {
 #pragma unroll
-    for (int e = 0; e < V; ++e) cp_async_elem<sizeof(T)>(dst + e, src + e, true);
-  }
+  for (int e = 0; e < 16 / (int)sizeof(T); ++e) cp_async_elem<sizeof(T)>(dst + e * 32, src + e * step, true);
 }
 
 // Two float multiply-adds in one instruction.
