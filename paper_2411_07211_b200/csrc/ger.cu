@@ -6,8 +6,14 @@
 
 namespace b2 {
 
+// Blocks per SM at least (0: as the compiler likes it): the tiles of a cut matrix, with all their loads in flight, would
+// otherwise take the registers of one of two blocks (packs: 509117 x 32 in double 41 us, 54 with one block) or of one
+// of four (double elements: 100003 x 64 18.8 and 20.4 us; in float the bound only makes the compiler use more).
 template <typename T, int V, class S>
-__global__ void __launch_bounds__(kThreads) ger_kernel(T* __restrict__ a, int64_t lda, int64_t rows, int64_t cols,
+constexpr int kGerBlocks = V > 1 ? 2 : sizeof(T) == 8 && S::CU == 1 ? 4 : 0;
+
+template <typename T, int V, class S>
+__global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* __restrict__ a, int64_t lda, int64_t rows, int64_t cols,
                                                        const T* __restrict__ xr, int64_t incxr,
                                                        const T* __restrict__ yc, int64_t incyc, T alpha,
                                                        int64_t rows_per_cta, int nct) {
@@ -43,7 +49,11 @@ __global__ void __launch_bounds__(kThreads) ger_kernel(T* __restrict__ a, int64_
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
 #pragma unroll
-        for (int u = 0; u < CU; ++u) av[ru][u] = ld_cs<T, V>(a + rowi[ru] * lda + c0 + (u * LPR + q) * V);
+        for (int u = 0; u < CU; ++u) {  // (single elements leave partly written sectors: evict-first ones were gone from
+          // L2 when the stores came, and had to be filled again; 1000000 x 16, lda 19, in double 80 us, 48 so)
+          const T* ap = a + rowi[ru] * lda + c0 + (u * LPR + q) * V;
+          av[ru][u] = V > 1 ? ld_cs<T, V>(ap) : ld_cg<T, V>(ap);
+        }
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
 #pragma unroll
