@@ -184,7 +184,8 @@ def prepare(thunk):
     """Runs `thunk` (calls of this module) once and returns a callable that repeats exactly those
     library calls with the arguments marshalled then -- same stream, same pointers -- without
     going through the interpreter for each of them.  For timing loops over small problems; the
-    returned callable returns the last status."""
+    returned callable returns the last status.  What is recorded are the calls that the thunk makes
+    on the thread that runs it; any number of threads may be inside prepare()."""
     return _native.record(thunk)
 
 

@@ -140,7 +140,9 @@ struct Recording {
     for (PyObject* o : keep) Py_DECREF(o);
   }
 };
-Recording* g_recording = nullptr;
+// The recording that the calls of this thread go to.  (One per thread: prepare() runs Python code, other threads run in
+// between, and their calls, or a second recording of theirs, are not this one's.)
+thread_local Recording* t_recording = nullptr;
 
 // args[0] is the context, args[1..] the arguments of the C function in order.  Returns false with
 // a Python error set when an argument does not convert.
@@ -157,7 +159,7 @@ bool call_typed(void* sym, PyObject* const* args, int* st, std::index_sequence<I
   rc = fn(&c, std::get<I>(a)...);
   Py_END_ALLOW_THREADS
   *st = rc;
-  if (g_recording) g_recording->calls.emplace_back([fn, c, a]() { return fn(&c, std::get<I>(a)...); });
+  if (t_recording) t_recording->calls.emplace_back([fn, c, a]() { return fn(&c, std::get<I>(a)...); });
   return true;
 }
 template <class... A>
@@ -356,11 +358,11 @@ PyType_Spec replay_spec = {"paper_2411_07211_b200._binding.Replay", sizeof(Repla
 PyTypeObject* g_replay_type = nullptr;
 
 PyObject* record(PyObject*, PyObject* thunk) {
-  Recording* const outer = g_recording;
+  Recording* const outer = t_recording;
   Recording* rec = new Recording();
-  g_recording = rec;
+  t_recording = rec;
   PyObject* r = PyObject_CallNoArgs(thunk);
-  g_recording = outer;
+  t_recording = outer;
   ReplayObject* o = r == nullptr ? nullptr : PyObject_New(ReplayObject, g_replay_type);
   Py_XDECREF(r);
   if (o == nullptr) {
@@ -375,7 +377,7 @@ PyObject* record(PyObject*, PyObject* thunk) {
 // keep(obj): while a recording runs, obj lives as long as its replay (host memory that a recorded
 // call points into).
 PyObject* keep(PyObject*, PyObject* obj) {
-  if (g_recording) g_recording->keep.push_back(Py_NewRef(obj));
+  if (t_recording) t_recording->keep.push_back(Py_NewRef(obj));
   Py_RETURN_NONE;
 }
 

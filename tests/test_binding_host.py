@@ -1,0 +1,76 @@
+"""Host side of the Python binding: what needs no GPU."""
+import sys
+import threading
+
+import pytest
+
+
+@pytest.fixture(scope="module")
+def b2():
+    from paper_2411_07211_b200 import build
+    build.build()
+    from paper_2411_07211_b200 import binding
+    return binding
+
+
+def test_recordings_of_two_threads_stay_apart(b2):
+    """Two prepare() calls whose thunks overlap, the first to begin also the first to end: what a thread hands to its
+    recording ends up in that one, and with both over nothing is recorded any more."""
+    began, both, first_over = threading.Event(), threading.Event(), threading.Event()
+    mine = {"a": object(), "b": object(), "after": object()}
+    held = lambda: [sys.getrefcount(mine[k]) for k in ("a", "b", "after")]
+    base = held()
+    over = lambda: [n - m for n, m in zip(held(), base)]  # references taken since then
+    replays = {}
+
+    def a():
+        began.set()
+        assert both.wait(20)
+        b2._native.keep(mine["a"])
+
+    def b():
+        assert began.wait(20)
+        both.set()
+        assert first_over.wait(20)
+        b2._native.keep(mine["b"])
+
+    def run(name, thunk, done=None):
+        replays[name] = b2.prepare(thunk)
+        if done:
+            done.set()
+
+    threads = [threading.Thread(target=run, args=("a", a, first_over)), threading.Thread(target=run, args=("b", b))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join(30)
+    assert set(replays) == {"a", "b"}
+    b2._native.keep(mine["after"])  # (no recording runs: nothing may hold on to it)
+    assert over() == [1, 1, 0]
+    del replays["a"]
+    assert over() == [0, 1, 0]
+    del replays["b"]
+    assert over() == [0, 0, 0]
+
+
+def test_recordings_nest(b2):
+    """A prepare() inside the thunk of another one, ended by an exception too, leaves the outer recording in place."""
+    inner, outer = object(), object()
+    base = sys.getrefcount(inner), sys.getrefcount(outer)
+    got = []
+
+    def fails():
+        raise RuntimeError("stop")
+
+    def thunk():
+        got.append(b2.prepare(lambda: b2._native.keep(inner)))
+        with pytest.raises(RuntimeError, match="stop"):
+            b2.prepare(fails)
+        b2._native.keep(outer)
+
+    replay = b2.prepare(thunk)
+    assert (sys.getrefcount(inner) - base[0], sys.getrefcount(outer) - base[1]) == (1, 1)
+    got.clear()
+    assert (sys.getrefcount(inner) - base[0], sys.getrefcount(outer) - base[1]) == (0, 1)
+    del replay
+    assert sys.getrefcount(outer) == base[1]
