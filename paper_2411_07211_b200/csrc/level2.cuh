@@ -185,9 +185,15 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
   // (gemv, both products of a 16384 matrix, 328 -> 308 us in float, 670 -> 606 in double; symv n = 16384 190 -> 181,
   // trmv n = 4096 in double 34 -> 31.  Not for shifted float rows, which spill here: symv n = 8191 72 -> 77 us.)
   constexpr bool STEADY = K::COLOUT && NCT == 1 && !(SHIFT && sizeof(T) == 4);
+  // CUT: the last column tile of an upper triangle, which is its longest column, takes part when the matrix edge cuts it,
+  // its loads under predicates that do not change along the way.  A step in the general form below lasts half a
+  // microsecond longer here than it does in a kernel without this loop, and with every step of that column in it these
+  // blocks were the tail of the launch: trmv in double, n = 5360, 26.2 us without any such loop, 30.0 with the loop
+  // for whole tiles only, 25.4 so; n = 3008 in float 14.9 -> 9.6; symv in float, n = 7400, 28.4, 30.9, 24.4.
+  constexpr bool CUT = STEADY && !SHIFT && K::TRI == TRI_UPPER;
   int64_t fast_lo = 0, fast_hi = 0;  // first row of the first such step, end of the last
   if constexpr (STEADY) {
-    if (c_lo + TC <= p.cols && (!SHIFT || c_lo > 0)) {
+    if (CUT || (c_lo + TC <= p.cols && (!SHIFT || c_lo > 0))) {
       fast_lo = r_begin, fast_hi = r_end;
       if (K::TRI == TRI_LOWER) fast_lo = max(r_begin, (c_lo + TC - 1) / RB * RB + RB);  // (rows past the last column)
       if (K::TRI == TRI_UPPER) fast_hi = min(r_end, c_lo - SH);
@@ -206,6 +212,55 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
         if (K::ROWOUT && xcv_ct[0] != ct_begin) {
           xcv_ct[0] = ct_begin;
           load_xc(xcv[0], c_lo);
+        }
+        if constexpr (CUT) {
+          if (c_lo + TC > p.cols) {
+            const int nc = (int)(p.cols - c_lo);  // columns that exist
+            auto cut_steps = [&](auto packs) {    // in whole packs, or by elements
+#pragma unroll 1
+              for (int st = 0; st < nst; ++st) {
+                P av[RU][CU];
+                T xv[RU];
+#pragma unroll
+                for (int ru = 0; ru < RU; ++ru)
+#pragma unroll
+                  for (int u = 0; u < CU; ++u) {
+                    const T* ap = at + ru * rstride + u * (LPR * V);
+                    const int lc = (u * LPR + q) * V;
+                    if constexpr (decltype(packs)::value) av[ru][u] = ld_nc_if<T, V>(ap, lc < nc);
+                    else {
+#pragma unroll
+                      for (int e = 0; e < V; ++e) av[ru][u].v[e] = ld_el_if<T>(ap + e, lc + e < nc);
+                    }
+                  }
+#pragma unroll
+                for (int ru = 0; ru < RU; ++ru) xv[ru] = __ldg(xp + ru * xstride);
+                at += astep;
+                xp += xstep;
+                T racc[RU];
+#pragma unroll
+                for (int ru = 0; ru < RU; ++ru) {
+                  racc[ru] = T(0);
+#pragma unroll
+                  for (int u = 0; u < CU; ++u)
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                      if (K::ROWOUT) racc[ru] = av[ru][u].v[e] * xcv[0][u][e] + racc[ru];
+                      colacc[0][u][e] = av[ru][u].v[e] * xv[ru] + colacc[0][u][e];
+                    }
+                }
+                if (K::ROWOUT) {
+                  const T sum = multi_group_sum<LPR, RU>(racc, lane);
+                  if (q % LPV == 0) *rp = sum;
+                  rp += RB;
+                }
+              }
+            };
+            if (nc % V == 0) cut_steps(std::true_type());
+            else cut_steps(std::false_type());
+            rb = fast_hi - RB;
+            continue;
+          }
         }
 #pragma unroll 1
         for (int st = 0; st < nst; ++st) {

@@ -318,6 +318,37 @@ def test_cluster_gather_kernel(b2, ctx, dtype, mode):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n,pad", [(63, 1), (130, 2), (513, 3), (516, 0), (641, 7), (1090, 2), (1151, 1), (1153, 0)])
+def test_upper_triangle_cut_last_column_tile(b2, ctx, dtype, n, pad):
+    """The tile kernels' column sums where the last column tile of an upper triangle (64 or 128 columns, the longest
+    of them) is cut by the matrix edge: on a pack boundary, inside a pack, with one column and with all but one, in
+    blocks of 512 rows that lie above the diagonal whole, in part and not at all; rows on and off 16-byte boundaries."""
+    old = b2.get_tuning(b2.KNOB_GATHER), b2.get_tuning(b2.KNOB_TRI_TILE)
+    b2.set_tuning(b2.KNOB_GATHER, 0)
+    b2.set_tuning(b2.KNOB_TRI_TILE, 0)
+    try:
+        for lda, diag, inc in ((n + pad, orc.NON_UNIT, 1), ((n + 7) // 4 * 4, orc.UNIT, 2)):
+            x, y = synth.vector_np(7, n, n, dtype), synth.vector_np(8, n, n, dtype)
+            a = tri_buf(12, n, lda, dtype, orc.ROW_MAJOR, orc.UPPER, diag)
+            ga, gx = Guarded(a), Guarded(place(x, inc))
+            b2.trmv(ctx, orc.ROW_MAJOR, orc.UPPER, orc.TRANS, diag, n, ga.t, lda, gx.t, inc)
+            ox = place(x, inc)
+            absterms = orc.trmv(orc.ROW_MAJOR, orc.UPPER, orc.TRANS, diag, n, a, lda, ox, inc)
+            assert_close(pick(gx.host(), n, inc), pick(ox, n, inc), absterms, dtype, f"trmv lda={lda}")
+            gx.check_guards()
+            a = tri_buf(9, n, lda, dtype, orc.ROW_MAJOR, orc.UPPER, orc.NON_UNIT)
+            ga, gx, gy = Guarded(a), Guarded(place(x, inc)), Guarded(y)
+            b2.symv(ctx, orc.ROW_MAJOR, orc.UPPER, n, 1.25, ga.t, lda, gx.t, inc, 0.5, gy.t, 1)
+            oy = y.copy()
+            absterms = orc.symv(orc.ROW_MAJOR, orc.UPPER, n, dtype(1.25), a, lda, place(x, inc), inc, dtype(0.5), oy, 1)
+            assert_close(gy.host(), oy, absterms, dtype, f"symv lda={lda}")
+            gy.check_guards()
+    finally:
+        b2.set_tuning(b2.KNOB_GATHER, old[0])
+        b2.set_tuning(b2.KNOB_TRI_TILE, old[1])
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("streams", [-1, 1, 0])
 def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
     """The cluster kernel at its edges: one unknown more and less than a block row, than the rows the solving
