@@ -12,7 +12,12 @@ namespace b2 {
 template <typename T, int V, class S>
 constexpr int kGerBlocks = V > 1 ? 2 : sizeof(T) == 8 && S::CU == 1 ? 4 : 0;
 
-template <typename T, int V, class S>
+// CUT: the kernel knows rows that end inside a pack.  Short row segments (CU == 1) leave that to a kernel of its own: with
+// the loads of cut packs in it the one for whole packs needs 141 registers instead of 92 in double, and bounded to 128 it
+// lost 2 % (200 x 90000 by columns: 51.2 us without them, 52.4 with, 50.5 so).  Long ones have it all in one: the kernel for whole
+// packs takes fewer registers than two resident blocks leave it, and a third one costs 2-5 % (4096 x 4096 in float
+// 23.1 -> 23.6 us, 6000 x 3000 25.3 -> 26.7).
+template <typename T, int V, class S, bool CUT>
 __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* __restrict__ a, int64_t lda, int64_t rows, int64_t cols,
                                                        const T* __restrict__ xr, int64_t incxr,
                                                        const T* __restrict__ yc, int64_t incyc, T alpha,
@@ -62,7 +67,7 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
           for (int e = 0; e < V; ++e) av[ru][u].v[e] = xv[ru] * yv[u][e] + av[ru][u].v[e];
           st_cs<T, V>(a + rowi[ru] * lda + c0 + (u * LPR + q) * V, av[ru][u]);
         }
-    } else if (V > 1 && (c0 + TC <= cols || (cols - c0) % V == 0)) {
+    } else if (V > 1 && (!CUT || c0 + TC <= cols || (cols - c0) % V == 0)) {
       // only the matrix edge cuts this tile, on pack boundaries (narrow matrices, short row
       // bands): the loads still go out together, each under its own row / pack predicate.
       // (Element-wise tiles, V == 1, stay on the plain path below: single-element streaming
@@ -72,8 +77,12 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
 #pragma unroll
-        for (int u = 0; u < CU; ++u)
-          if (rowi[ru] < r_end && u * LPR + q < npk) av[ru][u] = ld_cs<T, V>(a + rowi[ru] * lda + c0 + (u * LPR + q) * V);
+        for (int u = 0; u < CU; ++u) {
+          const T* ap = a + rowi[ru] * lda + c0 + (u * LPR + q) * V;
+          const bool in = rowi[ru] < r_end && u * LPR + q < npk;
+          if constexpr (CU == 1) av[ru][u] = ld_cg_if<T, V>(ap, in);
+          else if (in) av[ru][u] = ld_cs<T, V>(ap);  // (as one predicated instruction: the registers again)
+        }
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
 #pragma unroll
@@ -83,7 +92,7 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
             for (int e = 0; e < V; ++e) av[ru][u].v[e] = xv[ru] * yv[u][e] + av[ru][u].v[e];
             st_cs<T, V>(a + rowi[ru] * lda + c0 + (u * LPR + q) * V, av[ru][u]);
           }
-    } else {
+    } else if constexpr (V == 1 || CUT) {
       // rows that end inside a pack, element-wise tiles: the loads go out together all the same.  (Plain stores here:
       // single-element streaming stores to rows that start off a sector boundary measured twice as slow.)
       P av[RU][CU];
@@ -190,8 +199,11 @@ static int ger_launch(const Launch& l, T* a, int64_t lda, int64_t rows, int64_t 
   const int64_t rows_per_cta = (int64_t)S::RB * knob(kKnobGerRows);
   const int64_t nrs = (rows + rows_per_cta - 1) / rows_per_cta;
   if (nrs * nct > 0x7fffffff) return B2_STATUS_NOT_IMPLEMENTED;
-  launch_chained(ger_kernel<T, V, S>, dim3((unsigned)(nrs * nct)), dim3(kThreads), 0, l.stream, a, lda, rows, cols, xr, incxr, yc, incyc, alpha,
-                                                                        rows_per_cta, nct);
+  auto kern = ger_kernel<T, V, S, (V > 1)>;
+  if constexpr (V > 1 && S::CU == 1)
+    if (cols % V == 0) kern = ger_kernel<T, V, S, false>;
+  launch_chained(kern, dim3((unsigned)(nrs * nct)), dim3(kThreads), 0, l.stream, a, lda, rows, cols, xr, incxr, yc, incyc, alpha,
+                 rows_per_cta, nct);
   return check_launch();
 }
 

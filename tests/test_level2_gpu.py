@@ -272,6 +272,26 @@ def test_ger_unpadded_odd_widths(b2, ctx, dtype, m, n):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n", [5, 16, 31, 33, 36, 63, 66, 127, 131, 252, 255, 509, 515, 1030])
+def test_ger_padded_rows(b2, ctx, dtype, n):
+    """Rows on 16-byte boundaries that end inside a pack or behind one, in every row segment length of the kernel (8, 16, 32
+    and 128 packs): the last tile cut by both edges, by one, by none; the padding keeps its NaN."""
+    lda = (n + 4) // 4 * 4
+    for m in (1, 129, 300):
+        a = synth.matrix_np(3, m, m, n, lda, dtype)
+        a[:, n:] = np.nan
+        x, y = synth.vector_np(5, m, m, dtype), synth.vector_np(6, n, n, dtype)
+        ga, gx, gy = Guarded(a.ravel()), Guarded(x), Guarded(place(y, -2))
+        b2.ger(ctx, orc.ROW_MAJOR, m, n, 0.75, gx.t, 1, gy.t, -2, ga.t, lda)
+        oa = a.ravel().copy()
+        absterms = orc.ger(orc.ROW_MAJOR, m, n, dtype(0.75), x, 1, place(y, -2), -2, oa, lda)
+        got = ga.host().reshape(m, lda)
+        assert_close(got[:, :n], oa.reshape(m, lda)[:, :n], absterms, dtype, f"ger m={m}")
+        assert np.isnan(got[:, n:]).all()
+        ga.check_guards()
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("mode", [0, 2, 3])
 def test_cluster_gather_kernel(b2, ctx, dtype, mode):
     """The one-launch kernel at its edges: one output more and less than a cluster owns, one element more and less
