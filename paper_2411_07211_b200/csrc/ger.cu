@@ -27,6 +27,15 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
   constexpr int LPR = S::LPR, CU = S::CU, RU = S::RU, G = S::G, RB = S::RB;
   constexpr int TC = LPR * V * CU;
   using P = Pack<T, V>;
+  // Packs, and single elements of which a warp takes 128 in a row: the sectors are written whole, or nearly so, and the
+  // matrix passes through L2 evict-first, loads and stores.  Elements of short rows leave partly written sectors: loaded
+  // evict-first they were gone from L2 when the stores came, and had to be filled again (1000000 x 16, lda 19, in
+  // double 80 us, 48 so); those of cut tiles are stored plainly (streaming, 100003 x 64 in float 9.9 -> 10.2 us).  Long
+  // rows off 16-byte boundaries, float, with plain L2 loads -> evict-first -> streaming stores of cut tiles too: 16000 x
+  // 8000 178.2 -> 170.5 -> 167.9 us, 5001 x 5000 37.2 -> 36.2 -> 36.2, 100000 x 300 45.8 -> 44.6 -> 42.7; double 309 ->
+  // 308 -> 305, 62.1 -> 62.0 -> 62.1, 77.2 -> 77.6 -> 73.5; streaming stores of whole tiles against plain ones
+  // 37.2 / 37.7 (5001 x 5000, float), 26.8 / 27.4 (509117 x 32), 94.1 / 87.0 (500000 x 100).
+  constexpr bool EVICT = V > 1 || CU > 1;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane / LPR, q = lane % LPR;
   const int ct = blockIdx.x % nct;
@@ -54,10 +63,9 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
 #pragma unroll
-        for (int u = 0; u < CU; ++u) {  // (single elements leave partly written sectors: evict-first ones were gone from
-          // L2 when the stores came, and had to be filled again; 1000000 x 16, lda 19, in double 80 us, 48 so)
+        for (int u = 0; u < CU; ++u) {
           const T* ap = a + rowi[ru] * lda + c0 + (u * LPR + q) * V;
-          av[ru][u] = V > 1 ? ld_cs<T, V>(ap) : ld_cg<T, V>(ap);
+          av[ru][u] = EVICT ? ld_cs<T, V>(ap) : ld_cg<T, V>(ap);
         }
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
@@ -70,8 +78,6 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
     } else if (V > 1 && (!CUT || c0 + TC <= cols || (cols - c0) % V == 0)) {
       // only the matrix edge cuts this tile, on pack boundaries (narrow matrices, short row
       // bands): the loads still go out together, each under its own row / pack predicate.
-      // (Element-wise tiles, V == 1, stay on the plain path below: single-element streaming
-      // stores to rows that start off a sector boundary measured twice as slow.)
       const int64_t npk = (min(cols, c0 + TC) - c0) / V;  // packs of this tile that exist
       P av[RU][CU];
 #pragma unroll
@@ -93,8 +99,7 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
             st_cs<T, V>(a + rowi[ru] * lda + c0 + (u * LPR + q) * V, av[ru][u]);
           }
     } else if constexpr (V == 1 || CUT) {
-      // rows that end inside a pack, element-wise tiles: the loads go out together all the same.  (Plain stores here:
-      // single-element streaming stores to rows that start off a sector boundary measured twice as slow.)
+      // rows that end inside a pack, element-wise tiles: the loads go out together all the same
       P av[RU][CU];
 #pragma unroll
       for (int ru = 0; ru < RU; ++ru)
@@ -122,7 +127,10 @@ __global__ void __launch_bounds__(kThreads, kGerBlocks<T, V, S>) ger_kernel(T* _
           } else {
 #pragma unroll
             for (int e = 0; e < V; ++e)
-              if (cv + e < cols) B2_STORE(ap + e, av[ru][u].v[e]);
+              if (cv + e < cols) {
+                if constexpr (V == 1 && EVICT) st_cs<T, 1>(ap, av[ru][u]);
+                else B2_STORE(ap + e, av[ru][u].v[e]);
+              }
           }
         }
     }

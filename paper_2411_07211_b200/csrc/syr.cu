@@ -176,6 +176,9 @@ __global__ void __launch_bounds__(kThreads, (syr_blocks<T, V, TWO>())) syr_kerne
         if (TWO) av[ru][u].v[e] = yi * xj[u][e] + (xi * yj[u][e] + av[ru][u].v[e]);
         else av[ru][u].v[e] = xi * xj[u][e] + av[ru][u].v[e];
       }
+      // (Single elements of a matrix off 16-byte boundaries are stored streaming here and above, those of cut packs
+      // plainly.  Plain stores throughout: better while the matrix lies in L2 -- syr2 in float, n = 5001, 24.0 -> 21.5 us,
+      // syr in double, n = 3001, 11.5 -> 9.9 -- and worse beyond: syr in float, n = 8001, 43.9 -> 47.3, 12001 93 -> 103.)
       if (jr >= lo[ru] && jr + V <= hi[ru]) {
         st_cs<T, V>(ap[ru] + u * 32 * V, av[ru][u]);
       } else if (V > 1) {
