@@ -59,7 +59,8 @@ enum {
  *                   first call (b2_workspace_reset does that); every call that completes
  *                   leaves it zero again.  The rest holds per-call partial results.
  *   workspace_bytes size of that memory.  Larger workspaces allow finer work splitting for
- *                   level-2 calls; b2_workspace_bytes() is a comfortable default.
+ *                   level-2 calls, and smaller ones than b2_workspace_query's send some of
+ *                   them to slower kernels; b2_workspace_bytes() is a comfortable default.
  *   device_status   optional device int.  trsv writes B2_STATUS_TIMEOUT there if a bounded
  *                   wait on another thread block ran out (the call's output is then invalid).
  *                   Never written otherwise; the caller zeroes it.  A timed-out call leaves
@@ -83,10 +84,15 @@ size_t b2_workspace_min_bytes(void); /* control block + level-1 partials        
  * 32768 x 32768 and vectors of any length without B2_STATUS_WORKSPACE_TOO_SMALL; the exact
  * need of one call is b2_workspace_query's. */
 size_t b2_workspace_bytes(void);
-/* Smallest workspace size with which no routine of this library returns
- * B2_STATUS_WORKSPACE_TOO_SMALL on an m x n matrix (vectors of max(m, n) elements; level-1
- * calls: pass m = n = 1) of elem_bytes-sized elements (4 or 8).  Larger workspaces only allow
- * finer work splitting.  Returns 0 for a negative size or another element size. */
+/* Workspace size with which every routine of this library runs an m x n matrix (vectors of
+ * max(m, n) elements; triangular and symmetric ones of order min(m, n); level-1 calls: pass
+ * m = n = 1) of elem_bytes-sized elements (4 or 8) on the kernel meant for it, and with which
+ * none returns B2_STATUS_WORKSPACE_TOO_SMALL.  Larger workspaces only allow finer work
+ * splitting.  A smaller one costs: trsv without room for the inverses of its diagonal blocks
+ * (about 512 bytes per unknown) falls back to kernels that take 1.3 to 2 times as long; symv and
+ * the column sums of narrow matrices fall back likewise, and below what is left then a call
+ * returns B2_STATUS_WORKSPACE_TOO_SMALL.  Returns 0 for a negative size or another element
+ * size. */
 size_t b2_workspace_query(int64_t m, int64_t n, size_t elem_bytes);
 int b2_workspace_reset(const b2_ctx* ctx); /* async memset of the control block to zero     */
 const char* b2_status_string(int status);

@@ -1,5 +1,9 @@
 // Library-wide pieces: workspace helpers, status strings, tuning knobs, device queries.
+#include <algorithm>
+#include <iterator>
+
 #include "common.cuh"
+#include "trsv_front.cuh"
 
 namespace b2 {
 
@@ -59,18 +63,25 @@ size_t b2_workspace_bytes(void) { return (size_t)256 << 20; }
 
 size_t b2_workspace_query(int64_t m, int64_t n, size_t elem_bytes) {
   if (m < 0 || n < 0 || (elem_bytes != 4 && elem_bytes != 8)) return 0;
-  // level 1: one partial per block of the reduction grid; level 2 with every split merged: one
-  // row of partials per output vector; symv, whose blocks produce row sums and column sums at
-  // once: one row of partials per column tile of 32 packs; trsv: one or two
-  // tagged 64-bit words per unknown
+  const size_t e = elem_bytes, V = 16 / e, seg = 32 * V;  // elements of a pack; columns of a 32-pack tile
   const size_t vec = (size_t)(m > n ? m : n), sq = (size_t)(m < n ? m : n);
-  const size_t tile_cols = 32 * (16 / elem_bytes);
-  const size_t level2 = ((size_t)m + (size_t)n) * elem_bytes + 1024;
-  const size_t symv = ((sq + tile_cols - 1) / tile_cols + 1) * sq * elem_bytes + 1024;
-  const size_t trsv = vec * 8 * (elem_bytes / 4);
-  size_t need = level2 > trsv ? level2 : trsv;
-  if (symv > need) need = symv;
-  return b2_workspace_min_bytes() + need;
+  auto tiles = [](size_t len, size_t of) { return (len + of - 1) / of; };
+  // column sums that a tile of shifted packs leaves to its neighbour (level2.cuh, SHIFT)
+  auto spill = [&](size_t cols) { return tiles(cols + V - 1, seg) * (V - 1) * e; };
+  const size_t parts[] = {
+      // level 2 with every split merged: one row of partials per output vector
+      ((size_t)m + (size_t)n) * e + spill(vec) + 1024,
+      // narrow matrices (from 2048 rows on), column sums: one partial row per block of a resident grid
+      sq <= 64 * V && vec >= 2048 ? (size_t)b2::sm_count() * 4 * sq * e : 0,
+      // symv, whose blocks produce row sums and column sums at once: one row of partials per column tile of 32 packs ...
+      (tiles(sq + V - 1, seg) + 1) * sq * e + spill(sq) + 1024,
+      // ... and, while it runs on the ring kernel, one per tile of a block row and one per block row
+      (double)sq * (double)sq * e / 2 <= b2::kSymvRingBytes ? (tiles(sq, seg) + tiles(sq, 128)) * sq * e + 512 : 0,
+      // trsv: tagged words and inverses of the cluster kernel; one or two words per unknown for the kernels behind it
+      b2::trsv_cluster_scratch((int64_t)sq, e),
+      vec * 8 * (e / 4),
+  };
+  return b2_workspace_min_bytes() + *std::max_element(std::begin(parts), std::end(parts));
 }
 
 int b2_workspace_reset(const b2_ctx* ctx) {

@@ -407,6 +407,9 @@ static void dbg_commit(Launch& l) {
 #define B2_DBG_COMMIT(l) ((void)0)
 #endif
 
+// Triangles (bytes) up to which symv runs on the tile kernel with the shared-memory ring (tri_impl.cuh).
+constexpr double kSymvRingBytes = 64.0 * 1024 * 1024;
+
 // Number of SMs of the current device (cached per device id).
 int sm_count();
 

@@ -75,7 +75,7 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
   // (double, upper triangle: that kind of the general kernel spills 132 bytes per thread at its
   // 64 registers and streams 10-15 % slower than the ring kernel at every size -- n = 32768:
   // 780 us against 684 us)
-  const bool small = (double)n * (double)n * sizeof(T) / 2 <= 64.0 * 1024 * 1024;
+  const bool small = (double)n * (double)n * sizeof(T) / 2 <= kSymvRingBytes;
   if (knob(kKnobTriTile) == 2 || (knob(kKnobTriTile) == 1 && (small || (sizeof(T) == 8 && upper)))) {
     bool handled = false;
     const int st = upper ? tt::tri_tile_run<T, true, true, TRI_UPPER, false, true>(l, a, lda, n, args.xc, incx, alpha, beta,

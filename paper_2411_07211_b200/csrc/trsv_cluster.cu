@@ -61,7 +61,7 @@ struct Args {
   int64_t incx;
   u64* xbuf;         // [K * NB] published x
   u64* far;          // [K * NB] published row sums of the tiles left of the near window
-  T* winv;           // [K][NB * NB] inverses of the diagonal blocks (of their transposes: Diag)
+  T* winv;           // [K - kCS][NB * NB] inverses of the diagonal blocks beyond the first kCS (of their transposes: Diag)
   unsigned* flags;   // [K] call tag once winv[k] is complete
   unsigned* ctl;
   int K;             // block rows
@@ -305,7 +305,7 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
     if (b.tid < kInvT) invert_small<T>(M, b.red, p.unit, block_len(p, I), b.tid);
     bar_block();
     invert_last<T>(M, b.red, b.tid);
-    T* dst = p.winv + (int64_t)k * NB * NB;
+    T* dst = p.winv + (int64_t)(k - kCS) * NB * NB;
 #pragma unroll 2
     for (int idx = b.tid; idx < NB * NB / V; idx += kCT) {
       T v[V];
@@ -674,7 +674,7 @@ __device__ __forceinline__ void solve_block(const Args<T>& p, Block<T>& b, int r
     bar_block();
     const bool self = s_self != 0;
     load_next(k);
-    const T* src = p.winv + (int64_t)k * NB * NB;
+    const T* src = p.winv + (int64_t)max(k - kCS, 0) * NB * NB;
     int pitch = NB;
     bool dry = false;
     if (self) {
@@ -822,19 +822,36 @@ static int launch_cluster(const Launch& l, Args<T>& p, bool* handled) {
   return check_launch();
 }
 
+// Workspace of a solve of K block rows: published x and far sums, inverses, their flags.
+template <typename T>
+struct Scratch {
+  size_t words, inverses, total;
+  explicit Scratch(int64_t K) {
+    constexpr size_t NB = Geo<T>::NB;
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    words = up((size_t)K * NB * Words<T>::N * 8);
+    inverses = up((size_t)std::max<int64_t>(0, K - kCS) * NB * NB * sizeof(T));
+    total = 2 * words + inverses + up((size_t)K * 4);
+  }
+};
+
 }  // namespace tc
+
+size_t trsv_cluster_scratch(int64_t n, size_t elem_bytes) {
+  if (elem_bytes == 4) return tc::Scratch<float>((n + tc::Geo<float>::NB - 1) / tc::Geo<float>::NB).total;
+  return tc::Scratch<double>((n + tc::Geo<double>::NB - 1) / tc::Geo<double>::NB).total;
+}
 
 template <typename T>
 int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, int64_t n, const T* a, int64_t lda, T* xbase, int64_t incx,
                      unsigned tag, bool* handled) {
   using namespace tc;
-  constexpr int NB = Geo<T>::NB, WPE = Words<T>::N;
+  constexpr int NB = Geo<T>::NB;
   *handled = false;
   const int64_t K = (n + NB - 1) / NB;
   if (K > (1 << 20)) return B2_STATUS_OK;
-  auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-  const size_t words = up((size_t)K * NB * WPE * 8), inverses = up((size_t)K * NB * NB * sizeof(T)), flags = up((size_t)K * 4);
-  if (2 * words + inverses + flags > l.scratch_bytes) return B2_STATUS_OK;
+  const Scratch<T> w(K);
+  if (w.total > l.scratch_bytes) return B2_STATUS_OK;
   Args<T> p = {};
   p.a = a;
   p.lda = lda;
@@ -842,9 +859,9 @@ int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, in
   p.x = xbase;
   p.incx = incx;
   p.xbuf = reinterpret_cast<u64*>(l.scratch);
-  p.far = reinterpret_cast<u64*>(l.scratch + words);
-  p.winv = reinterpret_cast<T*>(l.scratch + 2 * words);
-  p.flags = reinterpret_cast<unsigned*>(l.scratch + 2 * words + inverses);
+  p.far = reinterpret_cast<u64*>(l.scratch + w.words);
+  p.winv = reinterpret_cast<T*>(l.scratch + 2 * w.words);
+  p.flags = reinterpret_cast<unsigned*>(l.scratch + 2 * w.words + w.inverses);
   p.ctl = l.ctl;
   p.K = (int)K;
   p.backward = backward;

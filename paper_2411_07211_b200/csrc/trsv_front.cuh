@@ -16,5 +16,6 @@ int trsv_front_try(const Launch& l, bool coltype, bool backward, bool unit, int6
 template <typename T>
 int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, int64_t n, const T* a, int64_t lda,
                      T* xbase, int64_t incx, unsigned tag, bool* handled);
+size_t trsv_cluster_scratch(int64_t n, size_t elem_bytes);  // bytes of workspace (past the control block) it needs
 
 }  // namespace b2

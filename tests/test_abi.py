@@ -35,6 +35,22 @@ def test_header_symbols_exported(b2):
     assert b"argument" in b2.lib().b2_status_string(-3)
 
 
+@pytest.mark.parametrize("size", [4, 8])
+@pytest.mark.parametrize("n", [1, 100, 1024, 2047, 4100, 8191, 8192, 16384, 20000])
+def test_workspace_query_covers_every_kernel(b2, n, size):
+    """What the kernels reserve past the 4 KiB control block: trsv the tagged words of x and of the row sums, the inverses
+    of all diagonal blocks but the first 16 and a flag per block; symv row partials per column tile, column partials
+    and, off 16-byte boundaries, V - 1 more columns per tile."""
+    have = b2.lib().b2_workspace_query(n, n, size) - 4096
+    nb, v = (128, 4) if size == 4 else (64, 2)
+    k = -(-n // nb)
+    assert have >= 2 * k * nb * 2 * size + max(0, k - 16) * nb * nb * size + 4 * k
+    tiles = -(-(n + v - 1) // (32 * v))
+    assert have >= tiles * n * size + n * size + tiles * (v - 1) * size
+    if n * n * size <= 128 << 20:
+        assert have >= (-(-n // (32 * v)) + -(-n // 128)) * n * size  # the ring kernel's
+
+
 def test_argument_validation_without_gpu(b2):
     """Invalid arguments are rejected on the host before any CUDA call."""
     h = b2.lib()

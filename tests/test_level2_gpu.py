@@ -446,6 +446,39 @@ def test_level2_determinism(b2, ctx, dtype):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+def test_workspace_query_keeps_the_kernels(b2, ctx, dtype):
+    """With exactly b2_workspace_query bytes trsv and symv run on the kernels they run on with the default workspace:
+    equal bits, which the kernels behind them do not give (their sums run in another order)."""
+    s = np.dtype(dtype).itemsize
+
+    def solve(c, n):
+        gx = Guarded(synth.vector_np(9, n, n, dtype))
+        b2.trsv(c, orc.ROW_MAJOR, orc.LOWER, orc.NO_TRANS, orc.NON_UNIT, n, tri.t, n, gx.t, 1)
+        assert c.device_status() == 0
+        return gx.host()
+
+    def product(c, n):
+        gx, gy = Guarded(synth.vector_np(9, n, n, dtype)), Guarded(np.zeros(n, dtype=dtype))
+        b2.symv(c, orc.ROW_MAJOR, orc.UPPER, n, 1.25, sym.t, n, gx.t, 1, 0.0, gy.t, 1)
+        return gy.host()
+
+    for n in (300, 2100, 2432):
+        tri = Guarded(tri_buf(21, n, n, dtype, orc.ROW_MAJOR, orc.LOWER, orc.NON_UNIT))
+        sym = Guarded(tri_buf(9, n, n, dtype, orc.ROW_MAJOR, orc.UPPER, orc.NON_UNIT))
+        small = b2.Context(workspace_bytes=b2.lib().b2_workspace_query(n, n, s))
+        small.reset()
+        for routine, knob, other in ((solve, b2.KNOB_TRSV_FRONT, 2), (product, b2.KNOB_TRI_TILE, 0)):
+            want = routine(ctx, n)
+            assert np.array_equal(routine(small, n), want), (n, routine.__name__)
+            old = b2.get_tuning(knob)
+            b2.set_tuning(knob, other)
+            try:
+                assert not np.array_equal(routine(ctx, n), want), (n, routine.__name__)
+            finally:
+                b2.set_tuning(knob, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 def test_workspace_query_is_enough(b2, dtype):
     """A workspace of exactly b2_workspace_query(m, n, s) bytes serves every level-2 routine on an
     m x n problem (the recommended default is only a default): a matrix of a few very long rows,
