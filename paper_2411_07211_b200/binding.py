@@ -18,9 +18,10 @@ import os
 import torch
 
 try:
-    from . import _binding as _native  # (built with the library; its absence is reported at the first call)
-except ImportError:
-    _native = None
+    from . import _binding as _native  # (built with the library; what keeps it from loading is reported at the first call)
+    _native_error = None
+except ImportError as e:
+    _native, _native_error = None, e
 
 ROW_MAJOR, COL_MAJOR = 101, 102
 NO_TRANS, TRANS = 111, 112
@@ -166,11 +167,18 @@ def _p(t):
     return t.data_ptr()
 
 
+def _need_native():
+    """The compiled module, or an ImportError that says why there is none."""
+    if _native is None:
+        lib()
+        raise ImportError(f"the compiled module paper_2411_07211_b200._binding does not load ({_native_error}): build it "
+                          "with `python -m paper_2411_07211_b200.build`") from _native_error
+    return _native
+
+
 def _missing(name):
     def call(*args, **kwargs):
-        lib()
-        raise ImportError("the compiled module paper_2411_07211_b200._binding is missing: build it with "
-                          "`python -m paper_2411_07211_b200.build`")
+        _need_native()
     call.__name__ = name
     return call
 
@@ -186,7 +194,7 @@ def prepare(thunk):
     going through the interpreter for each of them.  For timing loops over small problems; the
     returned callable returns the last status.  What is recorded are the calls that the thunk makes
     on the thread that runs it; any number of threads may be inside prepare()."""
-    return _native.record(thunk)
+    return _need_native().record(thunk)
 
 
 # Every routine ends with `check=True`: raise B2Error on a non-zero status instead of returning it.
@@ -210,7 +218,7 @@ def rotm(ctx, n, x, incx, y, incy, param, check=True):
         return _routines["rotm"](ctx, n, x, incx, y, incy, None, check)
     ctype = ctypes.c_float if x.dtype == torch.float32 else ctypes.c_double
     host = (ctype * 5)(*[float(v) for v in param])
-    _native.keep(host)
+    _need_native().keep(host)
     return _routines["rotm"](ctx, n, x, incx, y, incy, ctypes.addressof(host), check)
 
 

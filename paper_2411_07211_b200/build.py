@@ -4,6 +4,7 @@ Python module _binding.so that calls it."""
 from __future__ import annotations
 
 import hashlib
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -18,6 +19,7 @@ OBJ_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(PKG, "libb2blas.so")
 DEBUG_LIB_PATH = os.path.join(PKG, "libb2blas_dbg.so")  # the bounds-checking build (-DB2_DEBUG_BOUNDS)
 
+BINDING_SOURCE = "binding_native.cpp"
 BINDING_PATH = os.path.join(PKG, "_binding.so")  # Python entry points (torch and CPython headers, no CUDA code)
 
 SOURCES = ["api_common.cu", "level1.cu", "gemv.cu", "ger.cu", "tri_f32.cu", "tri_f64.cu", "trsv.cu", "trsv_front.cu", "trsv_cluster.cu", "syr.cu"]
@@ -33,14 +35,29 @@ def _nvcc() -> str:
 
 
 def _digest() -> str:
+    """Of what the library is made of."""
     h = hashlib.sha256(" ".join(NVCC_FLAGS).encode())
     files = sorted(os.listdir(CSRC)) + [os.path.join(INCLUDE, "b2blas.h")]
     for name in files:
         path = name if os.path.isabs(name) else os.path.join(CSRC, name)
-        if os.path.isfile(path):
+        if os.path.isfile(path) and name != BINDING_SOURCE:
             h.update(name.encode())
             h.update(open(path, "rb").read())
     return h.hexdigest()
+
+
+def _binding_digest() -> str:
+    """Of what the Python module is made of; it fits one interpreter and one build of torch."""
+    h = hashlib.sha256()
+    for part in (sys.version, sysconfig.get_config_var("EXT_SUFFIX"), importlib.metadata.version("torch"), os.environ.get("CXX", "g++")):
+        h.update(repr(part).encode())
+    for path in (os.path.join(CSRC, BINDING_SOURCE), os.path.join(INCLUDE, "b2blas.h")):
+        h.update(open(path, "rb").read())
+    return h.hexdigest()
+
+
+def _is_built(path: str, stamp: str, digest: str) -> bool:
+    return os.path.exists(path) and os.path.exists(stamp) and open(stamp).read() == digest
 
 
 def _compile_binding() -> None:
@@ -50,7 +67,7 @@ def _compile_binding() -> None:
                         os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")] for a in ("-I", d)]
     tmp = BINDING_PATH + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", *incs,
-           os.path.join(CSRC, "binding_native.cpp"), "-o", tmp, *[a for d in library_paths() for a in ("-L", d)],
+           os.path.join(CSRC, BINDING_SOURCE), "-o", tmp, *[a for d in library_paths() for a in ("-L", d)],
            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-ldl"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
@@ -60,17 +77,21 @@ def _compile_binding() -> None:
 
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
     """Compile every .cu under csrc/, link libb2blas.so and build the Python module; a no-op when
-    sources are unchanged.  debug_bounds=True builds the bounds-checking variant (libb2blas_dbg.so)
-    of the library instead."""
+    sources are unchanged (and, for the module, the interpreter and torch).  debug_bounds=True
+    builds the bounds-checking variant (libb2blas_dbg.so) of the library instead."""
     lib_path = DEBUG_LIB_PATH if debug_bounds else LIB_PATH
     obj_dir = os.path.join(OBJ_DIR, "dbg") if debug_bounds else OBJ_DIR
-    extra = ["-DB2_DEBUG_BOUNDS"] if debug_bounds else []
-    stamp = os.path.join(obj_dir, "stamp.txt")
-    digest = _digest()
-    have = os.path.exists(lib_path) and (debug_bounds or os.path.exists(BINDING_PATH))
-    if not force and have and os.path.exists(stamp) and open(stamp).read() == digest:
-        return lib_path
     os.makedirs(obj_dir, exist_ok=True)
+    if not debug_bounds:
+        stamp, digest = os.path.join(obj_dir, "binding_stamp.txt"), _binding_digest()
+        if force or not _is_built(BINDING_PATH, stamp, digest):
+            _compile_binding()
+            with open(stamp, "w") as f:
+                f.write(digest)
+    extra = ["-DB2_DEBUG_BOUNDS"] if debug_bounds else []
+    stamp, digest = os.path.join(obj_dir, "stamp.txt"), _digest()
+    if not force and _is_built(lib_path, stamp, digest):
+        return lib_path
     nvcc = _nvcc()
 
     def compile_one(src):
@@ -85,11 +106,8 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
             sys.stderr.write(res.stderr)
         return obj
 
-    with ThreadPoolExecutor(max_workers=min(8, len(SOURCES) + 1)) as pool:
-        binding = None if debug_bounds else pool.submit(_compile_binding)
+    with ThreadPoolExecutor(max_workers=min(8, len(SOURCES))) as pool:
         objs = list(pool.map(compile_one, SOURCES))
-        if binding is not None:
-            binding.result()
     tmp = lib_path + f".tmp{os.getpid()}"
     res = subprocess.run([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"],
                          capture_output=True, text=True)

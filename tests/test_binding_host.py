@@ -1,8 +1,12 @@
 """Host side of the Python binding: what needs no GPU."""
+import os
+import subprocess
 import sys
 import threading
 
 import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
@@ -74,3 +78,38 @@ def test_recordings_nest(b2):
     assert (sys.getrefcount(inner) - base[0], sys.getrefcount(outer) - base[1]) == (0, 1)
     del replay
     assert sys.getrefcount(outer) == base[1]
+
+
+def test_the_reason_why_the_module_does_not_load_is_told(b2):
+    """Importing the package works without the compiled module; the first call says what the import said."""
+    code = """
+import sys
+class Refuse:
+    def find_spec(self, name, path=None, target=None):
+        if name.endswith('._binding'):
+            raise ImportError('undefined symbol: _ZN3c10')
+sys.meta_path.insert(0, Refuse())
+from paper_2411_07211_b200 import binding as b2
+for call in (lambda: b2.axpy(None, 1, 1.0, None, 1, None, 1), lambda: b2.prepare(lambda: None)):
+    try:
+        call()
+    except ImportError as e:
+        assert 'undefined symbol: _ZN3c10' in str(e) and isinstance(e.__cause__, ImportError), e
+    else:
+        raise AssertionError('no error')
+print('told')
+"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and "told" in res.stdout, res.stdout + res.stderr
+
+
+def test_another_interpreter_or_torch_rebuilds_the_module(monkeypatch):
+    from paper_2411_07211_b200 import build
+    now, library = build._binding_digest(), build._digest()
+    with monkeypatch.context() as m:
+        m.setattr(build.importlib.metadata, "version", lambda name: "0.0")
+        assert build._binding_digest() != now
+    with monkeypatch.context() as m:
+        m.setattr(sys, "version", "4.0")
+        assert build._binding_digest() != now and build._digest() == library
+    assert build._binding_digest() == now
