@@ -13,6 +13,7 @@ CUDA library is missing the import of the symbols fails loudly.
 from __future__ import annotations
 
 import ctypes
+import inspect
 import os
 
 import torch
@@ -185,7 +186,18 @@ def _missing(name):
 
 _NAMES = ("axpy", "scal", "copy", "swap", "rot", "rotm", "dot", "dsdot", "sdsdot", "asum", "nrm2", "iamax",
           "gemv", "ger", "syr", "syr2", "symv", "trmv", "trsv")
-_routines = _native.routines(LIB_PATH, B2Error, lib) if _native else {name: _missing(name) for name in _NAMES}
+
+
+def _signature(params):
+    kind = inspect.Parameter.POSITIONAL_OR_KEYWORD
+    return inspect.Signature([inspect.Parameter(p, kind) for p in params.split()] + [inspect.Parameter("check", kind, default=True)])
+
+
+def _routine(name):
+    return _routines[name]
+
+
+_routines = _native.routines(LIB_PATH, B2Error, lib, _signature, _routine) if _native else {name: _missing(name) for name in _NAMES}
 
 
 def prepare(thunk):
@@ -197,19 +209,20 @@ def prepare(thunk):
     return _need_native().record(thunk)
 
 
-# Every routine ends with `check=True`: raise B2Error on a non-zero status instead of returning it.
+# help() of a routine tells its parameters.  Every one ends with `check=True`: raise B2Error on a non-zero status
+# instead of returning it.
 # ---- level 1 ----------------------------------------------------------------------------
-axpy = _routines["axpy"]      # (ctx, n, alpha, x, incx, y, incy, check=True)
-scal = _routines["scal"]      # (ctx, n, alpha, x, incx, check=True)
-copy = _routines["copy"]      # (ctx, n, x, incx, y, incy, check=True)
-swap = _routines["swap"]      # (ctx, n, x, incx, y, incy, check=True)
-rot = _routines["rot"]        # (ctx, n, x, incx, y, incy, c, s, check=True)
-dsdot = _routines["dsdot"]    # (ctx, n, x, incx, y, incy, result, check=True): float32 vectors, float64 device result
-sdsdot = _routines["sdsdot"]  # (ctx, n, sb, x, incx, y, incy, result, check=True)
-dot = _routines["dot"]        # (ctx, n, x, incx, y, incy, result, check=True)
-asum = _routines["asum"]      # (ctx, n, x, incx, result, check=True)
-nrm2 = _routines["nrm2"]      # (ctx, n, x, incx, result, check=True)
-iamax = _routines["iamax"]    # (ctx, n, x, incx, result, check=True)
+axpy = _routines["axpy"]
+scal = _routines["scal"]
+copy = _routines["copy"]
+swap = _routines["swap"]
+rot = _routines["rot"]
+dsdot = _routines["dsdot"]
+sdsdot = _routines["sdsdot"]
+dot = _routines["dot"]
+asum = _routines["asum"]
+nrm2 = _routines["nrm2"]
+iamax = _routines["iamax"]
 
 
 def rotm(ctx, n, x, incx, y, incy, param, check=True):
@@ -223,13 +236,13 @@ def rotm(ctx, n, x, incx, y, incy, param, check=True):
 
 
 # ---- level 2 ----------------------------------------------------------------------------
-gemv = _routines["gemv"]      # (ctx, order, trans, m, n, alpha, a, lda, x, incx, beta, y, incy, check=True)
-ger = _routines["ger"]        # (ctx, order, m, n, alpha, x, incx, y, incy, a, lda, check=True)
-syr = _routines["syr"]        # (ctx, order, uplo, n, alpha, x, incx, a, lda, check=True)
-syr2 = _routines["syr2"]      # (ctx, order, uplo, n, alpha, x, incx, y, incy, a, lda, check=True)
-symv = _routines["symv"]      # (ctx, order, uplo, n, alpha, a, lda, x, incx, beta, y, incy, check=True)
-trmv = _routines["trmv"]      # (ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True)
-trsv = _routines["trsv"]      # (ctx, order, uplo, trans, diag, n, a, lda, x, incx, check=True)
+gemv = _routines["gemv"]
+ger = _routines["ger"]
+syr = _routines["syr"]
+syr2 = _routines["syr2"]
+symv = _routines["symv"]
+trmv = _routines["trmv"]
+trsv = _routines["trsv"]
 
 
 def set_tuning(knob: int, value: int):

@@ -29,6 +29,8 @@ namespace {
 constexpr int kMaxParams = 16;
 PyObject* g_error_class = nullptr;   // B2Error
 PyObject* g_ensure_loaded = nullptr; // binding.lib: loads the library or raises
+PyObject* g_signature = nullptr;     // binding._signature: parameter names -> inspect.Signature
+PyObject* g_lookup = nullptr;        // binding._routine: name -> callable (how a routine is pickled)
 std::string g_lib_path;
 void* g_lib = nullptr;
 
@@ -175,31 +177,51 @@ struct RoutineDef {
   bool (*run[2])(void*, PyObject* const*, int*);
   int type_of;
   const char* params;  // space-separated
+  const char* doc;
 };
 #define B2_INVOKER(FN) +[](void* s, PyObject* const* a, int* st) { return invoke(static_cast<decltype(&FN)>(nullptr), s, a, st); }
 #define B2_PAIR(S, D) {#S, #D}, {B2_INVOKER(S), B2_INVOKER(D)}
 #define B2_ONE(S) {#S, nullptr}, {B2_INVOKER(S), nullptr}
 
 const RoutineDef kRoutines[] = {
-    {"axpy", B2_PAIR(b2_saxpy, b2_daxpy), 3, "ctx n alpha x incx y incy"},
-    {"scal", B2_PAIR(b2_sscal, b2_dscal), 3, "ctx n alpha x incx"},
-    {"copy", B2_PAIR(b2_scopy, b2_dcopy), 2, "ctx n x incx y incy"},
-    {"swap", B2_PAIR(b2_sswap, b2_dswap), 2, "ctx n x incx y incy"},
-    {"rot", B2_PAIR(b2_srot, b2_drot), 2, "ctx n x incx y incy c s"},
-    {"rotm", B2_PAIR(b2_srotm, b2_drotm), 2, "ctx n x incx y incy param"},
-    {"dot", B2_PAIR(b2_sdot, b2_ddot), 2, "ctx n x incx y incy result"},
-    {"dsdot", B2_ONE(b2_dsdot), -1, "ctx n x incx y incy result"},
-    {"sdsdot", B2_ONE(b2_sdsdot), -1, "ctx n sb x incx y incy result"},
-    {"asum", B2_PAIR(b2_sasum, b2_dasum), 2, "ctx n x incx result"},
-    {"nrm2", B2_PAIR(b2_snrm2, b2_dnrm2), 2, "ctx n x incx result"},
-    {"iamax", B2_PAIR(b2_isamax, b2_idamax), 2, "ctx n x incx result"},
-    {"gemv", B2_PAIR(b2_sgemv, b2_dgemv), 6, "ctx order trans m n alpha a lda x incx beta y incy"},
-    {"ger", B2_PAIR(b2_sger, b2_dger), 9, "ctx order m n alpha x incx y incy a lda"},
-    {"syr", B2_PAIR(b2_ssyr, b2_dsyr), 7, "ctx order uplo n alpha x incx a lda"},
-    {"syr2", B2_PAIR(b2_ssyr2, b2_dsyr2), 9, "ctx order uplo n alpha x incx y incy a lda"},
-    {"symv", B2_PAIR(b2_ssymv, b2_dsymv), 5, "ctx order uplo n alpha a lda x incx beta y incy"},
-    {"trmv", B2_PAIR(b2_strmv, b2_dtrmv), 6, "ctx order uplo trans diag n a lda x incx"},
-    {"trsv", B2_PAIR(b2_strsv, b2_dtrsv), 6, "ctx order uplo trans diag n a lda x incx"},
+    {"axpy", B2_PAIR(b2_saxpy, b2_daxpy), 3, "ctx n alpha x incx y incy",
+     "y <- alpha*x + y."},
+    {"scal", B2_PAIR(b2_sscal, b2_dscal), 3, "ctx n alpha x incx",
+     "x <- alpha*x."},
+    {"copy", B2_PAIR(b2_scopy, b2_dcopy), 2, "ctx n x incx y incy",
+     "y <- x."},
+    {"swap", B2_PAIR(b2_sswap, b2_dswap), 2, "ctx n x incx y incy",
+     "x <-> y."},
+    {"rot", B2_PAIR(b2_srot, b2_drot), 2, "ctx n x incx y incy c s",
+     "(x, y) <- (c*x + s*y, c*y - s*x)."},
+    {"rotm", B2_PAIR(b2_srotm, b2_drotm), 2, "ctx n x incx y incy param",
+     "Modified Givens rotation; param: the address of 5 host values."},
+    {"dot", B2_PAIR(b2_sdot, b2_ddot), 2, "ctx n x incx y incy result",
+     "result[0] <- sum of x*y."},
+    {"dsdot", B2_ONE(b2_dsdot), -1, "ctx n x incx y incy result",
+     "result[0] <- sum of x*y in double: float32 vectors, float64 device result."},
+    {"sdsdot", B2_ONE(b2_sdsdot), -1, "ctx n sb x incx y incy result",
+     "result[0] <- sb + sum of x*y, accumulated in double: float32 vectors and result."},
+    {"asum", B2_PAIR(b2_sasum, b2_dasum), 2, "ctx n x incx result",
+     "result[0] <- sum of |x|."},
+    {"nrm2", B2_PAIR(b2_snrm2, b2_dnrm2), 2, "ctx n x incx result",
+     "result[0] <- square root of the sum of x*x."},
+    {"iamax", B2_PAIR(b2_isamax, b2_idamax), 2, "ctx n x incx result",
+     "result[0] (int64) <- the first index, from 0, of the largest |x|."},
+    {"gemv", B2_PAIR(b2_sgemv, b2_dgemv), 6, "ctx order trans m n alpha a lda x incx beta y incy",
+     "y <- alpha*op(A)*x + beta*y, A m x n."},
+    {"ger", B2_PAIR(b2_sger, b2_dger), 9, "ctx order m n alpha x incx y incy a lda",
+     "A <- alpha*x*y^T + A, A m x n."},
+    {"syr", B2_PAIR(b2_ssyr, b2_dsyr), 7, "ctx order uplo n alpha x incx a lda",
+     "A <- alpha*x*x^T + A on the uplo triangle."},
+    {"syr2", B2_PAIR(b2_ssyr2, b2_dsyr2), 9, "ctx order uplo n alpha x incx y incy a lda",
+     "A <- alpha*(x*y^T + y*x^T) + A on the uplo triangle."},
+    {"symv", B2_PAIR(b2_ssymv, b2_dsymv), 5, "ctx order uplo n alpha a lda x incx beta y incy",
+     "y <- alpha*A*x + beta*y, A symmetric, its uplo triangle stored."},
+    {"trmv", B2_PAIR(b2_strmv, b2_dtrmv), 6, "ctx order uplo trans diag n a lda x incx",
+     "x <- op(A)*x, A triangular."},
+    {"trsv", B2_PAIR(b2_strsv, b2_dtrsv), 6, "ctx order uplo trans diag n a lda x incx",
+     "x <- the solution of op(A)*x = b, A triangular; b is passed in x."},
 };
 
 struct RoutineObject {
@@ -313,14 +335,30 @@ void routine_dealloc(PyObject* self) {
   tp->tp_free(self);
   Py_DECREF(tp);
 }
+// What a Python function has: name, module, docstring, signature, pickling by name.
+PyObject* routine_doc(PyObject* self, void*) {
+  const RoutineDef* d = reinterpret_cast<RoutineObject*>(self)->def;
+  std::string head = std::string(d->name) + "(" + d->params + " check=True)";
+  for (size_t i = 0; i < head.size(); ++i)
+    if (head[i] == ' ') head.insert(i++, ",");
+  return PyUnicode_FromFormat("%s\n\n%s  check: raise B2Error on a non-zero status instead of returning it.", head.c_str(), d->doc);
+}
+PyObject* routine_signature(PyObject* self, void*) { return PyObject_CallFunction(g_signature, "s", reinterpret_cast<RoutineObject*>(self)->def->params); }
+PyObject* routine_reduce(PyObject* self, PyObject*) { return Py_BuildValue("O(s)", g_lookup, reinterpret_cast<RoutineObject*>(self)->def->name); }
+PyMethodDef routine_methods[] = {{"__reduce__", routine_reduce, METH_NOARGS, nullptr}, {nullptr, nullptr, 0, nullptr}};
 PyObject* routine_name(PyObject* self, void*) { return PyUnicode_FromString(reinterpret_cast<RoutineObject*>(self)->def->name); }
 PyMemberDef routine_members[] = {{"__vectorcalloffset__", T_PYSSIZET, offsetof(RoutineObject, vectorcall), READONLY, nullptr},
                                  {nullptr, 0, 0, 0, nullptr}};
-PyGetSetDef routine_getset[] = {{"__name__", routine_name, nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr, nullptr, nullptr}};
+PyGetSetDef routine_getset[] = {{"__name__", routine_name, nullptr, nullptr, nullptr},
+                                {"__qualname__", routine_name, nullptr, nullptr, nullptr},
+                                {"__doc__", routine_doc, nullptr, nullptr, nullptr},
+                                {"__signature__", routine_signature, nullptr, nullptr, nullptr},
+                                {nullptr, nullptr, nullptr, nullptr, nullptr}};
 PyType_Slot routine_slots[] = {{Py_tp_dealloc, (void*)routine_dealloc},
                                {Py_tp_call, (void*)PyVectorcall_Call},
                                {Py_tp_repr, (void*)routine_repr},
                                {Py_tp_members, routine_members},
+                               {Py_tp_methods, routine_methods},
                                {Py_tp_getset, routine_getset},
                                {0, nullptr}};
 PyType_Spec routine_spec = {"paper_2411_07211_b200._binding.Routine", sizeof(RoutineObject), 0,
@@ -381,14 +419,16 @@ PyObject* keep(PyObject*, PyObject* obj) {
   Py_RETURN_NONE;
 }
 
-// routines(lib_path, error_class, ensure_loaded) -> {name: callable}
+// routines(lib_path, error_class, ensure_loaded, signature, lookup) -> {name: callable}
 PyObject* routines(PyObject*, PyObject* args) {
   const char* path;
-  PyObject *err, *ensure;
-  if (!PyArg_ParseTuple(args, "sOO", &path, &err, &ensure)) return nullptr;
+  PyObject *err, *ensure, *signature, *lookup;
+  if (!PyArg_ParseTuple(args, "sOOOO", &path, &err, &ensure, &signature, &lookup)) return nullptr;
   g_lib_path = path;
   Py_XSETREF(g_error_class, Py_NewRef(err));
   Py_XSETREF(g_ensure_loaded, Py_NewRef(ensure));
+  Py_XSETREF(g_signature, Py_NewRef(signature));
+  Py_XSETREF(g_lookup, Py_NewRef(lookup));
   PyObject* out = PyDict_New();
   for (const RoutineDef& d : kRoutines) {
     RoutineObject* r = PyObject_New(RoutineObject, g_routine_type);

@@ -113,3 +113,23 @@ def test_another_interpreter_or_torch_rebuilds_the_module(monkeypatch):
         m.setattr(sys, "version", "4.0")
         assert build._binding_digest() != now and build._digest() == library
     assert build._binding_digest() == now
+
+
+def test_routines_describe_themselves(b2):
+    """Name, docstring, signature and pickling, as Python functions have them."""
+    import copy
+    import inspect
+    import pickle
+    for name in b2._NAMES:
+        f = getattr(b2, name)
+        sig = inspect.signature(f)
+        assert list(sig.parameters)[0] == "ctx" and sig.parameters["check"].default is True
+        assert f.__name__ == name and inspect.getdoc(f)
+        assert pickle.loads(pickle.dumps(f)) is f and copy.deepcopy(f) is f
+        if name != "rotm":  # (a Python function around the native one)
+            assert f.__doc__.startswith(f"{name}{sig}") and f.__qualname__ == name
+    assert list(inspect.signature(b2.gemv).parameters) == ["ctx", "order", "trans", "m", "n", "alpha", "a", "lda", "x", "incx",
+                                                           "beta", "y", "incy", "check"]
+    inspect.signature(b2.trsv).bind(1, 2, 3, 4, 5, 6, "a", 7, x="x", incx=1)
+    with pytest.raises(TypeError):
+        inspect.signature(b2.copy).bind(1, 2)
