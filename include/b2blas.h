@@ -19,6 +19,8 @@
  *     must not overlap (except where the routine is in place by definition).
  *   - Matrices: order B2_ROW_MAJOR: A(i,j) = a[i*lda + j], lda >= max(1, #columns);
  *     order B2_COL_MAJOR: A(i,j) = a[j*lda + i], lda >= max(1, #rows).
+ *   - Calls may be captured into a CUDA graph (after a first call outside any capture, which
+ *     loads the kernels) and replayed; replays that share a workspace are ordered like calls.
  *   - Return value: 0 on success; -k when argument number k is invalid (1-based, not
  *     counting ctx; nothing is launched); a positive B2_STATUS_* code otherwise.
  *   - n == 0 (or m == 0 or n == 0 for matrices) is a successful no-op; reductions then

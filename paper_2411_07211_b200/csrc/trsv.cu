@@ -553,12 +553,27 @@ static int trsv_variant(const Launch& l, const TrsvArgs<T>& args, bool coltype, 
 }
 
 // Call tags: unique per call within the process, never 0, so that words left in the workspace
-// by earlier calls can never look "ready".
+// by earlier calls can never look "ready" (replays of a captured call: trsv_forget_if_captured).
 static unsigned next_tag() {
   static std::atomic<unsigned> counter{0x2b7e1516u};
   unsigned t = counter.fetch_add(1u) + 1u;
   if (t == 0u) t = counter.fetch_add(1u) + 1u;
   return t;
+}
+
+__global__ void __launch_bounds__(kThreads) trsv_forget(unsigned long long* words, size_t n) {
+  grid_dep_wait();
+  grid_dep_launch();
+  for (size_t i = (size_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (size_t)gridDim.x * kThreads) words[i] = 0ull;
+}
+int trsv_forget_if_captured(const Launch& l, size_t bytes) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(l.stream, &st) != cudaSuccess) (void)cudaGetLastError();  // (the launch will say what is wrong)
+  if (st == cudaStreamCaptureStatusNone) return B2_STATUS_OK;
+  const size_t n = bytes / 8, blocks = (n + kThreads - 1) / kThreads;
+  const size_t cap = (size_t)sm_count() * 8;
+  launch_chained(trsv_forget, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(kThreads), 0, l.stream, reinterpret_cast<unsigned long long*>(l.scratch), n);
+  return check_launch();
 }
 
 template <typename T>
@@ -620,6 +635,7 @@ static int trsv_impl(const b2_ctx* ctx, int order, int uplo, int trans, int diag
     int64_t d = knob(kKnobTrsvPrefetchBytes) / (tile_bytes * args.nb);
     args.pf_dist = (int)(d < 0 ? 0 : d > 64 ? 64 : d);
   }
+  if (int st = trsv_forget_if_captured(l, xbuf_bytes)) return st;
   constexpr int V = VecLen<T>::value;
   if (aligned_to(a, 16) && lda % V == 0) return trsv_variant<T, V>(l, args, coltype, !eff_lower, unit);
   return trsv_variant<T, 1>(l, args, coltype, !eff_lower, unit);

@@ -793,7 +793,7 @@ static int max_clusters() {
 }
 
 template <typename T, bool COLTYPE, bool AL>
-static int launch_cluster(const Launch& l, Args<T>& p, bool* handled) {
+static int launch_cluster(const Launch& l, Args<T>& p, size_t tagged_bytes, bool* handled) {
   constexpr int SPB = Geo<T>::NB / kStrip;
   int room = max_clusters<T, COLTYPE, AL>() - 1;
   if (room < 0) return B2_STATUS_OK;
@@ -805,6 +805,7 @@ static int launch_cluster(const Launch& l, Args<T>& p, bool* handled) {
   p.H = streams * kCS;
   if (strips > kStrips * p.H && cap != 0) return B2_STATUS_OK;  // (no streaming blocks at all: a test's choice)
   *handled = true;
+  if (int st = trsv_forget_if_captured(l, tagged_bytes)) return st;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -822,16 +823,17 @@ static int launch_cluster(const Launch& l, Args<T>& p, bool* handled) {
   return check_launch();
 }
 
-// Workspace of a solve of K block rows: published x and far sums, inverses, their flags.
+// Workspace of a solve of K block rows: published x and far sums, flags of the inverses -- what carries tags -- and the
+// inverses.
 template <typename T>
 struct Scratch {
-  size_t words, inverses, total;
+  size_t words, tagged, total;
   explicit Scratch(int64_t K) {
     constexpr size_t NB = Geo<T>::NB;
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
     words = up((size_t)K * NB * Words<T>::N * 8);
-    inverses = up((size_t)std::max<int64_t>(0, K - kCS) * NB * NB * sizeof(T));
-    total = 2 * words + inverses + up((size_t)K * 4);
+    tagged = 2 * words + up((size_t)K * 4);
+    total = tagged + (size_t)std::max<int64_t>(0, K - kCS) * NB * NB * sizeof(T);
   }
 };
 
@@ -860,8 +862,8 @@ int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, in
   p.incx = incx;
   p.xbuf = reinterpret_cast<u64*>(l.scratch);
   p.far = reinterpret_cast<u64*>(l.scratch + w.words);
-  p.winv = reinterpret_cast<T*>(l.scratch + 2 * w.words);
-  p.flags = reinterpret_cast<unsigned*>(l.scratch + 2 * w.words + w.inverses);
+  p.flags = reinterpret_cast<unsigned*>(l.scratch + 2 * w.words);
+  p.winv = reinterpret_cast<T*>(l.scratch + w.tagged);
   p.ctl = l.ctl;
   p.K = (int)K;
   p.backward = backward;
@@ -877,8 +879,8 @@ int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, in
   }
 #endif
   const bool al = aligned_to(a, 16) && lda % Geo<T>::V == 0;
-  if (coltype) return al ? launch_cluster<T, true, true>(l, p, handled) : launch_cluster<T, true, false>(l, p, handled);
-  return al ? launch_cluster<T, false, true>(l, p, handled) : launch_cluster<T, false, false>(l, p, handled);
+  if (coltype) return al ? launch_cluster<T, true, true>(l, p, w.tagged, handled) : launch_cluster<T, true, false>(l, p, w.tagged, handled);
+  return al ? launch_cluster<T, false, true>(l, p, w.tagged, handled) : launch_cluster<T, false, false>(l, p, w.tagged, handled);
 }
 
 template int trsv_cluster_try<float>(const Launch&, bool, bool, bool, int64_t, const float*, int64_t, float*, int64_t, unsigned, bool*);

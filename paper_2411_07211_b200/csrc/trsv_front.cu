@@ -866,6 +866,7 @@ int trsv_front_try(const Launch& l, bool coltype, bool backward, bool unit, int6
   // (measured at n = 11520 / 8192: block by block with the premultiplied last tile is the
   // fastest form for both precisions -- float 156-162 us against 168-175 us in clusters of 8,
   // double 180 us against 216 us -- so clusters are off by default)
+  if (int st = trsv_forget_if_captured(l, xbuf_words * 8)) return st;
   const bool want_cluster = nb >= 2 && (knob(kKnobTrsvCluster) >= 2 || (knob(kKnobTrsvCluster) == 1 && sizeof(T) == 4));
   if (coltype)
     return backward ? launch_diag<T, true, true>(l, args, nb, want_cluster, unit)

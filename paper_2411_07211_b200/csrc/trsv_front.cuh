@@ -4,6 +4,12 @@
 
 namespace b2 {
 
+// Clears the first `bytes` (a multiple of 8) of the workspace in front of a solve that is being captured into a graph; does nothing
+// otherwise.  The kernels tell values of this call from older ones by a tag that is drawn when the call is made; a
+// captured solve carries the same tag on every replay, and without this would take the words that the replay before it
+// left for its own.
+int trsv_forget_if_captured(const Launch& l, size_t bytes);
+
 // Tries the sub-block kernel.  Returns a status; *handled is false (and nothing was launched)
 // when the call does not meet the kernel's preconditions (16-byte aligned matrix, lda a
 // multiple of the pack length, workspace large enough) -- the caller then uses the general

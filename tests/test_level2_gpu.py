@@ -446,6 +446,41 @@ def test_level2_determinism(b2, ctx, dtype):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("kernel", [0, 2, 3])
+def test_trsv_replayed_from_a_graph(b2, dtype, kernel):
+    """A captured solve is replayed with other data in the same buffers: every replay gives the bits of a plain call.
+    (Its values in the workspace carry the tag of the captured call every time.)"""
+    old = b2.get_tuning(b2.KNOB_TRSV_FRONT)
+    b2.set_tuning(b2.KNOB_TRSV_FRONT, kernel)
+    try:
+        for n in (131, 2435):
+            ctx = b2.Context()
+            ctx.reset()
+            mats = [torch.from_numpy(tri_buf(s, n, n + 1, dtype, orc.ROW_MAJOR, orc.LOWER, orc.NON_UNIT)).cuda() for s in (21, 22, 23)]
+            rhs = [torch.from_numpy(synth.vector_np(s, n, n, dtype)).cuda() for s in (5, 6, 7)]
+            call = lambda c, a, x: b2.trsv(c, orc.ROW_MAJOR, orc.LOWER, orc.NO_TRANS, orc.NON_UNIT, n, a, n + 1, x, 1)
+            want = []
+            for a, b in zip(mats, rhs):
+                want.append(b.clone())
+                call(ctx, a, want[-1])
+            a, x = mats[0].clone(), rhs[0].clone()
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                call(ctx, a, x)
+                b2.scal(ctx, n, 1.0, x, 1)
+            for k in (0, 1, 2, 2, 0):
+                a.copy_(mats[k])
+                x.copy_(rhs[k])
+                graph.replay()
+                torch.cuda.synchronize()
+                assert ctx.device_status() == 0 and torch.equal(x, want[k]), (n, k)
+            del graph
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_FRONT, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 def test_workspace_query_keeps_the_kernels(b2, ctx, dtype):
     """With exactly b2_workspace_query bytes trsv and symv run on the kernels they run on with the default workspace:
     equal bits, which the kernels behind them do not give (their sums run in another order)."""
