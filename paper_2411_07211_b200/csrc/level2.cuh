@@ -190,7 +190,10 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
   // microsecond longer here than it does in a kernel without this loop, and with every step of that column in it these
   // blocks were the tail of the launch: trmv in double, n = 5360, 26.2 us without any such loop, 30.0 with the loop
   // for whole tiles only, 25.4 so; n = 3008 in float 14.9 -> 9.6; symv in float, n = 7400, 28.4, 30.9, 24.4.
-  constexpr bool CUT = STEADY && !SHIFT && K::TRI == TRI_UPPER;
+  // With shifted packs the first tile of a lower triangle, its longest column, is cut as well, by the beginning of the
+  // rows: symv in double, n = 4001, upper / lower, by elements 26.3 / 25.5, in shifted packs 26.6 / 28.4, 21.5 / 23.0 so.
+  constexpr bool CUT = STEADY && (K::TRI == TRI_UPPER || (SHIFT && K::TRI == TRI_LOWER));
+  constexpr bool CUT_FIRST = CUT && K::TRI == TRI_LOWER;
   int64_t fast_lo = 0, fast_hi = 0;  // first row of the first such step, end of the last
   if constexpr (STEADY) {
     if (CUT || (c_lo + TC <= p.cols && (!SHIFT || c_lo > 0))) {
@@ -214,8 +217,8 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
           load_xc(xcv[0], c_lo);
         }
         if constexpr (CUT) {
-          if (c_lo + TC > p.cols) {
-            const int nc = (int)(p.cols - c_lo);  // columns that exist
+          if (CUT_FIRST ? c_lo == 0 : c_lo + TC > p.cols) {
+            const int nc = (int)min((int64_t)(TC + SH), p.cols - c_lo);  // columns that exist (CUT_FIRST: from 0 on)
             auto cut_steps = [&](auto packs) {    // in whole packs, or by elements
 #pragma unroll 1
               for (int st = 0; st < nst; ++st) {
@@ -226,11 +229,11 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
 #pragma unroll
                   for (int u = 0; u < CU; ++u) {
                     const T* ap = at + ru * rstride + u * (LPR * V);
-                    const int lc = (u * LPR + q) * V;
+                    const int lc = (u * LPR + q) * V - s;
                     if constexpr (decltype(packs)::value) av[ru][u] = ld_nc_if<T, V>(ap, lc < nc);
                     else {
 #pragma unroll
-                      for (int e = 0; e < V; ++e) av[ru][u].v[e] = ld_el_if<T>(ap + e, lc + e < nc);
+                      for (int e = 0; e < V; ++e) av[ru][u].v[e] = ld_el_if<T>(ap + e, CUT_FIRST ? lc + e >= 0 : lc + e < nc);
                     }
                   }
 #pragma unroll
@@ -256,7 +259,7 @@ __global__ void __launch_bounds__(kThreads, S::MINB) l2_tile_kernel(const L2Args
                 }
               }
             };
-            if (nc % V == 0) cut_steps(std::true_type());
+            if (!SHIFT && nc % V == 0) cut_steps(std::bool_constant<!SHIFT>());
             else cut_steps(std::false_type());
             rb = fast_hi - RB;
             continue;
@@ -556,6 +559,7 @@ __global__ void __launch_bounds__(kThreads) l2_scale_y(T* y, int64_t incy, int64
 // ------------------------------------------------------------------------------- host side
 struct L2Plan {
   int shape;             // index into the shape table
+  int tile_cols = 0;     // columns of a column tile (row-dot plans)
   int64_t rows_per_cta;  // multiple of the shape's RB
   int ctiles_per_cta;
 };
@@ -713,6 +717,7 @@ static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok) {
     cpc = std::max(cpc, (nct + want_ncs - 1) / want_ncs);
   }
   p.ctiles_per_cta = (int)cpc;
+  p.tile_cols = shape_packs_per_row(p.shape) * V;
   p.rows_per_cta = shape_rb(p.shape);
   return p;
 }

@@ -339,7 +339,7 @@ def test_cluster_gather_kernel(b2, ctx, dtype, mode):
 
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(63, 1), (130, 2), (513, 3), (516, 0), (641, 7), (1090, 2), (1151, 1), (1153, 0)])
-def test_upper_triangle_cut_last_column_tile(b2, ctx, dtype, n, pad):
+def test_cut_longest_column_tile(b2, ctx, dtype, n, pad):
     """The tile kernels' column sums where the last column tile of an upper triangle (64 or 128 columns, the longest
     of them) is cut by the matrix edge: on a pack boundary, inside a pack, with one column and with all but one, in
     blocks of 512 rows that lie above the diagonal whole, in part and not at all; rows on and off 16-byte boundaries."""
@@ -356,13 +356,14 @@ def test_upper_triangle_cut_last_column_tile(b2, ctx, dtype, n, pad):
             absterms = orc.trmv(orc.ROW_MAJOR, orc.UPPER, orc.TRANS, diag, n, a, lda, ox, inc)
             assert_close(pick(gx.host(), n, inc), pick(ox, n, inc), absterms, dtype, f"trmv lda={lda}")
             gx.check_guards()
-            a = tri_buf(9, n, lda, dtype, orc.ROW_MAJOR, orc.UPPER, orc.NON_UNIT)
-            ga, gx, gy = Guarded(a), Guarded(place(x, inc)), Guarded(y)
-            b2.symv(ctx, orc.ROW_MAJOR, orc.UPPER, n, 1.25, ga.t, lda, gx.t, inc, 0.5, gy.t, 1)
-            oy = y.copy()
-            absterms = orc.symv(orc.ROW_MAJOR, orc.UPPER, n, dtype(1.25), a, lda, place(x, inc), inc, dtype(0.5), oy, 1)
-            assert_close(gy.host(), oy, absterms, dtype, f"symv lda={lda}")
-            gy.check_guards()
+            for uplo, off in itertools.product(UPLOS, (0, 1)):  # (off 16-byte boundaries a lower triangle's first tile is cut too)
+                a = tri_buf(9, n, lda, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+                ga, gx, gy = Guarded(a, off), Guarded(place(x, inc)), Guarded(y)
+                b2.symv(ctx, orc.ROW_MAJOR, uplo, n, 1.25, ga.t, lda, gx.t, inc, 0.5, gy.t, 1)
+                oy = y.copy()
+                absterms = orc.symv(orc.ROW_MAJOR, uplo, n, dtype(1.25), a, lda, place(x, inc), inc, dtype(0.5), oy, 1)
+                assert_close(gy.host(), oy, absterms, dtype, f"symv lda={lda} {uplo} off={off}")
+                gy.check_guards()
     finally:
         b2.set_tuning(b2.KNOB_GATHER, old[0])
         b2.set_tuning(b2.KNOB_TRI_TILE, old[1])
