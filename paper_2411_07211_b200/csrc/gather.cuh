@@ -1,4 +1,4 @@
-// Small and middle-sized gemv, symv and trmv in one launch (Section 6.2.2): every output is gathered by one cluster.
+// Small and middle-sized gemv, symv and trmv (column sums) in one launch (Section 6.2.2): every output is gathered by one cluster.
 //
 // What bounds such a call is latency: launches, passes over partial sums, barriers.  A cluster of 1 .. 8 blocks
 // owns 32 outputs and reads everything they depend on -- 32 rows of the canonical row-major view (row part), 32
@@ -51,12 +51,14 @@ struct Args {
 template <typename T>
 __device__ __forceinline__ T ld_x(const T* p) { return B2_GUARD(p, sizeof(T)) ? *p : T(0); }
 
-// ROWOUT / COLOUT of the kind: row part / column part.  Triangular kinds that are not symmetric work in place.
+// ROWOUT / COLOUT of the kind: row part / column part.  Triangular kinds that are not symmetric work in place (and
+// have a column part only: see run()).
 template <typename T, bool AL, class K>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kernel(const Args<T> p) {
   constexpr int V = VecLen<T>::value, SH = AL ? 0 : V - 1;
   constexpr int CH = 2 * 32 * V;                              // columns of a row-part chunk
   constexpr bool INPLACE = K::TRI != TRI_FULL && !K::SYM;
+  static_assert(!(INPLACE && K::ROWOUT), "row sums are not formed in place");
   using P = Pack<T, V>;
   __shared__ T s_row[R], s_col[kWarps][R], s_sum[kMaxCluster][R];
   __shared__ int s_last;
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
   bool last_reader = false;
   if (INPLACE) {
     T* xs = reinterpret_cast<T*>(gather_smem);
-    const int lo = K::ROWOUT ? rlo : clo, hi = K::ROWOUT ? rhi : chi;
+    const int lo = clo, hi = chi;
     for (int t0 = lo + tid; t0 < hi; t0 += 8 * kThreads) {  // eight loads in flight
       T v[8];
 #pragma unroll
@@ -146,8 +148,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
 #pragma unroll
           for (int e = 0; e < V; ++e) {
             const bool in = c + e >= rlo && c + e < rhi;
-            if constexpr (INPLACE) xv[h][e] = in ? x_at(c + e) : T(0);
-            else xv[h][e] = ld_el_if<T>(xp + (int64_t)(c + e) * xi, in);
+            xv[h][e] = ld_el_if<T>(xp + (int64_t)(c + e) * xi, in);
           }
         }
 #pragma unroll
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(T) == 8 ? 3 : 4) gather_kerne
 
 // Launches the kernel; *handled is false (nothing launched) where the sizes do not allow it.
 template <typename T, bool AL, class K>
-static int launch(const Launch& l, const L2Args<T>& q, bool* handled) {
+static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_launch) {
   constexpr int V = VecLen<T>::value, CH = 2 * 32 * V;
   constexpr bool INPLACE = K::TRI != TRI_FULL && !K::SYM;
   const int64_t nout = K::ROWOUT ? q.rows : q.cols, len = K::ROWOUT ? q.cols : q.rows;
@@ -308,7 +309,14 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled) {
   int nr = 1;
   while (nr < kMaxCluster && 2 * nr <= items && groups * nr * (INPLACE ? 2 : 1) <= wave) nr *= 2;
   const int64_t bytes = q.rows * q.cols * (int64_t)sizeof(T) / (INPLACE ? 2 : 1);
-  if (knob(kKnobGather) < 2 && bytes > kMaxBytesPerBlock * groups * nr) return B2_STATUS_OK;
+  if (knob(kKnobGather) < 2) {  // (see run())
+    if (bytes > kMaxBytesPerBlock * groups * nr) return B2_STATUS_OK;
+    const bool turns = items > nr, late = groups * nr * 8 > wave * 7;
+    if (K::TRI == TRI_FULL && K::ROWOUT &&
+        ((late && !(sizeof(T) == 8 && items == 1)) || (turns && nr <= 2) ||
+         (one_launch && (turns || (!AL && len <= (sizeof(T) == 4 ? 768 : 512)))))) return B2_STATUS_OK;
+    if (K::TRI == TRI_FULL && K::COLOUT && sizeof(T) == 4 && AL && late) return B2_STATUS_OK;
+  }
   Args<T> p = {};
   p.a = q.a;
   p.lda = q.lda;
@@ -340,20 +348,42 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled) {
   (void)cudaLaunchKernelEx(&cfg, gather_kernel<T, AL, K>, p);
   return check_launch();
 }
-// Where one launch by clusters is the faster way (total matrix bytes; measured with three matrices in turn, against
-// the tile kernels and their finalize pass): gemv up to 20 MB (n = 1500 double 16.1 -> 10.0 us for two calls, 2000
-// float 13.1 -> 11.1), off 16-byte boundaries up to 34 MB (2001 double 22.1 -> 19.9); trmv up to 36 MB (2000 double
-// 20 -> 17.7 us with its copy, 3000 float 20.2 -> 19.3), unaligned up to 72 MB (3001 double 40 -> 26.6); symv, which
-// reads its elements twice, up to 6 MB (1000 float 11.8 -> 8.4), unaligned up to 72 MB (1001 float 21.7 -> 9,
-// 3001 float 40 -> 29).
+// Where one launch by clusters is the faster way: up to a matrix size (of the whole square, where a triangle is read).
+// Against the tile kernels and their second pass, three matrices in turn, tile kernel / this one in us, with the last
+// size in MB where this one wins and the first where it does not:
+//   gemv row part   the blocks must fit one wave: a second one costs more than the second pass (double 4000 x 400, 12.8
+//                   MB, 4.1 / 5.6), except in double where a row is a single chunk (16000 x 128 5.1 / 3.7).  Where the tile kernel needs no second pass either (one_launch:
+//                   short rows) it is the faster one as soon as blocks here take turns (float 4899 x 612, 12 MB: 4.5 / 6.1;
+//                   8 MB: 4.7 / 3.7), and off 16-byte boundaries nearly always (double 2000 x 256 2.7 / 3.9, float 4000
+//                   x 512 4.0 / 4.9; 1000 x 707 3.8 / 4.5, but 1000 x 1000 4.5 / 3.5).
+//                   Float 16 MB 5.2 / 4.8, 24 6.4 / 5.8, 32 7.4 / 7.6 (866 x 6928 and like it); double 50 11.7 / 11.2, 64
+//                   13.4 / 13.5; unaligned to 100 MB and beyond (21.2 / 18.5).
+//   gemv column part  float 16 MB 6.3 / 5.8, 20 7.0 / 7.4, one wave of blocks here too (707 x 5656 6.2 / 7.8); double 20
+//                   8.2 / 6.6, 24 7.4 / 7.5 (32 11.7 / 9.2, but 36 9.6 / 11.6); unaligned float 32
+//                   12.6 / 12.5, 40 13.6 / 15.1, double 64 16.7 / 15.5, 80 18.6 / 22.3.
+//   trmv row part   never, and not built: the tile kernel's second pass costs less than the in-place protocol (n = 64 4.6 / 4.9, 512 4.6 /
+//                   5.7, 3008 in float 6.9 / 9.2; unaligned 4.6 / 4.9, 5.9 / 6.2, n = 3001 8.7 / 10.5).
+//   trmv column part  float 16 MB 8.9 / 8.5, 20 8.5 / 11.2; double 50 11.1 / 10.0, 64 11.2 / 11.9 (20 and 24 MB 7.3 / 8.8 and
+//                   7.9 / 9.8 on the lower triangle, 7.0 / 6.8 and 7.7 / 7.2 on the upper one); unaligned float 80 MB
+//                   20.8 / 15.1, 100 21.6 / 22.5, double 160 26.7 / 24.8 (beyond that x does not fit shared memory).
+//   symv            reads its elements twice: float 20 MB 7.9 / 7.6, 24 7.9 / 9.3 (between 6 and 20 within 5 %); double 20
+//                   7.6 / 6.5, 24 7.5 / 7.6; unaligned float 80 25.0 / 20.4, 100 24.4 / 27.8 (upper), double 72 18.5 /
+//                   18.1, 98 19.1 / 26.1 (upper).
 template <typename T, class K>
-static int run(const Launch& l, const L2Args<T>& q, bool* handled) {
+constexpr int64_t max_mb(bool al) {
+  constexpr bool F = sizeof(T) == 4;
+  if (K::SYM) return al ? (F ? 20 : 22) : (F ? 85 : 80);
+  if (K::TRI != TRI_FULL) return al ? (F ? 17 : 55) : (F ? 85 : 170);
+  if (K::ROWOUT) return al ? (F ? 24 : 50) : 110;
+  return al ? (F ? 17 : 22) : (F ? 35 : 70);
+}
+template <typename T, class K>
+static int run(const Launch& l, const L2Args<T>& q, bool* handled, bool one_launch = false) {
   *handled = false;
   if (knob(kKnobGather) == 0) return B2_STATUS_OK;
   const bool al = aligned_to(q.a, 16) && q.lda % VecLen<T>::value == 0;
-  const int64_t mb = K::TRI == TRI_FULL ? (al ? 20 : 34) : K::SYM ? (al ? 6 : 73) : (al ? 36 : 73);
-  if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)mb * 1e6) return B2_STATUS_OK;
-  return al ? launch<T, true, K>(l, q, handled) : launch<T, false, K>(l, q, handled);
+  if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)max_mb<T, K>(al) * 1e6) return B2_STATUS_OK;
+  return al ? launch<T, true, K>(l, q, handled, one_launch) : launch<T, false, K>(l, q, handled, one_launch);
 }
 
 }  // namespace ga

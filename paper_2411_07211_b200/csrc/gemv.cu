@@ -47,16 +47,17 @@ static int gemv_impl(const b2_ctx* ctx, int order, int trans, int64_t m, int64_t
   if (rowdot) {
     args.xc = vec_base(x, lenx, incx);
     args.incxc = incx;
+    const L2Plan plan = plan_rowout(args, true, kShortRowsGemv);
     {
       bool handled = false;
-      const int st = ga::run<T, GemvRow>(l, args, &handled);
+      const int st = ga::run<T, GemvRow>(l, args, &handled, plan.ctiles_per_cta * plan.tile_cols >= args.cols);
       if (handled) return st;
     }
     if (knob(kKnobNarrowBlock) && block_narrow_applies(a, lda, args.rows, args.cols))
       return block_rowdot<T>(l, a, args.rows, args.cols, args.xc, incx, alpha, beta, args.y, incy);
     if (skinny_applies(a, lda, args.rows, args.cols, true))
       return skinny_rowdot<T>(l, a, args.rows, args.cols, args.xc, incx, alpha, beta, args.y, incy);
-    return l2_dispatch<T, GemvRow, true>(l, args, plan_rowout(args, true), true);
+    return l2_dispatch<T, GemvRow, true>(l, args, plan, true);
   }
   args.xr = vec_base(x, lenx, incx);
   args.incxr = incx;

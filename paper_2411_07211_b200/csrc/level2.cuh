@@ -677,9 +677,15 @@ static int l2_launch(const Launch& l, const L2Args<T>& args, const L2Plan& plan,
 // kinds with one sum per element (gemv 8193 x 8191 175 us against 193, trmv n = 8191 95 against 112) and lose for
 // symv (142 against 120).  Float: symv n = 8191 120 -> 72 us a pair, 11519 210 -> 115, trmv 8191 67 -> 58 with its
 // copy, 11519 124 -> 100, gemv 8193 x 8191 108 -> 94.
+// Row sums of short rows stay with element loads while the matrix is small (short_rows: up to which length).  Up to 1024
+// elements a block covers the whole row then, and gemv needs no second pass: float 4000 x 512 6.4 us in shifted packs,
+// 4.0 so, 1000 x 1000 5.0 / 4.5; with 707 columns 16 MB 6.5 / 6.1, 20 MB 6.6 / 7.0.  trmv: n = 256 5.3 / 4.0, 700 6.0 / 5.4,
+// 900 5.7 / 6.0.
+constexpr int kShortRowsGemv = 1024, kShortRowsTrmv = 768;
 template <typename T>
-static bool l2_shift(const L2Args<T>& a, bool sym) {
+static bool l2_shift(const L2Args<T>& a, bool sym, int short_rows) {
   constexpr int V = VecLen<T>::value;
+  if (a.cols <= short_rows && (double)a.rows * (double)a.cols * sizeof(T) < 18e6) return false;
   return (sizeof(T) == 4 || sym) && !(aligned_to(a.a, 16) && a.lda % V == 0) && a.cols > 16 * V && a.rows >= ShapeMid::RB;
 }
 
@@ -688,7 +694,7 @@ template <typename T, class K, bool NARROW>
 static int l2_dispatch(const Launch& l, const L2Args<T>& args, const L2Plan& plan, bool allow_direct) {
   constexpr int V = VecLen<T>::value;
   if (aligned_to(args.a, 16) && args.lda % V == 0) return l2_launch<T, V, K, NARROW>(l, args, plan, allow_direct);
-  if (l2_shift(args, K::SYM) && plan.shape == SHAPE_MID) {
+  if (l2_shift(args, K::SYM, K::COLOUT ? 0 : K::TRI == TRI_FULL ? kShortRowsGemv : kShortRowsTrmv) && plan.shape == SHAPE_MID) {
     const int st = l2_launch_shape<T, V, K, ShapeMid, true>(l, args, plan.rows_per_cta, plan.ctiles_per_cta, allow_direct);
     if (st != B2_STATUS_WORKSPACE_TOO_SMALL) return st;
   }
@@ -698,12 +704,13 @@ static int l2_dispatch(const Launch& l, const L2Args<T>& args, const L2Plan& pla
 // Plans.  ROWOUT-only kinds: one row step per block, several column tiles per block so that a
 // block streams about `tile_bytes`; the remaining column splits become partials.
 template <typename T>
-static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, false) ? VecLen<T>::value : 1;
+static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok, int short_rows) {
+  const bool shift = l2_shift(a, false, short_rows);
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || shift ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
   // (shifted packs: short segments, 4 x values for 8 packs instead of 16)
-  p.shape = nv >= 128 && !l2_shift(a, false) ? SHAPE_WIDE : (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
+  p.shape = nv >= 128 && !shift ? SHAPE_WIDE : (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
   const int64_t tile_bytes = (int64_t)shape_rb(p.shape) * shape_packs_per_row(p.shape) * V * sizeof(T);
   int64_t cpc = knob(kKnobGemvNTileBytes) / tile_bytes;
   if (cpc < 1) cpc = 1;
@@ -724,7 +731,7 @@ static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok) {
 // COLOUT kinds: one column tile per block, tall row bands; the bands become partials.
 template <typename T>
 static L2Plan plan_colout(const L2Args<T>& a, bool narrow_ok, int64_t rows_per_cta) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, false) ? VecLen<T>::value : 1;
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, false, 0) ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
   p.shape = (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;

@@ -24,10 +24,10 @@ static int check_square(int order, int64_t n, const T* a, int64_t lda, int arg_o
 
 template <typename T>
 static L2Plan plan_tri(const L2Args<T>& a) {
-  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, true) ? VecLen<T>::value : 1;
+  const int V = (aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0) || l2_shift(a, true, 0) ? VecLen<T>::value : 1;
   const int64_t nv = (a.cols + V - 1) / V;
   L2Plan p;
-  p.shape = (nv >= 512 && !l2_shift(a, true) && knob(kKnobTriWide)) ? SHAPE_WIDE : SHAPE_MID;
+  p.shape = (nv >= 512 && !l2_shift(a, true, 0) && knob(kKnobTriWide)) ? SHAPE_WIDE : SHAPE_MID;
   p.ctiles_per_cta = 1;
   p.rows_per_cta = knob(kKnobTriRows);
   return p;
@@ -91,10 +91,12 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
 
 template <typename T, bool ROW, int TRI>
 static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
-  if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {
-    bool handled = false;
-    const int st = unit ? ga::run<T, Kind<ROW, !ROW, TRI, true, false>>(l, args, &handled) : ga::run<T, Kind<ROW, !ROW, TRI, false, false>>(l, args, &handled);
-    if (handled) return st;
+  if constexpr (!ROW) {
+    if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {
+      bool handled = false;
+      const int st = unit ? ga::run<T, Kind<false, true, TRI, true, false>>(l, args, &handled) : ga::run<T, Kind<false, true, TRI, false, false>>(l, args, &handled);
+      if (handled) return st;
+    }
   }
   // The tile kernel with the shared-memory ring serves trmv where it measured faster than the
   // general tile kernel: float row sums with a strided x (knob value 2: always, for the tests).
@@ -108,7 +110,7 @@ static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
                                                                 args.y, args.incy, &handled);
     if (handled) return st;
   }
-  const L2Plan plan = ROW ? plan_rowout(args, false) : plan_colout(args, false, knob(kKnobTriRows));
+  const L2Plan plan = ROW ? plan_rowout(args, false, kShortRowsTrmv) : plan_colout(args, false, knob(kKnobTriRows));
   if (unit) return l2_dispatch<T, Kind<ROW, !ROW, TRI, true, false>, false>(l, args, plan, false);
   return l2_dispatch<T, Kind<ROW, !ROW, TRI, false, false>, false>(l, args, plan, false);
 }
