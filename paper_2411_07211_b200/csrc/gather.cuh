@@ -315,7 +315,7 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_l
     if (K::TRI == TRI_FULL && K::ROWOUT &&
         ((late && !(sizeof(T) == 8 && items == 1)) || (turns && nr <= 2) ||
          (one_launch && (turns || (!AL && len <= (sizeof(T) == 4 ? 768 : 512)))))) return B2_STATUS_OK;
-    if (K::TRI == TRI_FULL && K::COLOUT && sizeof(T) == 4 && AL && late) return B2_STATUS_OK;
+    if (K::TRI == TRI_FULL && K::COLOUT && sizeof(T) == 4 && AL && (late || items > 4 * nr)) return B2_STATUS_OK;
   }
   Args<T> p = {};
   p.a = q.a;
@@ -349,23 +349,26 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_l
   return check_launch();
 }
 // Where one launch by clusters is the faster way: up to a matrix size (of the whole square, where a triangle is read).
-// Against the tile kernels and their second pass, three matrices in turn, tile kernel / this one in us, with the last
-// size in MB where this one wins and the first where it does not:
+// Against the tile kernels and their second pass, three matrices in turn, tile kernel / this one in us (each product
+// repeated; "both": the two products of a pass one after the other, which read the matrix through different SMs), with
+// the last size where this one wins and the first where it does not:
 //   gemv row part   the blocks must fit one wave: a second one costs more than the second pass (double 4000 x 400, 12.8
-//                   MB, 4.1 / 5.6), except in double where a row is a single chunk (16000 x 128 5.1 / 3.7).  Where the tile kernel needs no second pass either (one_launch:
-//                   short rows) it is the faster one as soon as blocks here take turns (float 4899 x 612, 12 MB: 4.5 / 6.1;
-//                   8 MB: 4.7 / 3.7), and off 16-byte boundaries nearly always (double 2000 x 256 2.7 / 3.9, float 4000
-//                   x 512 4.0 / 4.9; 1000 x 707 3.8 / 4.5, but 1000 x 1000 4.5 / 3.5).
-//                   Float 16 MB 5.2 / 4.8, 24 6.4 / 5.8, 32 7.4 / 7.6 (866 x 6928 and like it); double 50 11.7 / 11.2, 64
-//                   13.4 / 13.5; unaligned to 100 MB and beyond (21.2 / 18.5).
-//   gemv column part  float 16 MB 6.3 / 5.8, 20 7.0 / 7.4, one wave of blocks here too (707 x 5656 6.2 / 7.8); double 20
-//                   8.2 / 6.6, 24 7.4 / 7.5 (32 11.7 / 9.2, but 36 9.6 / 11.6); unaligned float 32
-//                   12.6 / 12.5, 40 13.6 / 15.1, double 64 16.7 / 15.5, 80 18.6 / 22.3.
-//   trmv row part   never, and not built: the tile kernel's second pass costs less than the in-place protocol (n = 64 4.6 / 4.9, 512 4.6 /
-//                   5.7, 3008 in float 6.9 / 9.2; unaligned 4.6 / 4.9, 5.9 / 6.2, n = 3001 8.7 / 10.5).
-//   trmv column part  float 16 MB 8.9 / 8.5, 20 8.5 / 11.2; double 50 11.1 / 10.0, 64 11.2 / 11.9 (20 and 24 MB 7.3 / 8.8 and
-//                   7.9 / 9.8 on the lower triangle, 7.0 / 6.8 and 7.7 / 7.2 on the upper one); unaligned float 80 MB
-//                   20.8 / 15.1, 100 21.6 / 22.5, double 160 26.7 / 24.8 (beyond that x does not fit shared memory).
+//                   MB, 4.1 / 5.6), except in double where a row is a single chunk (16000 x 128 5.1 / 3.7).  Where the
+//                   tile kernel needs no second pass either (one_launch: short rows) it is the faster one as soon as
+//                   blocks here take turns (float 4899 x 612, 12 MB, 4.5 / 6.1; 8 MB 4.7 / 3.7), and off 16-byte
+//                   boundaries nearly always (double 2000 x 256 2.7 / 3.9, float 4000 x 512 4.0 / 4.9, 1000 x 707
+//                   3.8 / 4.5, but 1000 x 1000 4.5 / 3.5).  Float 16 MB 5.2 / 4.8, 24 6.4 / 5.8, 32 7.4 / 7.6 (866 x 6928
+//                   and like it); double 50 11.7 / 11.2, 64 13.4 / 13.5; unaligned to 100 MB and beyond (21.2 / 18.5).
+//   gemv column part  float 16 MB 6.3 / 5.8, 20 7.0 / 7.4, one wave of blocks here too (707 x 5656 6.2 / 7.8) and no more
+//                   than four turns of them (both, 4896 x 608, 10.2 / 10.8 to 13.8); double 20 8.2 / 6.6, 24 7.4 / 7.5
+//                   (32 11.7 / 9.2, but 36 9.6 / 11.6); unaligned float 32 12.6 / 12.5, 40 13.6 / 15.1, double 64
+//                   16.7 / 15.5, 80 18.6 / 22.3.
+//   trmv row part   never, and not built: the tile kernel's second pass costs less than the in-place protocol (n = 64
+//                   4.6 / 4.9, 512 4.6 / 5.7, 3008 in float 6.9 / 9.2; unaligned 4.6 / 4.9, 5.9 / 6.2, n = 3001 8.7 / 10.5).
+//   trmv column part  both, lower and upper triangle: float 4 MB 12.8 / 10.9 and 12.1 / 11.9, 6 MB 12.6 / 11.3 and
+//                   12.2 / 13.3; double 18 13.3 / 13.2 and 13.8 / 14.2, 20 13.1 / 16.0 and 13.8 / 13.7 (equal from 32 to 50);
+//                   unaligned float 80 MB 20.8 / 15.1, 100 21.6 / 22.5, double 160 26.7 / 24.8 (beyond that x does not
+//                   fit shared memory).
 //   symv            reads its elements twice: float 20 MB 7.9 / 7.6, 24 7.9 / 9.3 (between 6 and 20 within 5 %); double 20
 //                   7.6 / 6.5, 24 7.5 / 7.6; unaligned float 80 25.0 / 20.4, 100 24.4 / 27.8 (upper), double 72 18.5 /
 //                   18.1, 98 19.1 / 26.1 (upper).
@@ -373,7 +376,7 @@ template <typename T, class K>
 constexpr int64_t max_mb(bool al) {
   constexpr bool F = sizeof(T) == 4;
   if (K::SYM) return al ? (F ? 20 : 22) : (F ? 85 : 80);
-  if (K::TRI != TRI_FULL) return al ? (F ? 17 : 55) : (F ? 85 : 170);
+  if (K::TRI != TRI_FULL) return al ? (F ? 5 : 18) : (F ? 85 : 170);
   if (K::ROWOUT) return al ? (F ? 24 : 50) : 110;
   return al ? (F ? 17 : 22) : (F ? 35 : 70);
 }
