@@ -76,7 +76,7 @@ size_t b2_workspace_query(int64_t m, int64_t n, size_t elem_bytes) {
       // symv, whose blocks produce row sums and column sums at once: one row of partials per column tile of 32 packs ...
       (tiles(sq + V - 1, seg) + 1) * sq * e + spill(sq) + 1024,
       // ... and, while it runs on the ring kernel, one per tile of a block row and one per block row
-      (double)sq * (double)sq * e / 2 <= b2::kSymvRingBytes ? (tiles(sq, seg) + tiles(sq, 128)) * sq * e + 512 : 0,
+      (double)sq * (double)sq * e / 2 <= b2::symv_ring_bytes(e) ? (tiles(sq, seg) + tiles(sq, 128)) * sq * e + 512 : 0,
       // trsv: tagged words and inverses of the cluster kernel; one or two words per unknown for the kernels behind it
       b2::trsv_cluster_scratch((int64_t)sq, e),
       vec * 8 * (e / 4),

@@ -408,7 +408,7 @@ static void dbg_commit(Launch& l) {
 #endif
 
 // Triangles (bytes) up to which symv runs on the tile kernel with the shared-memory ring (tri_impl.cuh).
-constexpr double kSymvRingBytes = 64.0 * 1024 * 1024;
+constexpr double symv_ring_bytes(size_t elem_bytes) { return (elem_bytes == 4 ? 42.0 : 68.0) * 1024 * 1024; }
 
 // Number of SMs of the current device (cached per device id).
 int sm_count();

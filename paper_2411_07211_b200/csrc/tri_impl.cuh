@@ -68,15 +68,13 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
                          : ga::run<T, Kind<true, true, TRI_LOWER, false, true>>(l, args, &handled);
     if (handled) return st;
   }
-  // The tile kernel with the shared-memory ring (16-byte aligned matrices) is the faster one while
-  // the triangle is small (n = 4096: 13 us against 19 us in float); from about 64 MiB of triangle
-  // on the general tile kernel streams faster (n = 32768 float: 320 us against 357 us).  Knob value
-  // 2 forces the ring kernel at every size (tests).
-  // (double, upper triangle: that kind of the general kernel spills 132 bytes per thread at its
-  // 64 registers and streams 10-15 % slower than the ring kernel at every size -- n = 32768:
-  // 780 us against 684 us)
-  const bool small = (double)n * (double)n * sizeof(T) / 2 <= kSymvRingBytes;
-  if (knob(kKnobTriTile) == 2 || (knob(kKnobTriTile) == 1 && (small || (sizeof(T) == 8 && upper)))) {
+  // The tile kernel with the shared-memory ring (16-byte aligned matrices) is the faster one while the triangle is small:
+  // its persistent blocks start at once, the general tile kernel streams faster.  Upper and lower triangle in turn,
+  // general / ring in us: float n = 4096 31.2 / 24.4, 4608 (40 MiB) 31.1 / 26.9, 4800 (44) 30.6 / 31.8, 5792 36.2 / 39.6,
+  // 8192 54.3 / 57.3; double n = 3008 28.1 / 24.1, 4096 (64) 37.9 / 36.7, 4352 (72) 39.8 / 40.0, 5008 47.3 / 49.8, 8192
+  // 96.9 / 106.3.  Knob value 2 forces the ring kernel at every size (tests).
+  const bool small = (double)n * (double)n * sizeof(T) / 2 <= symv_ring_bytes(sizeof(T));
+  if (knob(kKnobTriTile) == 2 || (knob(kKnobTriTile) == 1 && small)) {
     bool handled = false;
     const int st = upper ? tt::tri_tile_run<T, true, true, TRI_UPPER, false, true>(l, a, lda, n, args.xc, incx, alpha, beta,
                                                                                   args.y, incy, &handled)
