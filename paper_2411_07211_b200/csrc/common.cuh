@@ -457,16 +457,17 @@ inline void launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);  // (a failure is picked up by check_launch())
 }
 
-// The same as ONE cluster of grid.x blocks.
+// The same in clusters of `cluster` blocks.
 template <typename... KArgs, typename... Args>
-inline void launch_one_cluster(void (*kernel)(KArgs...), unsigned blocks, dim3 block, cudaStream_t stream, Args&&... args) {
+inline void launch_clusters(void (*kernel)(KArgs...), unsigned blocks, unsigned cluster, dim3 block, size_t smem, cudaStream_t stream, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = blocks;
+  attr[0].val.clusterDim.x = cluster;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;

@@ -332,20 +332,7 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_l
   p.rows = (int)q.rows;
   p.cols = (int)q.cols;
   *handled = true;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)nr;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)(groups * nr));
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = l.stream;
-  cfg.attrs = at;
-  cfg.numAttrs = knob(kKnobUsePdl) ? 2 : 1;
-  (void)cudaLaunchKernelEx(&cfg, gather_kernel<T, AL, K>, p);
+  launch_clusters(gather_kernel<T, AL, K>, (unsigned)(groups * nr), (unsigned)nr, dim3(kThreads), smem, l.stream, p);
   return check_launch();
 }
 // Where one launch by clusters is the faster way: up to a matrix size (of the whole square, where a triangle is read).

@@ -640,7 +640,7 @@ static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, co
     const int64_t nvec = (n - head) / V;
     const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV);
     if (nchunks > 1 && nchunks <= kClusterChunks) {
-      launch_one_cluster(l1_reduce_unit<T, Op, NV>, cluster_blocks(nchunks), dim3(kThreads), l.stream, x, Op::RY ? y : x, n, head, nvec, nchunks, partials,
+      launch_clusters(l1_reduce_unit<T, Op, NV>, cluster_blocks(nchunks), cluster_blocks(nchunks), dim3(kThreads), 0, l.stream, x, Op::RY ? y : x, n, head, nvec, nchunks, partials,
                          ticket, result);
       return check_launch();
     }
@@ -657,7 +657,7 @@ static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, co
     const int64_t nvec = (span - head) / V;
     const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV);
     if (nchunks > 1 && nchunks <= kClusterChunks) {
-      launch_one_cluster(l1_reduce_unit<T, Op, NV, 2>, cluster_blocks(nchunks), dim3(kThreads), l.stream, x, Op::RY ? y : x, span, head, nvec, nchunks,
+      launch_clusters(l1_reduce_unit<T, Op, NV, 2>, cluster_blocks(nchunks), cluster_blocks(nchunks), dim3(kThreads), 0, l.stream, x, Op::RY ? y : x, span, head, nvec, nchunks,
                          partials, ticket, result);
       return check_launch();
     }

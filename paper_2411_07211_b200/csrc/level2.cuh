@@ -567,16 +567,7 @@ struct L2Plan {
 template <typename T, class K, int SLICES>
 static void launch_finalize(const Launch& l, const L2Args<T>& args, int RB, int TC, int64_t nout, int SH = 0) {
   constexpr int OUTB = kThreads / SLICES;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((nout + OUTB - 1) / OUTB));
-  cfg.blockDim = dim3(kThreads);
-  cfg.stream = l.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = knob(kKnobUsePdl) ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, l2_finalize<T, K, SLICES>, args, RB, TC, SH);
+  launch_chained(l2_finalize<T, K, SLICES>, dim3((unsigned)((nout + OUTB - 1) / OUTB)), dim3(kThreads), 0, l.stream, args, RB, TC, SH);
 }
 
 // Launches the tile kernel (+ finalize when partials are needed) for one shape.

@@ -547,16 +547,7 @@ static int tri_tile_run_cap(const Launch& l, const T* a, int64_t lda, int64_t n,
   const int grid = nunits < sm_count() * kBlocksPerSm ? nunits : sm_count() * kBlocksPerSm;
   launch_chained(kern, dim3(grid), dim3(kThreads), smem, l.stream, args, tmap);
   if (int st = check_launch()) return st;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + 31) / 32));
-  cfg.blockDim = dim3(fin_warps<T>() * 32);
-  cfg.stream = l.stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = knob(kKnobUsePdl) ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, tri_tile_finalize<T, CAP, ROW, COL, TRI>, args);
+  launch_chained(tri_tile_finalize<T, CAP, ROW, COL, TRI>, dim3((unsigned)((n + 31) / 32)), dim3(fin_warps<T>() * 32), 0, l.stream, args);
   return check_launch();
 }
 

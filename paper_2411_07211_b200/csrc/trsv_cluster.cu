@@ -806,20 +806,7 @@ static int launch_cluster(const Launch& l, Args<T>& p, size_t tagged_bytes, bool
   if (strips > kStrips * p.H && cap != 0) return B2_STATUS_OK;  // (no streaming blocks at all: a test's choice)
   *handled = true;
   if (int st = trsv_forget_if_captured(l, tagged_bytes)) return st;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = kCS;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3((unsigned)(1 + streams) * kCS);
-  cfg.blockDim = dim3(kCT);
-  cfg.dynamicSmemBytes = Smem<T>::TOTAL;
-  cfg.stream = l.stream;
-  cfg.attrs = at;
-  cfg.numAttrs = knob(kKnobUsePdl) ? 2 : 1;
-  (void)cudaLaunchKernelEx(&cfg, trsv_cluster_kernel<T, COLTYPE, AL>, p);
+  launch_clusters(trsv_cluster_kernel<T, COLTYPE, AL>, (unsigned)((1 + streams) * kCS), (unsigned)kCS, dim3(kCT), Smem<T>::TOTAL, l.stream, p);
   return check_launch();
 }
 

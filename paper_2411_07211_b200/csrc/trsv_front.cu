@@ -76,11 +76,6 @@ __device__ __forceinline__ void ld_word2(const unsigned long long* p, unsigned l
 }
 // Thread-block cluster pieces: rank, cluster-wide barrier, address of a peer's shared memory,
 // (predicated) stores into it.
-__device__ __forceinline__ unsigned cluster_rank() {
-  unsigned r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ void cluster_sync_all() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
