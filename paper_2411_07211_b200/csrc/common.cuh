@@ -384,6 +384,7 @@ static void dbg_collect_this_unit(unsigned long long* out) {
   const DbgReport zero = {};
   cudaMemcpyToSymbol(g_dbg_report, &zero, sizeof(zero));
 }
+static __global__ void dbg_set_table(DbgTable t) { g_dbg_table = t; }
 static void dbg_commit(Launch& l) {
   static bool registered = false;  // (one flag per translation unit, like the device symbols)
   if (!registered) {
@@ -395,7 +396,7 @@ static void dbg_commit(Launch& l) {
   for (int i = 0; i < l.dbg_n && i < 8; ++i) t.lo[i] = l.dbg_lo[i], t.hi[i] = l.dbg_hi[i];
   t.n = l.dbg_n < 8 ? l.dbg_n : 8;
   t.shrink = dbg_shrink();
-  cudaMemcpyToSymbolAsync(g_dbg_table, &t, sizeof(t), 0, cudaMemcpyHostToDevice, l.stream);
+  dbg_set_table<<<1, 1, 0, l.stream>>>(t);  // (by value: a captured copy would read this stack frame on every replay)
   --l.dbg_n;  // (a second commit of the same call adds the workspace again)
 }
 #define B2_DBG_VEC(l, p, n, inc) ::b2::dbg_vec(l, p, n, inc)
