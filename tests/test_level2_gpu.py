@@ -228,9 +228,9 @@ def test_trsv_bounded_wait_reports_timeout(b2):
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("front,cluster,pm_from", [(0, 0, 16), (2, 0, 0), (2, 0, 5), (2, 2, 0), (2, 2, 3)])
 def test_trsv_every_kernel_choice(b2, ctx, dtype, front, cluster, pm_from):
-    """trsv has three code paths (block-row kernel; sub-block kernel block by block; sub-block
-    kernel in clusters), and the sub-block kernel premultiplies the last tile of a block row from
-    a given row on.  The defaults pick one per precision and view; here each is forced for every
+    """Behind the cluster kernel trsv has three more code paths (block-row kernel; sub-block kernel block by block;
+    sub-block kernel in clusters), and the sub-block kernel premultiplies the last tile of a block row from
+    a given row on.  Workspaces too small for the cluster kernel reach them; here each is forced for every
     view, on sizes with a ragged last block and more block rows than one cluster holds, with the
     premultiplied tile starting at the first row and inside the matrix."""
     old = (b2.get_tuning(b2.KNOB_TRSV_FRONT), b2.get_tuning(b2.KNOB_TRSV_CLUSTER), b2.get_tuning(b2.KNOB_TRSV_PM_FROM))
