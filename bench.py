@@ -14,6 +14,7 @@ the last line of stdout; the per-variant rows go to a table file (--table).
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import math
 import os
@@ -31,13 +32,24 @@ FALLBACK_PEAK_GBS = 6650.0
 NOMINAL_PEAK_GBS = 8000.0  # the vendor's spec-sheet HBM3e figure for this part (second denominator)
 
 
+def kernel_digest(files) -> str:
+    """Of the sources (names under csrc/) that hold a kernel."""
+    h = hashlib.sha256()
+    for name in files:
+        with open(os.path.join(ROOT, "paper_2411_07211_b200", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def ncu_dram_bytes_per_launch():
     """dram__bytes_read.sum + dram__bytes_write.sum per launch of each kernel template at the
-    bench sizes, as recorded beside the ncu summaries (one entry per kernel family; null once a
-    kernel has changed and its counters have not been retaken)."""
+    bench sizes, as recorded beside the ncu summaries: one entry per kernel family, with the digest
+    of its sources at the capture.  A family whose sources have changed since is left out: its
+    counters have not been retaken."""
     try:
         with open(os.path.join(ROOT, "profiles", "ncu_dram_bytes_per_launch.json")) as f:
-            return json.load(f)["bytes_per_launch"]
+            rows = json.load(f)["families"]
+        return {k: v["bytes_per_launch"] for k, v in rows.items() if v["digest"] == kernel_digest(v["sources"])}
     except Exception:
         return {}
 

@@ -111,3 +111,32 @@ def test_clock_summary_windows():
     out = bench.ClockSampler.summarise(lines, t_load=0.9, t0=2.12, t1=2.2)  # one sample inside: widen
     assert out["samples"] == 6 and out["window"].startswith("warm-up") and out["sm_mhz"] == 1965
     assert bench.ClockSampler.summarise([], None, None, None)["sm_mhz"] is None
+
+
+def test_traffic_is_reported_for_the_captured_kernel_only(tmp_path, monkeypatch):
+    """An entry counts while the sources of its kernel are those of the capture, and not after."""
+    import json
+    prof = tmp_path / "profiles"
+    csrc = tmp_path / "paper_2411_07211_b200" / "csrc"
+    prof.mkdir()
+    csrc.mkdir(parents=True)
+    (csrc / "k.cu").write_text("kernel")
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    assert bench.ncu_dram_bytes_per_launch() == {}
+    row = {"kernel": "k", "sources": ["k.cu"], "digest": bench.kernel_digest(["k.cu"]), "bytes_per_launch": 5.0}
+    (prof / "ncu_dram_bytes_per_launch.json").write_text(json.dumps({"families": {"trsv": row}}))
+    assert bench.ncu_dram_bytes_per_launch() == {"trsv": 5.0}
+    (csrc / "k.cu").write_text("another kernel")
+    assert bench.ncu_dram_bytes_per_launch() == {}
+
+
+def test_recorded_traffic_names_the_kernels_that_run():
+    """Each recorded family names a kernel that its listed sources define."""
+    import json
+    import re
+    with open(os.path.join(ROOT, "profiles", "ncu_dram_bytes_per_launch.json")) as f:
+        rows = json.load(f)["families"]
+    assert set(rows) <= {sp["family"] for sp in bench.variant_specs()}
+    for fam, row in rows.items():
+        text = "".join(open(os.path.join(ROOT, "paper_2411_07211_b200", "csrc", n)).read() for n in row["sources"])
+        assert re.search(r"__global__[^;{]*\b%s\(" % row["kernel"], text), (fam, row["kernel"])
