@@ -781,7 +781,7 @@ def main():
     ap.add_argument("--configs", action="store_true", help="time the size sweeps beside the headline set (rows go "
                                                            "to the table file; --filter selects among them)")
     ap.add_argument("--table", default=None, help="where the per-variant table (JSON) is written "
-                                                  "(default: bench_table.json in the run's output folder)")
+                                                  "(default: build/bench_table.json, or build/bench_configs_table.json)")
     args = ap.parse_args()
     if args.impl == "reference":
         reference_arm(args)
@@ -809,7 +809,7 @@ def main():
         peak, peak_src = peak_gbs()
         table = configs_leg(device, peak, max(5, min(args.steps, 10)), args.filter)
         table["peak_gbs"], table["peak_source"] = peak, peak_src
-        path = args.table or os.path.join(ROOT, "gpurun_out", "bench_configs_table.json")
+        path = args.table or os.path.join(ROOT, "build", "bench_configs_table.json")
         os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
         with open(path, "w") as f:
             json.dump(table, f, indent=1)
@@ -934,7 +934,7 @@ def main():
     if world == 1 and not args.filter:
         table["next_rows"] = next_rows_leg(wl, min(args.steps, 10), peak)
         out["next_rows_geomean_frac"] = table["next_rows"]["geomean_frac"]
-    path = args.table or os.path.join(ROOT, "gpurun_out", "bench_table.json")
+    path = args.table or os.path.join(ROOT, "build", "bench_table.json")
     os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
     with open(path, "w") as f:
         json.dump(table, f, indent=1)
