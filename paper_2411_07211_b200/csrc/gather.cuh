@@ -359,20 +359,25 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_l
 //   symv            reads its elements twice: float 20 MB 7.9 / 7.6, 24 7.9 / 9.3 (between 6 and 20 within 5 %); double 20
 //                   7.6 / 6.5, 24 7.5 / 7.6; unaligned (both triangles) float 21 MB 20.5 / 19.3, 23 20.5 / 20.5, 29 21.4 / 23.5, 35
 //                   23.0 / 26.6, double 29 22.8 / 19.0, 32 23.1 / 23.0, 35 23.8 / 24.8, 72 32.3 / 35.0.
+// room: whether the tile kernels' partials fit the workspace without much longer blocks; where they do not, this kernel, which
+// needs none or one vector, goes on off 16-byte boundaries (64 KB of scratch, us, tile kernel / this one: trmv in float n = 3001 32.9 / 13.2,
+// 4001 58.8 / 15.6, double 3001 75.0 / 13.0; symv in float n = 2501 with 264 KB 20.6 / 10.5, 3501 with 464 38.5 / 15.7, with less none).
 template <typename T, class K>
-constexpr int64_t max_mb(bool al) {
+constexpr int64_t max_mb(bool al, bool room) {
   constexpr bool F = sizeof(T) == 4;
+  if (!al && !room && K::SYM) return F ? 85 : 80;
+  if (!al && !room && K::TRI != TRI_FULL) return F ? 85 : 101;
   if (K::SYM) return al ? (F ? 20 : 22) : (F ? 23 : 33);
   if (K::TRI != TRI_FULL) return al ? (F ? 5 : 18) : (F ? 50 : 170);
   if (K::ROWOUT) return al ? (F ? 24 : 50) : 110;
   return al ? (F ? 17 : 22) : (F ? 35 : 70);
 }
 template <typename T, class K>
-static int run(const Launch& l, const L2Args<T>& q, bool* handled, bool one_launch = false) {
+static int run(const Launch& l, const L2Args<T>& q, bool* handled, bool one_launch = false, bool room = true) {
   *handled = false;
   if (knob(kKnobGather) == 0) return B2_STATUS_OK;
   const bool al = aligned_to(q.a, 16) && q.lda % VecLen<T>::value == 0;
-  if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)max_mb<T, K>(al) * 1e6) return B2_STATUS_OK;
+  if (knob(kKnobGather) < 2 && (double)q.rows * (double)q.cols * sizeof(T) > (double)max_mb<T, K>(al, room) * 1e6) return B2_STATUS_OK;
   return al ? launch<T, true, K>(l, q, handled, one_launch) : launch<T, false, K>(l, q, handled, one_launch);
 }
 

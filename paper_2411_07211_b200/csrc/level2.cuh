@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(kThreads) l2_scale_y(T* y, int64_t incy, int64
 // ------------------------------------------------------------------------------- host side
 struct L2Plan {
   int shape;             // index into the shape table
-  int tile_cols = 0;     // columns of a column tile (row-dot plans)
+  int tile_cols;         // columns of a column tile
   int64_t rows_per_cta;  // multiple of the shape's RB
   int ctiles_per_cta;
 };
@@ -740,6 +740,7 @@ static L2Plan plan_colout(const L2Args<T>& a, bool narrow_ok, int64_t rows_per_c
   p.shape = (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
   // element-wise rows (not 16-byte aligned): a 32-element column tile makes tiny blocks, take 128
   if (V == 1 && nv >= 128) p.shape = SHAPE_WIDE;
+  p.tile_cols = shape_packs_per_row(p.shape) * V;
   p.ctiles_per_cta = 1;
   if ((a.rows + rows_per_cta - 1) / rows_per_cta > 1024) rows_per_cta = (a.rows + 1023) / 1024;
   p.rows_per_cta = rows_per_cta;

@@ -44,8 +44,18 @@ static L2Plan plan_tri(const L2Args<T>& a) {
   L2Plan p;
   p.shape = (nv >= 512 && !l2_shift(a, true, 0) && knob(kKnobTriWide)) ? SHAPE_WIDE : SHAPE_MID;
   p.ctiles_per_cta = 1;
-  p.rows_per_cta = tri_rows(a, shape_packs_per_row(p.shape) * V);
+  p.tile_cols = shape_packs_per_row(p.shape) * V;
+  p.rows_per_cta = tri_rows(a, p.tile_cols);
   return p;
+}
+
+// Whether the workspace holds the partials of a kind with column sums (sym: row sums too) in blocks of up to twice the planned
+// rows.  (With 800 KB symv in float n = 3501 takes 13.7 us so, 15.7 in the gather kernel; twice as long again 17.8 / 17.8 at 4001.)
+template <typename T>
+static bool tri_room(const Launch& l, const L2Args<T>& a, const L2Plan& p, bool sym) {
+  const int64_t tiles = (a.cols + p.tile_cols - 1) / p.tile_cols, bands = (a.rows + 2 * p.rows_per_cta - 1) / (2 * p.rows_per_cta);
+  const int64_t spill = l2_shift(a, sym, 0) ? bands * (tiles + 1) * (VecLen<T>::value - 1) : 0;
+  return (size_t)(((sym ? tiles : 0) + bands) * a.cols + spill) * sizeof(T) + 512 <= l.scratch_bytes;
 }
 
 template <typename T>
@@ -77,10 +87,12 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
   args.incy = incy;
   // the stored triangle as it sits in the row-major view of the buffer
   const bool upper = (order == B2_ROW_MAJOR) == (uplo == B2_UPPER);
+  const L2Plan plan = plan_tri(args);
   if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {  // (a forced tile kernel stays forced)
     bool handled = false;
-    const int st = upper ? ga::run<T, Kind<true, true, TRI_UPPER, false, true>>(l, args, &handled)
-                         : ga::run<T, Kind<true, true, TRI_LOWER, false, true>>(l, args, &handled);
+    const bool room = tri_room(l, args, plan, true);
+    const int st = upper ? ga::run<T, Kind<true, true, TRI_UPPER, false, true>>(l, args, &handled, false, room)
+                         : ga::run<T, Kind<true, true, TRI_LOWER, false, true>>(l, args, &handled, false, room);
     if (handled) return st;
   }
   // The tile kernel with the shared-memory ring (16-byte aligned matrices) is the faster one while the triangle is small:
@@ -97,17 +109,21 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
                                                                                   args.y, incy, &handled);
     if (handled) return st;
   }
-  const L2Plan plan = plan_tri(args);
   if (upper) return l2_dispatch<T, Kind<true, true, TRI_UPPER, false, true>, false>(l, args, plan, false);
   return l2_dispatch<T, Kind<true, true, TRI_LOWER, false, true>, false>(l, args, plan, false);
 }
 
 template <typename T, bool ROW, int TRI>
 static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
+  // (column tiles of 128 elements, of 64 in double on aligned matrices: plan_colout)
+  const bool narrow = sizeof(T) == 8 && aligned_to(args.a, 16) && args.lda % VecLen<T>::value == 0;
+  const L2Plan plan = ROW ? plan_rowout(args, false, kShortRowsTrmv) : plan_colout(args, false, tri_rows(args, narrow ? 64 : 128));
   if constexpr (!ROW) {
     if (knob(kKnobTriTile) == 1 || knob(kKnobGather) >= 2) {
       bool handled = false;
-      const int st = unit ? ga::run<T, Kind<false, true, TRI, true, false>>(l, args, &handled) : ga::run<T, Kind<false, true, TRI, false, false>>(l, args, &handled);
+      const bool room = tri_room(l, args, plan, false);
+      const int st = unit ? ga::run<T, Kind<false, true, TRI, true, false>>(l, args, &handled, false, room)
+                          : ga::run<T, Kind<false, true, TRI, false, false>>(l, args, &handled, false, room);
       if (handled) return st;
     }
   }
@@ -123,9 +139,6 @@ static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
                                                                 args.y, args.incy, &handled);
     if (handled) return st;
   }
-  // (column tiles of 128 elements, of 64 in double on aligned matrices: plan_colout)
-  const bool narrow = sizeof(T) == 8 && aligned_to(args.a, 16) && args.lda % VecLen<T>::value == 0;
-  const L2Plan plan = ROW ? plan_rowout(args, false, kShortRowsTrmv) : plan_colout(args, false, tri_rows(args, narrow ? 64 : 128));
   if (unit) return l2_dispatch<T, Kind<ROW, !ROW, TRI, true, false>, false>(l, args, plan, false);
   return l2_dispatch<T, Kind<ROW, !ROW, TRI, false, false>, false>(l, args, plan, false);
 }

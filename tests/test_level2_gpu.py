@@ -423,6 +423,34 @@ def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("extra", [0, 400 << 10])
+def test_small_workspace_off_boundaries(b2, dtype, extra):
+    """symv and trmv's column sums with the smallest workspace and with a little more, off 16-byte boundaries, at sizes where
+    the tile kernels' partials would need more, up to the largest that the gather kernel takes; the next one is refused."""
+    small = b2.Context(workspace_bytes=b2.lib().b2_workspace_min_bytes() + extra)
+    small.reset()
+    for n in (2401, 3001, 4001, 4601) if dtype == np.float32 else (2043, 2501, 3101):
+        x, y = synth.vector_np(7, n, n, dtype), synth.vector_np(8, n, n, dtype)
+        for uplo in UPLOS:
+            a = tri_buf(26, n, n, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+            ga, gx, gy = Guarded(a), Guarded(x), Guarded(y)
+            b2.symv(small, orc.ROW_MAJOR, uplo, n, 1.25, ga.t, n, gx.t, 1, 0.5, gy.t, 1)
+            oy = y.copy()
+            absterms = orc.symv(orc.ROW_MAJOR, uplo, n, dtype(1.25), a, n, x, 1, dtype(0.5), oy, 1)
+            assert_close(gy.host(), oy, absterms, dtype, f"symv {n} {uplo}")
+            b2.trmv(small, orc.ROW_MAJOR, uplo, orc.TRANS, orc.NON_UNIT, n, ga.t, n, gx.t, 1)
+            ox = x.copy()
+            absterms = orc.trmv(orc.ROW_MAJOR, uplo, orc.TRANS, orc.NON_UNIT, n, a, n, ox, 1)
+            assert_close(gx.host(), ox, absterms, dtype, f"trmv {n} {uplo}")
+            gx.check_guards(), gy.check_guards()
+    n = 4701 if dtype == np.float32 else 3201
+    a, v = torch.zeros(n * n, dtype=torch.from_numpy(y).dtype, device="cuda"), torch.from_numpy(np.resize(y, n)).cuda()
+    with pytest.raises(b2.B2Error) as e:
+        b2.symv(small, orc.ROW_MAJOR, orc.UPPER, n, 1.25, a, n, v, 1, 0.5, v.clone(), 1)
+    assert e.value.status == b2.STATUS_WORKSPACE_TOO_SMALL
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2)])
 def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
     """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, the last one cut."""
