@@ -451,6 +451,33 @@ def test_small_workspace_off_boundaries(b2, dtype, extra):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n", [8, 77, 300])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 90, 2.0 ** -90])
+def test_trsv_divides_by_the_diagonal(b2, ctx, dtype, n, scale):
+    """Multiples of the diagonal below ones in every eighth row, right-hand side one there and else zero: the solution is the
+    negated factors and exact, for each unknown is one quotient of whole numbers.  The product with a rounded reciprocal is
+    not that quotient for many of the divisors (49 in double, 41 in float).  Scaled also by powers of two beyond the range in
+    which such a product is corrected."""
+    a = np.zeros((n, n), dtype=dtype)
+    want = np.zeros(n, dtype=dtype)
+    for i in range(n):
+        one = i % 8 == 0
+        a[i, i] = 1 if one else (2 * i + 27) * scale
+        want[i] = 1 if one else -(i % 5)
+        if not one:
+            a[i, i - i % 8] = -want[i] * a[i, i]
+    hx = np.where(np.arange(n) % 8 == 0, 1, 0).astype(dtype)
+    for lda in (n + n % 2 * 3, n | 1):  # on and off 16-byte boundaries
+        for uplo, trans, view in ((orc.LOWER, orc.NO_TRANS, a), (orc.UPPER, orc.TRANS, a.T)):
+            buf = np.full((n, lda), np.nan, dtype=dtype)
+            buf[:, :n] = view
+            gm, gx = Guarded(buf), Guarded(hx)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, gm.t, lda, gx.t, 1)
+            assert ctx.device_status() == 0
+            assert np.array_equal(gx.host(), want), (lda, uplo, trans)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2)])
 def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
     """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, the last one cut."""
