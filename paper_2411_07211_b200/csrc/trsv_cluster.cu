@@ -218,6 +218,17 @@ __device__ __forceinline__ void add_to(T (&acc)[kStrips][Strip<T, COLTYPE>::NA],
   }
 }
 
+// Diagonal block I once more, from the matrix (cold path; all copies of this thread that are in flight are waited for).
+template <typename T, bool COLTYPE, bool AL>
+__device__ __noinline__ void invert_again(const Args<T>& p, unsigned s_off, int I, int tid) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  T* const S = reinterpret_cast<T*>(smem_raw + s_off);
+  Diag<T, COLTYPE, AL>::stage(p.a, p.lda, p.n, I, p.backward, S, tid);
+  cp_async_wait<0>();
+  bar_block();
+  invert_rows<T>(S, p.unit, block_len(p, I), tid);
+}
+
 // ---- streaming block -----------------------------------------------------------------------------------
 template <typename T, bool COLTYPE, bool AL>
 __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int h) {
@@ -313,7 +324,7 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
       cp_async_wait<0>();
     }
     bar_block();
-    invert_block<T>(smem_off(M), smem_off(b.red), p.unit, block_len(p, I), b.tid);
+    if (invert_block<T>(smem_off(M), smem_off(b.red), p.unit, block_len(p, I), b.tid)) invert_again<T, COLTYPE, AL>(p, smem_off(M), I, b.tid);
     T* dst = p.winv + (int64_t)(k - kCS) * NB * NB;
 #pragma unroll 2
     for (int idx = b.tid; idx < NB * NB / V; idx += kCT) {
@@ -730,7 +741,8 @@ __device__ __forceinline__ unsigned solve_block(const Args<T>& p, Block<T>& b, i
   };
   auto invert = [&](int k) {
     bar_block();
-    invert_block<T>(smem_off(S), smem_off(b.red), p.unit, block_len(p, mem_block(p, k)), b.tid);
+    const int I = mem_block(p, k);
+    if (invert_block<T>(smem_off(S), smem_off(b.red), p.unit, block_len(p, I), b.tid)) invert_again<T, COLTYPE, AL>(p, smem_off(S), I, b.tid);
   };
   auto stage = [&](int k) { Diag<T, COLTYPE, AL>::stage(p.a, p.lda, p.n, mem_block(p, k), p.backward, S, b.tid); };
 

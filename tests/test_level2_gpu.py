@@ -478,6 +478,32 @@ def test_trsv_divides_by_the_diagonal(b2, ctx, dtype, n, scale):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, bad):
+    """An infinite or NaN element of the matrix in a diagonal block: the unknowns that the solve reaches before it do not depend
+    on it.  The element lies beside the diagonal, on it, and in the lower left part of a block of every level of the
+    inversion; in a whole block, in one that the streaming blocks invert and in the ragged last one."""
+    nb = 128 if dtype == np.float32 else 64
+    n = 18 * nb + 44
+    places = [(1, 0), (3, 1), (7, 0), (7, 6), (7, 7), (12, 3), (15, 2), (23, 16), (30, 9), (39, 37), (45, 45), (63, 1), (61, 35)]
+    if nb == 128:
+        places += [(76, 65), (99, 10), (100, 63), (127, 64), (127, 127)]
+    for block, length, where in ((1, nb, places), (17, nb, places[3::4]), (18, 44, [(43, 40), (20, 3), (43, 43)])):
+        for (row, col), uplo, trans in itertools.product(where, UPLOS, TRANSES):
+            upper = (uplo == orc.UPPER) == (trans == orc.NO_TRANS)  # of op(A): solved from the last row on
+            i, j = (block * nb + (length - 1 - q if upper else q) for q in (row, col))
+            a = tri_buf(24, n, n, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+            a.reshape(n, n)[(i, j) if trans == orc.NO_TRANS else (j, i)] = bad
+            hx = synth.vector_np(9, n, n, dtype)
+            ga, gx = Guarded(a), Guarded(hx)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n, gx.t, 1)
+            assert ctx.device_status() == 0
+            resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n, hx, 1, gx.host(), 1)
+            before = slice(i + 1, n) if upper else slice(0, i)
+            assert np.all(resid[before] <= TOL[np.dtype(dtype)] * scale[before]), (block, row, col, uplo, trans)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2)])
 def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
     """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, the last one cut."""
