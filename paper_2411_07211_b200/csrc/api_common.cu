@@ -26,6 +26,7 @@ static int64_t g_knobs[kKnobCount] = {
     /* kKnobTriBulk         */ 0,
     /* kKnobTrsvStreams     */ -1,
     /* kKnobGather          */ 1,
+    /* kKnobTrsvDebugLate   */ 0,
 };
 
 unsigned long long g_launch_count = 0;

@@ -434,7 +434,8 @@ enum Knob {
   kKnobTriBulk = 15,           // tile kernel with the shared-memory ring: 1 = a tile arrives as one tiled TMA copy (measured equal to the 16-byte copies; off by default)
   kKnobTrsvStreams = 16,       // streaming clusters of the cluster trsv kernel at most (-1: as many as fit)
   kKnobGather = 17,            // gemv / symv / trmv by one cluster per 32 outputs: 0 never, 1 where it is the faster kernel, 2 wherever it can, 3 the same with trmv's late outputs forced
-  kKnobCount = 18
+  kKnobTrsvDebugLate = 18,     // test hook: polls for which the first cluster of the cluster trsv kernel waits to be overtaken (0 = none)
+  kKnobCount = 19
 };
 int64_t knob(int id);
 

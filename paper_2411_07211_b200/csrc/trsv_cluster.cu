@@ -56,6 +56,9 @@ constexpr int kStrip = 32;      // rows of op(A) in a strip
 constexpr int kDepth = 6;       // slots of a streaming block's ring, two tiles (32 KB) each
 constexpr int kStrips = 12;     // strips per streaming block at most
 constexpr int kTilePacks = 4;   // packs of a strip's tile per thread
+// Polls of the first cluster's ticket before another cluster draws one.  (A copy and two solves with 64 / without, us: float n = 1001
+// 49.0 / 50.8, 3001 83.8 / 87.0, 11520 216 / 212, 16383 612 / 621, double 1024 42.5 / 44.2, 3001 105.8 / 100.5, 8192 225 / 220.)
+constexpr int kHeadStart = 64;
 
 template <typename T>
 struct Args {
@@ -75,6 +78,7 @@ struct Args {
   u64 wait_limit;
   int* device_status;
   int debug_skip;
+  int debug_late;  // test hook: polls for which the first cluster lets another one draw the first ticket
 };
 
 // Shared memory: one region that is the solving block's near-tile ring and inversion scratch or the
@@ -461,8 +465,8 @@ __device__ __forceinline__ void draw_ticket(const Args<T>& p, unsigned* ticket, 
   unsigned t = 0xffffffffu;
   // The first cluster, whose blocks start as solving ones, is let go first; if it has not started after a while, another
   // one solves.
-  if (!early)
-    for (int i = 0; i < 64 && ld_flag(p.ctl + kCtlTrsvTicket) == 0u; ++i) {}
+  const int polls = early ? p.debug_late : kHeadStart;
+  for (int i = 0; i < polls && ld_flag(p.ctl + kCtlTrsvTicket) == 0u; ++i) {}
   // (abort word up: left by an earlier timed-out call on a workspace that was not reset, or raised
   // meanwhile: nothing is solved, and the caller must be able to see that)
   if (ld_flag(p.ctl + kCtlTrsvAbort) == 0u) t = atomicAdd(p.ctl + kCtlTrsvTicket, 1u);
@@ -957,6 +961,7 @@ int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, in
   p.wait_limit = l.wait_limit;
   p.device_status = l.device_status;
   p.debug_skip = (int)knob(kKnobTrsvDebugSkip);
+  p.debug_late = (int)knob(kKnobTrsvDebugLate);
 #ifdef B2_DEBUG_BOUNDS
   {  // (this translation unit has its own copy of the range table)
     Launch lc = l;

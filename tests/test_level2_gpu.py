@@ -504,6 +504,31 @@ def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, bad):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("streams", [-1, 1])
+def test_trsv_first_cluster_overtaken(b2, ctx, dtype, streams):
+    """The first cluster, whose blocks have staged their diagonal blocks by then, draws a ticket other than the first and
+    streams: with fewer block rows than blocks in a cluster, with more, ragged, on and off 16-byte boundaries."""
+    nb, near = (128, 4) if dtype == np.float32 else (64, 6)
+    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
+    b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 1 << 16)  # (polls; the other clusters draw their tickets within a hundred)
+    try:
+        for n, pad in [((near + 3) * nb, 0), ((near + 4) * nb + 1, 0), (18 * nb + 4, 0), (21 * nb + 3, 2)]:
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                a = tri_buf(25, n, n + pad, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+                hx = synth.vector_np(9, n, n, dtype)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                assert ctx.device_status() == 0
+                gx.check_guards()
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n + pad, hx, 1, gx.host(), 1)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
+        b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 0)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2)])
 def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
     """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, the last one cut."""
