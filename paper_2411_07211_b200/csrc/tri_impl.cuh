@@ -22,8 +22,8 @@ static int check_square(int order, int64_t n, const T* a, int64_t lda, int arg_o
   return 0;
 }
 
-// Rows per block of the kinds with column sums: about 480 blocks that hold any of the triangle, three or four for each SM, as
-// long as they keep 64 rows; longer blocks where the matrix is larger, up to what measured fastest (a block is a sequence of
+// Rows per block of the kinds with column sums: 3 1/4 blocks for each SM (480) that hold any of the triangle, as long as they
+// keep 64 rows; longer blocks where the matrix is larger, up to what measured fastest (a block is a sequence of
 // steps; off 16-byte boundaries, where a step takes longer, the last blocks are waited for longer).  Us, with 512 rows for
 // all / with this rule: symv in float n = 4944 32.3 / 29.6, 4945 51.5 / 35.7, 6001 57.9 / 43.8, 9934 by columns 94 / 84, in double
 // 3473 39.7 / 32.4; a copy and both products of trmv in double n = 3581 33.4 / 27.2, 3580 27.5 / 25.7, 11001 163 / 158; the same
@@ -33,7 +33,7 @@ static int64_t tri_rows(const L2Args<T>& a, int tile_cols) {
   if (const int64_t k = knob(kKnobTriRows)) return k;
   const bool aligned = aligned_to(a.a, 16) && a.lda % VecLen<T>::value == 0;
   const int64_t most = !aligned ? 256 : sizeof(T) == 4 ? 512 : 384;
-  const double rows = (double)a.rows * (double)a.cols / (2.0 * tile_cols * 480);
+  const double rows = (double)a.rows * (double)a.cols / (2.0 * tile_cols * 3.25 * sm_count());
   return rows > (double)most ? most : std::min(most, std::max<int64_t>(64, (int64_t)(rows + 32) / 64 * 64));
 }
 
