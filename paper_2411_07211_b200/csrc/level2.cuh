@@ -631,11 +631,12 @@ using ShapeWide4 = Shape<32, 4, 4>;   // the same, 32 rows per step
 using ShapeMid = Shape<32, 1, 8>;     // 512 B row segments, 64 rows per step
 using ShapeHalf = Shape<16, 1, 8>;    // 256 B row segments, 128 rows per step
 using ShapeQuarter = Shape<8, 1, 8>;  // 128 B row segments, 256 rows per step
-enum { SHAPE_WIDE = 0, SHAPE_MID = 1, SHAPE_HALF = 2, SHAPE_QUARTER = 3 };
+enum { SHAPE_WIDE = 0, SHAPE_MID = 1, SHAPE_HALF = 2, SHAPE_QUARTER = 3, SHAPE_WIDE4 = 4 };
 
 inline int shape_rb(int shape) {
   switch (shape) {
     case SHAPE_WIDE: return ShapeWide::RB;
+    case SHAPE_WIDE4: return ShapeWide4::RB;
     case SHAPE_MID: return ShapeMid::RB;
     case SHAPE_HALF: return ShapeHalf::RB;
     default: return ShapeQuarter::RB;
@@ -643,25 +644,30 @@ inline int shape_rb(int shape) {
 }
 inline int shape_packs_per_row(int shape) {  // packs of one row segment
   switch (shape) {
-    case SHAPE_WIDE: return 128;
+    case SHAPE_WIDE:
+    case SHAPE_WIDE4: return 128;
     case SHAPE_MID: return 32;
     case SHAPE_HALF: return 16;
     default: return 8;
   }
 }
 
+// The shape of gemv where rows are read element by element in wide segments.  In double such loads are half as wide, so a
+// thread has twice as many in flight, four rows instead of two (both products, us: 5003 x 3001 45.7 / 42.9, 3001 x 3001 29.4 /
+// 26.1, 757600 x 141 353 / 291, 8001 x 8001 164 / 155; row product 20001 x 1001 with blocks of 64 KB as everywhere 27.5, of 128 KB 29.4).  Small matrices and few rows need the shorter blocks (2001 x 1001
+// 11.4 / 12.5, 33 x 200001 25.9 / 26.5), and so does trmv (column sums n = 3581 26.4 / 27.2, row sums n = 1301 14.2 / 14.7).
 constexpr double kWide4Elems = 4e6;
 constexpr int64_t kWide4Rows = 1024;
+template <typename T>
+static int gemv_wide_shape(const L2Args<T>& a, int V) {
+  return V == 1 && sizeof(T) == 8 && a.rows >= kWide4Rows && (double)a.rows * (double)a.cols >= kWide4Elems ? SHAPE_WIDE4 : SHAPE_WIDE;
+}
 
 // NARROW = false drops the two narrow shapes (kinds that never use them compile faster).
 template <typename T, int V, class K, bool NARROW>
 static int l2_launch(const Launch& l, const L2Args<T>& args, const L2Plan& plan, bool allow_direct) {
-  // gemv in double off 16-byte boundaries: element loads are half as wide, so a thread has twice as many in flight, four
-  // rows instead of two (both products, us: 5003 x 3001 45.7 / 42.9, 3001 x 3001 29.4 / 26.1, 757600 x 141 353 / 291,
-  // 8001 x 8001 164 / 155).  Small matrices and few rows need the shorter blocks (2001 x 1001 11.4 / 12.5, 33 x 200001
-  // 25.9 / 26.5), and so does trmv (column sums n = 3581 26.4 / 27.2, row sums n = 1301 14.2 / 14.7).
   if constexpr (V == 1 && sizeof(T) == 8 && K::TRI == TRI_FULL) {
-    if (plan.shape == SHAPE_WIDE && args.rows >= kWide4Rows && (double)args.rows * (double)args.cols >= kWide4Elems)
+    if (plan.shape == SHAPE_WIDE4)
       return l2_launch_shape<T, V, K, ShapeWide4>(l, args, plan.rows_per_cta, plan.ctiles_per_cta, allow_direct);
   }
   if (plan.shape == SHAPE_WIDE)
@@ -714,9 +720,12 @@ static L2Plan plan_rowout(const L2Args<T>& a, bool narrow_ok, int short_rows) {
   L2Plan p;
   // (shifted packs: short segments, 4 x values for 8 packs instead of 16)
   p.shape = nv >= 128 && !shift ? SHAPE_WIDE : (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
+  if (narrow_ok && p.shape == SHAPE_WIDE) p.shape = gemv_wide_shape(a, V);
   const int64_t tile_bytes = (int64_t)shape_rb(p.shape) * shape_packs_per_row(p.shape) * V * sizeof(T);
   int64_t cpc = knob(kKnobGemvNTileBytes) / tile_bytes;
   if (cpc < 1) cpc = 1;
+  // (a row of up to 512 in one block, without a second pass: 12001 x 511 10.2 us, 11.5 in two, but 40001 x 301 19.7 and 19.0)
+  if (p.shape == SHAPE_WIDE4 && a.cols <= 2 * cpc * shape_packs_per_row(p.shape)) cpc *= 2;
   // A matrix of a few long rows (at most 8 row steps) would get one partial per column split
   // and a finalize pass that adds thousands of them per row: there the splits are limited to
   // about eight resident blocks per SM in all.
@@ -739,7 +748,7 @@ static L2Plan plan_colout(const L2Args<T>& a, bool narrow_ok, int64_t rows_per_c
   L2Plan p;
   p.shape = (nv > 16 || !narrow_ok) ? SHAPE_MID : nv > 8 ? SHAPE_HALF : SHAPE_QUARTER;
   // element-wise rows (not 16-byte aligned): a 32-element column tile makes tiny blocks, take 128
-  if (V == 1 && nv >= 128) p.shape = SHAPE_WIDE;
+  if (V == 1 && nv >= 128) p.shape = narrow_ok ? gemv_wide_shape(a, V) : SHAPE_WIDE;
   p.tile_cols = shape_packs_per_row(p.shape) * V;
   p.ctiles_per_cta = 1;
   if ((a.rows + rows_per_cta - 1) / rows_per_cta > 1024) rows_per_cta = (a.rows + 1023) / 1024;

@@ -557,16 +557,22 @@ def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
 
 @pytest.mark.parametrize("order", ORDERS)
 @pytest.mark.parametrize("trans", TRANSES)
-@pytest.mark.parametrize("m,n", [(1999, 2001), (2001, 2001), (1023, 4099), (1025, 3911), (31009, 129)])
+@pytest.mark.parametrize("m,n", [(1999, 2001), (2001, 2001), (1023, 4099), (1025, 3911), (31009, 129), (8009, 511), (7999, 513)])
 def test_gemv_double_unaligned_steps(b2, ctx, order, trans, m, n):
-    """gemv in double off 16-byte boundaries around the size from which a step has four rows instead of two per thread."""
+    """gemv in double off 16-byte boundaries around the size from which a step of the tile kernel has four rows instead of two
+    per thread, and where a block has a whole row and where it has not."""
     minor, major = (n, m) if order == orc.ROW_MAJOR else (m, n)
     lda = minor + 1 - minor % 2  # odd
     lenx, leny = (n, m) if trans == orc.NO_TRANS else (m, n)
     a = matbuf(m + n, major, minor, lda, np.float64)
     x, y = synth.vector_np(1, m + n, lenx, np.float64), synth.vector_np(2, m + n, leny, np.float64)
     ga, gx, gy = Guarded(a), Guarded(x), Guarded(y)
-    b2.gemv(ctx, order, trans, m, n, 1.25, ga.t, lda, gx.t, 1, 0.5, gy.t, 1)
+    old = b2.get_tuning(b2.KNOB_GATHER)
+    b2.set_tuning(b2.KNOB_GATHER, 0)
+    try:
+        b2.gemv(ctx, order, trans, m, n, 1.25, ga.t, lda, gx.t, 1, 0.5, gy.t, 1)
+    finally:
+        b2.set_tuning(b2.KNOB_GATHER, old)
     oy = y.copy()
     absterms = orc.gemv(order, trans, m, n, 1.25, a, lda, x, 1, 0.5, oy, 1)
     assert_close(gy.host(), oy, absterms, np.float64, f"gemv {m} {n} {order} {trans}")
