@@ -339,13 +339,16 @@ def test_cluster_gather_kernel(b2, ctx, dtype, mode):
 
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n,pad", [(63, 1), (130, 2), (513, 3), (516, 0), (641, 7), (1090, 2), (1151, 1), (1153, 0)])
-def test_cut_longest_column_tile(b2, ctx, dtype, n, pad):
+@pytest.mark.parametrize("rows", [512, 0])
+def test_cut_longest_column_tile(b2, ctx, dtype, n, pad, rows):
     """The tile kernels' column sums where the last column tile of an upper triangle (64 or 128 columns, the longest
     of them) is cut by the matrix edge: on a pack boundary, inside a pack, with one column and with all but one, in
-    blocks of 512 rows that lie above the diagonal whole, in part and not at all; rows on and off 16-byte boundaries."""
-    old = b2.get_tuning(b2.KNOB_GATHER), b2.get_tuning(b2.KNOB_TRI_TILE)
+    blocks of 512 rows that lie above the diagonal whole, in part and not at all, and of as many as the size asks for
+    (one step of 64); rows on and off 16-byte boundaries."""
+    old = b2.get_tuning(b2.KNOB_GATHER), b2.get_tuning(b2.KNOB_TRI_TILE), b2.get_tuning(b2.KNOB_TRI_ROWS)
     b2.set_tuning(b2.KNOB_GATHER, 0)
     b2.set_tuning(b2.KNOB_TRI_TILE, 0)
+    b2.set_tuning(b2.KNOB_TRI_ROWS, rows)
     try:
         for lda, diag, inc in ((n + pad, orc.NON_UNIT, 1), ((n + 7) // 4 * 4, orc.UNIT, 2)):
             x, y = synth.vector_np(7, n, n, dtype), synth.vector_np(8, n, n, dtype)
@@ -367,6 +370,7 @@ def test_cut_longest_column_tile(b2, ctx, dtype, n, pad):
     finally:
         b2.set_tuning(b2.KNOB_GATHER, old[0])
         b2.set_tuning(b2.KNOB_TRI_TILE, old[1])
+        b2.set_tuning(b2.KNOB_TRI_ROWS, old[2])
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
@@ -403,12 +407,14 @@ def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
 @pytest.mark.parametrize("streams", [-1, 1])
 def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
     """Solves whose strips end with the first and with the second tile of a pair (the streaming blocks take tiles in
-    pairs), whole and ragged, on and off 16-byte boundaries (one near row fewer in float)."""
+    pairs), whole and ragged, on and off 16-byte boundaries (one near row fewer in float); with one strip for each streaming
+    block and, on one cluster of them, with several."""
     nb, near = (128, 4) if dtype == np.float32 else (64, 6)
     old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
     b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
     try:
-        for n, pad in [((near + 2) * nb - 4, 0), ((near + 3) * nb, 0), ((near + 4) * nb + 4, 4), (near * nb + 1, 0), ((near + 3) * nb - 1, 2)]:
+        for n, pad in [((near + 2) * nb - 4, 0), ((near + 3) * nb, 0), ((near + 4) * nb + 4, 4), (near * nb + 1, 0), ((near + 3) * nb - 1, 2),
+                       ((near + 9) * nb, 0), ((near + 10) * nb + 4, 0)]:
             for uplo, trans in itertools.product(UPLOS, TRANSES):
                 a = tri_buf(23, n, n + pad, dtype, orc.COL_MAJOR, uplo, orc.NON_UNIT)
                 hx = synth.vector_np(9, n, n, dtype)
@@ -529,9 +535,10 @@ def test_trsv_first_cluster_overtaken(b2, ctx, dtype, streams):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
-@pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2)])
+@pytest.mark.parametrize("n,pad", [(1985, 0), (3440, 0), (3441, 0), (4130, 2), (5801, 0)])
 def test_rows_per_block_by_size(b2, ctx, dtype, n, pad):
-    """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, the last one cut."""
+    """symv and trmv's column sums on the tile kernel in blocks of 64, 128 and more rows, off 16-byte boundaries up to
+    the longest of 256, the last one cut."""
     old = b2.get_tuning(b2.KNOB_GATHER), b2.get_tuning(b2.KNOB_TRI_TILE)
     b2.set_tuning(b2.KNOB_GATHER, 0)
     b2.set_tuning(b2.KNOB_TRI_TILE, 0)
