@@ -654,8 +654,9 @@ inline int shape_packs_per_row(int shape) {  // packs of one row segment
 
 // The shape of gemv where rows are read element by element in wide segments.  In double such loads are half as wide, so a
 // thread has twice as many in flight, four rows instead of two (both products, us: 5003 x 3001 45.7 / 42.9, 3001 x 3001 29.4 /
-// 26.1, 757600 x 141 353 / 291, 8001 x 8001 164 / 155; row product 20001 x 1001 with blocks of 64 KB as everywhere 27.5, of 128 KB 29.4).  Small matrices and few rows need the shorter blocks (2001 x 1001
-// 11.4 / 12.5, 33 x 200001 25.9 / 26.5), and so does trmv (column sums n = 3581 26.4 / 27.2, row sums n = 1301 14.2 / 14.7).
+// 26.1, 757600 x 141 353 / 291, 8001 x 8001 164 / 155; row product 20001 x 1001 with blocks of 64 KB as everywhere 27.2, of
+// 128 KB 29.4).  Small matrices and few rows need the shorter blocks (2001 x 1001 11.4 / 12.5, 33 x 200001 25.9 / 26.5), and so
+// does trmv (column sums n = 3581 26.4 / 27.2, row sums n = 1301 14.2 / 14.7).
 constexpr double kWide4Elems = 4e6;
 constexpr int64_t kWide4Rows = 1024;
 template <typename T>

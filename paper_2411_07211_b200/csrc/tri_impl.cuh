@@ -97,9 +97,10 @@ static int symv_impl(const b2_ctx* ctx, int order, int uplo, int64_t n, T alpha,
   }
   // The tile kernel with the shared-memory ring (16-byte aligned matrices) is the faster one while the triangle is small:
   // its persistent blocks start at once, the general tile kernel streams faster.  Upper and lower triangle in turn,
-  // general / ring in us: float n = 4096 31.2 / 24.4, 4608 (40 MiB) 31.1 / 26.9, 4800 (44) 30.6 / 31.8, 5792 36.2 / 39.6,
-  // 8192 54.3 / 57.3; double n = 3008 28.1 / 24.1, 4096 (64) 37.9 / 36.7, 4352 (72) 39.8 / 40.0, 5008 47.3 / 49.8, 8192
-  // 96.9 / 106.3.  Knob value 2 forces the ring kernel at every size (tests).
+  // general / ring, us for the pair: float n = 4096 25.0 / 23.5, 4608 (40 MiB) 26.9 / 27.1, 4800 (44) 27.4 / 31.1, 5792 33.8 / 39.4,
+  // 8192 53.2 / 56.3; double n = 3008 24.8 / 24.6, 4096 (64) 33.1 / 35.5, 4352 (72) 36.0 / 39.2, 5008 44.9 / 49.1, 8192 99.3 /
+  // 103.8.  (The line in double is from before tri_rows, when 4096 took 37.9 / 36.7.)
+  // Knob value 2 forces the ring kernel at every size (tests).
   const bool small = (double)n * (double)n * sizeof(T) / 2 <= symv_ring_bytes(sizeof(T));
   if (knob(kKnobTriTile) == 2 || (knob(kKnobTriTile) == 1 && small)) {
     bool handled = false;

@@ -35,8 +35,8 @@
 // row is solved: its diagonal block is there after 2 to 3 us, asked for ahead of the near tiles and of the cluster's role, and
 // inverted in 1.5 / 5.4 us (trsv_cluster.cuh; 14 us until the inverse was there before both).  From n = 11520 on in
 // double the streaming blocks (112 of them, the clusters leave 20 SMs idle), 5 TB/s.  A copy and both solves, us, before the
-// early start, the inverse by matrix instructions and what NearRows and stream_block say / now: float n = 80 33.5 / 25,
-// 1000 53.5 / 45, 11520 226 / 208, 3001 92.5 / 82, 8191 236 / 229; double 80 27 / 18, 1024 50.3 / 41.2, 9008 274 / 261, 8191 334 / 326.
+// early start, the inverse by matrix instructions and what NearRows and stream_block say / now: float n = 80 33.5 / 24.8,
+// 1000 52.1 / 44.7, 11520 224 / 208, 3001 92.6 / 82, 8191 236 / 230; double 80 27.3 / 18.1, 1024 50.5 / 42.8, 9008 275 / 262, 8191 336 / 329.
 // Against the sub-block kernel of trsv_front.cu, per solve, N / T views, before that: float n = 1024 22.5 / 25.6 us (27 / 27), 11520
 // 104 / 116 us (141 / 134); double n = 1024 24.4 / 24.9 us (32 / 30), 11520 164 / 160 us (238 / 228); rows off 16-byte
 // boundaries, against the block-row kernel: float n = 4097 61 / 63 us (103 / 128), double n = 4097 65 / 67 us (126 / 116).
@@ -373,9 +373,9 @@ __device__ __forceinline__ void stream_block(const Args<T>& p, Block<T>& b, int 
     };
     while (lo < S - 1 && s_last[lo] < j) ++lo;
     // A strip that ends with tile j goes first and without x_(j+1), which the chain has one row later: its sums are due
-    // W rows after x_j.  (With both awaited, every second row of the chain waited for them: n = 11520 215 us a pair of
-    // solves, so 211.  In double the slack is longer, off 16-byte boundaries the strips
-    // take longer, and the second barrier costs more: double n = 9008 261, 266, float n = 8191 236, 244.)
+    // W rows after x_j.  (With both awaited, every second row of the chain waited for them: a pair of solves of n = 11520
+    // took 2 % longer.  In double the slack is longer, off 16-byte boundaries the strips take longer, and the second barrier
+    // costs more: double n = 9008 2 %, float n = 8191 3 % longer with it.)
     const bool alone = sizeof(T) == 4 && AL && s_last[lo] == j;
     const bool second = b.tid >= NB * WPE;  // this thread's word belongs to x_(j+1)
     if (!(alone && second)) receive();
