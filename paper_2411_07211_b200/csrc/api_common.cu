@@ -27,6 +27,7 @@ static int64_t g_knobs[kKnobCount] = {
     /* kKnobTrsvStreams     */ -1,
     /* kKnobGather          */ 1,
     /* kKnobTrsvDebugLate   */ 0,
+    /* kKnobTrsvShortRows   */ -1,
 };
 
 unsigned long long g_launch_count = 0;

@@ -1,6 +1,8 @@
 // Asynchronous copies global -> shared memory and shared-memory barriers (inline PTX).
 #pragma once
 
+#include <cuda.h>  // CUtensorMap (types only: the encoder is fetched from the driver at run time)
+
 #include "common.cuh"
 
 namespace b2 {
@@ -48,6 +50,42 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// One tiled TMA copy: the box of the tensor map at element coordinates (x, y) -> shared memory.
+// x * element size must be a multiple of 16 bytes; what lies outside the tensor arrives as zeros.
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, unsigned long long* bar) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(map), "r"(x), "r"(y), "r"((unsigned)__cvta_generic_to_shared(bar))
+               : "memory");
+}
+
+// Tensor map of the n x n row-major matrix with boxes of box_rows x box_cols.  The encoder lives in the driver; it is looked
+// up once.  false: no encoder, or the matrix does not meet the map's rules (the caller then uses the 16-byte copies).
+template <typename T>
+static bool encode_tile_map(CUtensorMap* map, const T* a, int64_t lda, int64_t n, int box_rows, int box_cols) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static Encode encode = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      fn = nullptr;
+    }
+    return reinterpret_cast<Encode>(fn);
+  }();
+  if (encode == nullptr || n > 0x7fffffff) return false;
+  if ((lda * sizeof(T)) % 16 != 0 || !aligned_to(a, 16)) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)n};
+  const cuuint64_t strides[1] = {(cuuint64_t)lda * sizeof(T)};
+  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUtensorMapDataType dt = sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
+  return encode(map, dt, 2, const_cast<T*>(a), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace b2

@@ -435,7 +435,8 @@ enum Knob {
   kKnobTrsvStreams = 16,       // streaming clusters of the cluster trsv kernel at most (-1: as many as fit)
   kKnobGather = 17,            // gemv / symv / trmv by one cluster per 32 outputs: 0 never, 1 where it is the faster kernel, 2 wherever it can, 3 the same with trmv's late outputs forced
   kKnobTrsvDebugLate = 18,     // test hook: polls for which the first cluster of the cluster trsv kernel waits to be overtaken (0 = none)
-  kKnobCount = 19
+  kKnobTrsvShortRows = 19,     // unknowns up to which the cluster trsv kernel cuts float problems into block rows of 64 (-1: where it is faster)
+  kKnobCount = 20
 };
 int64_t knob(int id);
 

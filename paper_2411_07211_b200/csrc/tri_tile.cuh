@@ -19,8 +19,6 @@
 // read it).
 #pragma once
 
-#include <cuda.h>  // CUtensorMap (types only: the encoder is fetched from the driver at run time)
-
 #include "async_copy.cuh"
 #include "level2.cuh"
 
@@ -95,15 +93,6 @@ __host__ __device__ __forceinline__ void col_range(int J, int64_t n, int nbr, in
   const int64_t c0 = (int64_t)J * TC, c1 = (c0 + TC < n ? c0 + TC : n) - 1;
   *ilo = TRI == TRI_LOWER ? (int)(c0 / kTR) : 0;
   *ihi = TRI == TRI_UPPER ? (int)(c1 / kTR) : nbr - 1;
-}
-
-// One tiled TMA copy: the box of the tensor map at element coordinates (x, y) -> shared memory.
-// x * element size must be a multiple of 16 bytes; what lies outside the tensor arrives as zeros.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-                   (unsigned)__cvta_generic_to_shared(dst)),
-               "l"(map), "r"(x), "r"(y), "r"((unsigned)__cvta_generic_to_shared(bar))
-               : "memory");
 }
 
 // Persistent blocks (one per SM).  Block b takes the units b, b + gridDim, ... of the dense unit
@@ -454,34 +443,6 @@ constexpr size_t tile_smem_bytes() {
                               (COL ? kWarps * (WALK_ROWS ? kUnitMax * TC : TC) : 0));
 }
 
-// Tensor map of the n x n row-major matrix with boxes of one tile (kTR rows x tc columns).  The
-// encoder lives in the driver; it is looked up once.  false: no encoder, or the matrix does not
-// meet the map's rules (the caller then uses the 16-byte copies).
-template <typename T>
-static bool encode_tile_map(CUtensorMap* map, const T* a, int64_t lda, int64_t n, int tc) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static Encode encode = [] {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
-      (void)cudaGetLastError();
-      fn = nullptr;
-    }
-    return reinterpret_cast<Encode>(fn);
-  }();
-  if (encode == nullptr) return false;
-  if ((lda * sizeof(T)) % 16 != 0 || !aligned_to(a, 16)) return false;
-  const cuuint64_t dims[2] = {(cuuint64_t)n, (cuuint64_t)n};
-  const cuuint64_t strides[1] = {(cuuint64_t)lda * sizeof(T)};
-  const cuuint32_t box[2] = {(cuuint32_t)tc, (cuuint32_t)kTR};
-  const cuuint32_t estr[2] = {1, 1};
-  const CUtensorMapDataType dt = sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
-  return encode(map, dt, 2, const_cast<T*>(a), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Launches both kernels.  *handled is false (nothing launched) when the matrix is not 16-byte
 // aligned, too large for the unit table, or the partials do not fit the workspace: the caller
 // then uses the general tile kernel.
@@ -536,7 +497,7 @@ static int tri_tile_run_cap(const Launch& l, const T* a, int64_t lda, int64_t n,
 #ifdef B2_DEBUG_BOUNDS
   bulk = false;  // (a TMA copy cannot be tested address by address: the checking build keeps the 16-byte copies)
 #endif
-  if (bulk) bulk = encode_tile_map<T>(&tmap, a, lda, n, TC);
+  if (bulk) bulk = encode_tile_map<T>(&tmap, a, lda, n, kTR, TC);
   auto kern = bulk ? tri_tile_kernel<T, CAP, ROW, COL, TRI, UNIT, SYM, true> : tri_tile_kernel<T, CAP, ROW, COL, TRI, UNIT, SYM, false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     (void)cudaGetLastError();

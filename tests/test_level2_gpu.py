@@ -428,6 +428,64 @@ def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
 
 
+@pytest.mark.parametrize("dtype,rows,room", [(np.float32, 0, True), (np.float32, 1 << 30, True), (np.float32, 1 << 30, False), (np.float64, -1, False)])
+def test_trsv_cluster_block_rows(b2, dtype, rows, room):
+    """Float in block rows of 128 where it would take 64 and the other way round; block rows of 64 with a workspace that holds the
+    inverses beyond one turn of the cluster and no premultiplied tiles.  One unknown more and less than a block row, than the
+    rows the solving cluster multiplies itself, than a turn; several strips for a streaming block."""
+    nb = 128 if rows == 0 else 64
+    sizes = [(21 * nb - 7) // 4 * 4, 22 * nb + 1] if not room else [nb - 1, nb + 4, 7 * nb, 9 * nb + 1, 17 * nb + 4, 45 * nb - 3]
+    ws = None
+    if not room:  # control block, x and far sums, flags, inverses
+        s = np.dtype(dtype).itemsize
+        ws = 4096 + 2 * 23 * nb * 2 * s + 512 + 7 * nb * nb * s
+    c = b2.Context() if ws is None else b2.Context(workspace_bytes=ws)
+    c.reset()
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+    try:
+        for n, order, trans, uplo in itertools.product(sizes, ORDERS, TRANSES, UPLOS):
+            a = tri_buf(27, n, n, dtype, order, uplo, orc.NON_UNIT)
+            hx = synth.vector_np(9, n, n, dtype)
+            ga, gx = Guarded(a), Guarded(hx)
+            b2.trsv(c, order, uplo, trans, orc.NON_UNIT, n, ga.t, n, gx.t, 1)
+            assert c.device_status() == 0
+            resid, scale = orc.trsv_residual(order, uplo, trans, orc.NON_UNIT, n, a, n, hx, 1, gx.host(), 1)
+            gx.check_guards()
+            assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, order, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_trsv_premultiplied_tile_overflows(b2, ctx, dtype):
+    """Tiles beside the diagonal whose products with the block's inverse are beyond the type, in the cluster's first turn and
+    after it, times unknowns that are zero: the solution is the right-hand side over the diagonal and exact."""
+    small, big = (-60, 90) if dtype == np.float32 else (-600, 500)
+    n = 18 * 64 + 8
+    m = np.diag(np.full(n, 2.0 ** small, dtype=dtype))
+    b = synth.vector_np(3, 1, n, dtype)
+    for k in (1, 17):  # tile (k, k - 1), and zeros for the unknowns it meets
+        m[k * 64:(k + 1) * 64, (k - 1) * 64:k * 64] = 2.0 ** big
+        b[(k - 1) * 64:k * 64] = 0
+    want = b / dtype(2.0 ** small)
+    for flip, order, trans in itertools.product((False, True), ORDERS, TRANSES):  # op(A) lower, upper
+        op = m[::-1, ::-1] if flip else m
+        stored = op if (order == orc.ROW_MAJOR) == (trans == orc.NO_TRANS) else op.T
+        uplo = orc.UPPER if flip != (trans == orc.TRANS) else orc.LOWER
+        da = torch.from_numpy(np.ascontiguousarray(stored).ravel()).cuda()
+        x = torch.from_numpy(b[::-1].copy() if flip else b.copy()).cuda()
+        # (blocks of 64 from the other end: whole when the order is turned round)
+        if flip:
+            da, x, length = da.view(n, n)[8:, 8:].reshape(-1).contiguous(), x[8:].contiguous(), n - 8
+        else:
+            length = n
+        b2.trsv(ctx, order, uplo, trans, orc.NON_UNIT, length, da, length, x, 1)
+        assert ctx.device_status() == 0
+        expect = want[::-1][8:] if flip else want
+        assert np.array_equal(x.cpu().numpy(), expect), (flip, order, trans)
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
