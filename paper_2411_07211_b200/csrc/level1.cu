@@ -136,12 +136,112 @@ __global__ void __launch_bounds__(kThreads) l1_map_unit(Op op, T* __restrict__ x
   }
 }
 
+// ---- unit stride, x and y misaligned differently -------------------------------------------------
+// y is read and written in packs as above, and so is x, in the aligned packs that lie S elements before those of y: a warp's
+// 32 packs of y meet the elements S .. of its first pack of x up to the first S of the pack after its last.  Those S
+// come by element loads, the others change lanes by S shuffles per pack.  Every element belongs to one warp, which alone uses
+// and writes it (the first S elements of the first pack are another's: loaded along, not used).
+//
+// Bound by memory like l1_map_unit; by elements, four times as many loads and stores (two in double), by those: map_route.
+template <typename T, int S>
+struct Shifted {
+  static constexpr int V = VecLen<T>::value;
+  using P = Pack<T, V>;
+  // elements S .. V - 1 of own and 0 .. S - 1 of the next lane's pack; extra: in lane c < S, element c of the pack behind the last
+  __device__ __forceinline__ static P take(const P& own, T extra, int lane) {
+    P r;
+#pragma unroll
+    for (int e = 0; e + S < V; ++e) r.v[e] = own.v[e + S];
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+      const T next = __shfl_down_sync(0xffffffffu, own.v[c], 1), last = __shfl_sync(0xffffffffu, extra, c);
+      r.v[V - S + c] = lane == 31 ? last : next;
+    }
+    return r;
+  }
+  // the way back, to the pack at `at` and, from the last lane, to the one behind it
+  __device__ __forceinline__ static void put(T* at, const P& r, int lane) {
+    P own;
+#pragma unroll
+    for (int e = 0; e + S < V; ++e) own.v[e + S] = r.v[e];
+#pragma unroll
+    for (int c = 0; c < S; ++c) own.v[c] = __shfl_up_sync(0xffffffffu, r.v[V - S + c], 1);
+    if (lane != 0) {
+      st_cs<T, V>(at, own);
+    } else {
+#pragma unroll
+      for (int c = S; c < V; ++c) B2_STORE(at + c, own.v[c]);
+    }
+    if (lane == 31) {
+#pragma unroll
+      for (int c = 0; c < S; ++c) B2_STORE(at + V + c, r.v[V - S + c]);
+    }
+  }
+};
+
+// Packs [head, head + nvec * V) of y, nvec a multiple of 32 (whole warps); the other elements, fewer than kThreads, one by
+// one by the threads of block 0.  xv: the aligned packs of x.
+template <typename T, class Op, int NV, int S>
+__global__ void __launch_bounds__(kThreads) l1_map_shifted(Op op, T* __restrict__ x, T* __restrict__ y, int64_t n, int64_t head,
+                                                           int64_t nvec, int64_t nchunks) {
+  grid_dep_wait();
+  grid_dep_launch();
+  constexpr int V = VecLen<T>::value;
+  using P = Pack<T, V>;
+  using SH = Shifted<T, S>;
+  T* const xv = x + head - S;
+  T* const yv = y + head;
+  const int lane = threadIdx.x & 31;
+  for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
+    const int64_t v0 = chunk * (int64_t)(kThreads * NV) + threadIdx.x;
+    P px[NV], py[NV];
+    T extra[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int64_t v = v0 + (int64_t)k * kThreads;
+      if (v < nvec) {  // (the same for a whole warp)
+        if (Op::RX) {
+          px[k] = ld_cs<T, V>(xv + v * V);
+          extra[k] = ld_el_if<T>(xv + (v - lane + 32) * V + lane, lane < S);
+        }
+        if (Op::RY) py[k] = ld_cs<T, V>(yv + v * V);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int64_t v = v0 + (int64_t)k * kThreads;
+      if (v < nvec) {
+        P xs = {};
+        if (Op::RX) xs = SH::take(px[k], extra[k], lane);
+#pragma unroll
+        for (int q = 0; q < V; ++q) op(xs.v[q], py[k].v[q]);
+        if (Op::WX) SH::put(xv + v * V, xs, lane);
+        if (Op::WY) st_cs<T, V>(yv + v * V, py[k]);
+      }
+    }
+  }
+  if (blockIdx.x == 0) {
+    const int64_t tail0 = head + nvec * V;
+    const int64_t i = (int64_t)threadIdx.x < head ? threadIdx.x : tail0 + (threadIdx.x - head);
+    if (i < n) {
+      T a = T(0), b = T(0);
+      if (Op::RX) a = x[i];
+      if (Op::RY) b = y[i];
+      op(a, b);
+      if (Op::WX) x[i] = a;
+      if (Op::WY) y[i] = b;
+    }
+  }
+}
+
 // Any stride: one element per thread and slot, NE slots in flight.  x and y are the bases
 // from vec_base(), so logical element i is at x[i*incx] for either sign.
-template <typename T, class Op, int NE>
+// UNIT: both increments are 1 (known to the compiler, a third of the instructions goes).
+template <typename T, class Op, int NE, bool UNIT = false>
 __global__ void __launch_bounds__(kThreads) l1_map_strided(Op op, T* __restrict__ x, int64_t incx,
                                                            T* __restrict__ y, int64_t incy, int64_t n,
                                                            int64_t nchunks) {
+  if (UNIT) incx = incy = 1;
   grid_dep_wait();
   grid_dep_launch();
   for (int64_t chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
@@ -481,11 +581,14 @@ __global__ void __launch_bounds__(kThreads) l1_reduce_unit(const T* __restrict__
   reduce_finish<Op, true>(a, partials, ticket, result);
 }
 
-template <typename T, class Op, int NE>
+// UNIT: both increments are 1 (dot of vectors misaligned differently, us, without / with it: float n = 1 million 4.6 / 3.9, 20 million
+// 32.5 / 27.1, double 1 million 5.3 / 4.6).
+template <typename T, class Op, int NE, bool UNIT = false>
 __global__ void __launch_bounds__(kThreads) l1_reduce_strided(const T* __restrict__ x, int64_t incx,
                                                               const T* __restrict__ y, int64_t incy, int64_t n,
                                                               int64_t nchunks, typename Op::Acc* partials,
                                                               unsigned* ticket, typename Op::Out* result) {
+  if (UNIT) incx = incy = 1;
   grid_dep_wait();
   grid_dep_launch();
   using Acc = typename Op::Acc;
@@ -585,6 +688,44 @@ static bool same_head(const T* x, const T* y, bool use_y, int64_t* head) {
   return mx == my;
 }
 
+// Two unit-stride vectors misaligned differently: by elements of any stride, or in shifted packs; by elements of stride 1 what
+// is neither, in float where both vectors are written (dot: always).  Us, by elements / of stride 1 / shifted packs:
+//   float   axpy n = 1 million 3.1 / 2.8 / 2.8, 4 million 8.0 / 6.5 / 6.6, 20 million 42.5 / 38.5 / 36.0; copy 20 million 41.5 / 35.9 / 25.1;
+//           swap 2 million 4.8 / 4.8 / 5.2, 4 million 11.0 / 11.0 / 10.1, 20 million 54 / 60 / 49; rot 2 million 5.8 / 4.9 / 5.2, 4 million 12.3 / 9.9 / 10.0,
+//           20 million 62 / 50 / 49
+//   double  copy 1 million 3.4 / 3.8 / 3.3, 20 million 70 / 72 / 48; axpy 1 million 4.3 / 4.6 / 3.7, 2 million 6.4 / 6.6 / 6.2, 4 million 17.4 / 19.5 / 19.3;
+//           swap 1 million 4.7 / 5.2 / 5.5, 20 million 103 / 99 / 108; rot 4.6 / 5.2 / 6.8, 96 / 97 / 130
+enum MapRoute { kByElements, kByShiftedPacks };
+template <typename T, class Op>
+static MapRoute map_route(int64_t n) {
+  if (n < 1024) return kByElements;  // (one block either way)
+  if (Op::WX) return sizeof(T) == 4 && n >= 3000000 ? kByShiftedPacks : kByElements;
+  return Op::RY && sizeof(T) == 8 && n > 2500000 ? kByElements : kByShiftedPacks;
+}
+
+// Regions of the shifted kernels: y's packs begin at *head, x's S elements before theirs (the return value; elements before x are not
+// touched); whole warps of packs.
+template <typename T>
+static int shifted_regions(const T* x, const T* y, int64_t n, int64_t* head, int64_t* nvec) {
+  constexpr int V = VecLen<T>::value;
+  const int mx = (int)((reinterpret_cast<uintptr_t>(x) % 16) / sizeof(T)), my = (int)((reinterpret_cast<uintptr_t>(y) % 16) / sizeof(T));
+  *head = (V - my) % V;
+  const int s = (int)((mx + *head) % V);
+  if (*head < s) *head += V;
+  *nvec = n > *head ? (n - *head) / V / 32 * 32 : 0;
+  return s;
+}
+
+template <typename T, class Op, int S>
+static void map_shifted(const Launch& l, Op op, int64_t n, T* x, T* y, int64_t head, int64_t nvec, int s) {
+  if constexpr (S < VecLen<T>::value) {
+    if (s != S) return map_shifted<T, Op, S + 1>(l, op, n, x, y, head, nvec, s);
+    constexpr int NV = 4;
+    const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV), grid = nchunks > (1 << 30) ? (1 << 30) : nchunks;
+    launch_chained(l1_map_shifted<T, Op, NV, S>, dim3((unsigned)grid), dim3(kThreads), 0, l.stream, op, x, y, n, head, nvec, nchunks);
+  }
+}
+
 template <typename T, class Op>
 static int run_map(const b2_ctx* ctx, Op op, int64_t n, T* x, int64_t incx, T* y, int64_t incy) {
   Launch l;
@@ -603,10 +744,20 @@ static int run_map(const b2_ctx* ctx, Op op, int64_t n, T* x, int64_t incx, T* y
     const int64_t nchunks = (nvec + kThreads * NV - 1) / (kThreads * NV);
     const int64_t grid = nchunks < 1 ? 1 : (nchunks > (1 << 30) ? (1 << 30) : nchunks);
     launch_chained(l1_map_unit<T, Op, NV>, dim3((unsigned)grid), dim3(kThreads), 0, l.stream, op, x, two ? y : x, n, head, nvec, nchunks);
+  } else if (two && incx == 1 && incy == 1 && map_route<T, Op>(n) == kByShiftedPacks) {
+    int64_t nvec = 0;
+    const int s = shifted_regions(x, y, n, &head, &nvec);
+    if constexpr (two) map_shifted<T, Op, 1>(l, op, n, x, y, head, nvec, s);
   } else {
     constexpr int NE = 8;
     const int64_t nchunks = (n + kThreads * NE - 1) / (kThreads * NE);
     const int64_t grid = nchunks > (1 << 30) ? (1 << 30) : nchunks;
+    if constexpr (two && Op::WX && sizeof(T) == 4) {
+      if (incx == 1 && incy == 1) {
+        launch_chained(l1_map_strided<T, Op, NE, true>, dim3((unsigned)grid), dim3(kThreads), 0, l.stream, op, x, incx, y, incy, n, nchunks);
+        return check_launch();
+      }
+    }
     launch_chained(l1_map_strided<T, Op, NE>, dim3((unsigned)grid), dim3(kThreads), 0, l.stream, op, vec_base(x, n, incx), incx, two ? vec_base(y, n, incy) : x, two ? incy : 1, n, nchunks);
   }
   return check_launch();
@@ -667,6 +818,15 @@ static int run_reduce(const b2_ctx* ctx, int64_t n, const T* x, int64_t incx, co
     const int64_t grid = nchunks < 1 ? 1 : (nchunks > wave ? wave : nchunks);
     launch_chained(l1_reduce_unit<T, Op, NV, 2>, dim3((unsigned)grid), dim3(kThreads), 0, l.stream, x, Op::RY ? y : x, span, head, nvec, nchunks,
                                                                            partials, ticket, result);
+  } else if (Op::RY && incx == 1 && incy == 1) {  // (misaligned differently)
+    if constexpr (Op::RY) {
+      constexpr int NE = 8;
+      const int64_t nchunks = (n + kThreads * NE - 1) / (kThreads * NE);
+      static WaveCache wc;
+      const int wave = one_wave(l1_reduce_strided<T, Op, NE, true>, cap, wc);
+      launch_chained(l1_reduce_strided<T, Op, NE, true>, dim3((unsigned)(nchunks > wave ? wave : nchunks)), dim3(kThreads), 0, l.stream, x, incx, y, incy, n,
+                     nchunks, partials, ticket, result);
+    }
   } else {
     constexpr int NE = Op::RY ? 8 : 16;
     const int64_t nchunks = (n + kThreads * NE - 1) / (kThreads * NE);

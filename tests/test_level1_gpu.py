@@ -90,6 +90,44 @@ def test_map_routines(b2, ctx, dtype, n, incx, incy, offset):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n", [1023, 1024, 1031, 4096, 4103, 8199, 70001])
+def test_different_alignments(b2, ctx, dtype, n):
+    """Two vectors that start at different places between 16-byte boundaries, every pair of places: the last length that goes by
+    elements, whole warps and blocks of packs with every remainder."""
+    v = 16 // np.dtype(dtype).itemsize
+    x, y = _vecs(n, dtype, 300 + n)
+    tdt = torch.float32 if dtype == np.float32 else torch.float64
+    for ox, oy in [(i, j) for i in range(v) for j in range(v) if i != j]:
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        res = torch.full((2,), float("nan"), dtype=tdt, device="cuda")
+        b2.dot(ctx, n, gx.t, 1, gy.t, 1, res[0:1])
+        d, dabs = orc.dot(n, x, 1, y, 1)
+        assert_close(res.cpu().numpy()[0], d, dabs, dtype, "dot")
+        if dtype == np.float32:
+            wide = torch.zeros(1, dtype=torch.float64, device="cuda")
+            b2.dsdot(ctx, n, gx.t, 1, gy.t, 1, wide)
+            d, dabs = orc.dsdot(n, x, 1, y, 1)
+            assert_close(wide.cpu().numpy()[0], d, dabs, np.float64, "dsdot")
+        wx, wy = x.copy(), y.copy()
+        b2.swap(ctx, n, gx.t, 1, gy.t, 1)
+        orc.swap(n, wx, 1, wy, 1)
+        assert np.array_equal(gx.host(), wx) and np.array_equal(gy.host(), wy)
+        b2.axpy(ctx, n, 1.5, gx.t, 1, gy.t, 1)
+        absterms = orc.axpy(n, dtype(1.5), wx, 1, wy, 1)
+        assert_close(gy.host(), wy, absterms, dtype, "axpy")
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        b2.rot(ctx, n, gx.t, 1, gy.t, 1, 0.6, 0.8)
+        wx, wy = x.copy(), y.copy()
+        ax, ay = orc.rot(n, wx, 1, wy, 1, dtype(0.6), dtype(0.8))
+        assert_close(gx.host(), wx, ax, dtype, "rot x"), assert_close(gy.host(), wy, ay, dtype, "rot y")
+        gx.check_guards(), gy.check_guards()
+        before = gx.host()
+        b2.copy(ctx, n, gx.t, 1, gy.t, 1)
+        assert np.array_equal(gy.host(), before) and np.array_equal(gx.host(), before)
+        gx.check_guards(), gy.check_guards()
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n", SIZES + [1 << 20, (1 << 22) + 5])
 @pytest.mark.parametrize("incx,incy", INCS)
 @pytest.mark.parametrize("offset", [0, 1])
