@@ -9,6 +9,7 @@
 #include "level2.cuh"
 #include "gather.cuh"
 #include "tri_tile.cuh"
+#include "trmv_small.cuh"
 
 namespace b2 {
 
@@ -125,6 +126,13 @@ static int trmv_kind(const Launch& l, const L2Args<T>& args, bool unit) {
       const bool room = tri_room(l, args, plan, false);
       const int st = unit ? ga::run<T, Kind<false, true, TRI, true, false>>(l, args, &handled, false, room)
                           : ga::run<T, Kind<false, true, TRI, false, false>>(l, args, &handled, false, room);
+      if (handled) return st;
+    }
+  }
+  if constexpr (ROW) {
+    if ((knob(kKnobTriTile) == 1 && knob(kKnobGather) != 0) || knob(kKnobGather) >= 2) {  // (a forced tile kernel stays forced)
+      bool handled = false;
+      const int st = ts::run<T, TRI>(l, args, unit, &handled);
       if (handled) return st;
     }
   }

@@ -428,6 +428,30 @@ def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("n", [1, 3, 4, 31, 33, 129, 240, 241, 255, 256, 257, 416, 417, 511, 512])
+def test_trmv_one_launch_rows(b2, ctx, dtype, n):
+    """Row sums of small triangles in place and in one launch: one row more and less than a warp, a cluster of 8 and one of 16 has, and
+    the sizes at which the tile kernel takes over; on and off 16-byte boundaries, strided, both triangles and diagonals."""
+    old = b2.get_tuning(b2.KNOB_GATHER)
+    try:
+        for knob, pad, inc, diag in [(1, 0, 1, orc.NON_UNIT), (1, 1, -2, orc.UNIT), (2, -n % 16, 3, orc.UNIT), (2, 3, 1, orc.NON_UNIT)]:
+            b2.set_tuning(b2.KNOB_GATHER, knob)
+            for uplo in UPLOS:
+                a = tri_buf(28, n, n + pad, dtype, orc.ROW_MAJOR, uplo, diag)
+                hx = place(synth.vector_np(9, n, n, dtype), inc)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trmv(ctx, orc.ROW_MAJOR, uplo, orc.NO_TRANS, diag, n, ga.t, n + pad, gx.t, inc)
+                ox = hx.copy()
+                absterms = orc.trmv(orc.ROW_MAJOR, uplo, orc.NO_TRANS, diag, n, a, n + pad, ox, inc)
+                rx = gx.host()
+                assert_close(pick(rx, n, inc), pick(ox, n, inc), absterms, dtype, f"trmv {n} {uplo} {pad}")
+                assert_same_gaps(rx, hx, n, inc)
+                gx.check_guards()
+    finally:
+        b2.set_tuning(b2.KNOB_GATHER, old)
+
+
 @pytest.mark.parametrize("dtype,rows,room", [(np.float32, 0, True), (np.float32, 1 << 30, True), (np.float32, 1 << 30, False), (np.float64, -1, False)])
 def test_trsv_cluster_block_rows(b2, dtype, rows, room):
     """Float in block rows of 128 where it would take 64 and the other way round; block rows of 64 with a workspace that holds the
