@@ -357,7 +357,8 @@ static int launch(const Launch& l, const L2Args<T>& q, bool* handled, bool one_l
 //                   unaligned float 49 MB 22.6 / 22.1, 58 23.2 / 25.5, 74 25.7 / 28.9 (with a copy and the row product), double the
 //                   same on twelve matrices, four views, 5 MB 11.8 - 12.0 / 11.8 - 12.9, 7.2 12.1 - 12.4 / 12.8 - 13.6, 9.7 14.0 - 15.2 /
 //                   14.3 - 15.0, 32 17.1 - 17.9 / 17.9 - 19.4, 98 25.5 - 27.3 / 28.2 - 30.6 (on three 5.8 12.8 / 11.9 - 12.6, 8 equal).
-//   symv            reads its elements twice: float 20 MB 7.9 / 7.6, 24 7.9 / 9.3 (between 6 and 20 within 5 %); double 20
+//   symv            reads its elements twice: float (ring kernel, both triangles) n = 1520 14.2 / 12.6, 1664 12.2 / 12.8, 2048 12.4 /
+//                   13.7, 2100 15.3 / 14.8, 2176 13.6 / 14.5, with room for its partials; double 20 MB
 //                   7.6 / 6.5, 24 7.5 / 7.6; unaligned (both triangles) float 21 MB 20.5 / 19.3, 23 20.5 / 20.5, 29 21.4 / 23.5, 35
 //                   23.0 / 26.6, double 29 22.8 / 19.0, 32 23.1 / 23.0, 35 23.8 / 24.8, 72 32.3 / 35.0.
 // room: whether the tile kernels' partials fit the workspace without much longer blocks; where they do not, this kernel, which
@@ -368,7 +369,7 @@ constexpr int64_t max_mb(bool al, bool room) {
   constexpr bool F = sizeof(T) == 4;
   if (!al && !room && K::SYM) return F ? 85 : 80;
   if (!al && !room && K::TRI != TRI_FULL) return F ? 85 : 101;
-  if (K::SYM) return al ? (F ? 20 : 22) : (F ? 23 : 33);
+  if (K::SYM) return al ? (F ? (room ? 11 : 20) : 22) : (F ? 23 : 33);
   if (K::TRI != TRI_FULL) return al ? (F ? 5 : 18) : (F ? 50 : 7);
   if (K::ROWOUT) return al ? (F ? 24 : 50) : 110;
   return al ? (F ? 17 : 22) : (F ? 35 : 70);

@@ -460,21 +460,29 @@ static int tri_tile_run_cap(const Launch& l, const T* a, int64_t lda, int64_t n,
   args.incx = incx;
   args.nbr = (int)nbr;
   args.nct = (int)nct;
-  // longer units mean fewer partials, fewer reductions and fewer block-wide barriers per tile; a
-  // dozen units per block keep the tail short (measured at 4096 tiles on 148 blocks: units of 2
-  // take symv from 57 / 53 us (upper / lower, float) to 50.5 us, units of 4 to 52 / 50 us)
-  const int64_t tiles = nbr * nct / 2;
-  const int64_t per_block = tiles / sm_count();
-  args.unit = (per_block >= 48 && kUnitMax >= 4) ? 4 : (per_block >= 12 && kUnitMax >= 2) ? 2 : 1;
-  const int64_t forced = knob(kKnobTriTileUnit);
-  if ((forced == 1 || forced == 2 || forced == 4) && forced <= kUnitMax) args.unit = (int)forced;
+  // Longer units mean fewer partials, reductions and block-wide barriers per tile, and a coarser last round: of 1, 2 and 4 tiles the
+  // one with which the busiest block gets the fewest tiles, the longest of several such.  (symv, upper and lower triangle in turn, us, with units
+  // of 1 / 2: float n = 3000 (3 rounds of 1, 2 of 2) 20.1 / 21.1, 4096 (4, 2) 23.7 / 22.6; double 2000 (2, 1) 16.2 / 15.5, 3000 (4, 3) 24.8 / 26.0, 4096 (8, 4)
+  // 36.4 / 33.0.)
   const int nmajor = WALK_ROWS ? args.nbr : args.nct;
-  int ngroups = 0;
-  for (int i = 0; i < nmajor; ++i) {
+  auto groups_of = [&](int i, int unit) {
     int lo, hi;
     if (WALK_ROWS) row_range<TRI, TC>(i, n, args.nct, &lo, &hi);
     else col_range<TRI, TC>(i, n, args.nbr, &lo, &hi);
-    const int ng = hi / args.unit - lo / args.unit + 1;
+    return hi / unit - lo / unit + 1;
+  };
+  const int64_t forced = knob(kKnobTriTileUnit);
+  int64_t least = INT64_MAX;
+  for (int unit = 1; unit <= kUnitMax; unit *= 2) {
+    int64_t units = 0;
+    for (int i = 0; i < nmajor; ++i) units += groups_of(i, unit);
+    const int64_t busiest = (units + sm_count() * kBlocksPerSm - 1) / (sm_count() * kBlocksPerSm) * unit;
+    if (forced == unit || (forced != 1 && forced != 2 && forced != 4 && busiest <= least)) least = busiest, args.unit = unit;
+  }
+  if (args.unit == 0) args.unit = kUnitMax;
+  int ngroups = 0;
+  for (int i = 0; i < nmajor; ++i) {
+    const int ng = groups_of(i, args.unit);
     args.prefix[i + 1] = args.prefix[i] + ng;
     ngroups = ng > ngroups ? ng : ngroups;
   }
