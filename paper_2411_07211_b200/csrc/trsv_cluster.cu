@@ -38,7 +38,7 @@
 // (112 of them, the clusters leave 20 SMs idle), 5 TB/s.
 // A copy and both solves, us, before the block rows of 64 in float, the premultiplied tiles, the tiled copies and the plain
 // shared-memory polls / now: float n = 64 24.2 / 15.4, 192 32.0 / 19.5, 731 (unaligned) 49.0 / 34.2, 1000 44.5 / 34.9, 2322 (unaligned) 71.0 / 62.2,
-// 4448 93.9 / 88.7, 11520 208.8 / 208.0; double 112 19.0 / 16.2, 608 32.9 / 28.8, 1024 42.5 / 36.7, 4224 123.6 / 108.6, 8512 231 / 202, 10752 293 / 268.
+// 4784 101.8 / 94.6, 11520 208.7 / 205.2, 13296 265.9 / 249.7; double 112 19.0 / 16.2, 608 32.9 / 28.8, 1024 42.5 / 36.7, 4224 123.6 / 108.6, 8512 231 / 202, 10752 293 / 268.
 // Slower: double off 16-byte boundaries from 8000 on, 473 / 486 at 10416.
 // Tried: clusters of 8 (column-type views 40 % slower in float: a block's pass over its near tiles takes
 // longer than its turn), the near tiles on the receiving side (0.8 us more per row: the last of them then
