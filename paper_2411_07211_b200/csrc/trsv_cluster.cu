@@ -915,7 +915,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
     }
 #pragma unroll 1
     for (int w = min(W, k); w > first; --w) take(sum_of(w));
-    const T r = (T)(hi + lo);
+    const T r = (T)(isfinite(lo) ? hi + lo : hi);  // (with hi infinite the error is NaN)
     b.rs[b.tid] = k >= first ? r - sum_of(first) : r;
   };
   // Where the words of element i of x_(k-1) lie: what neighbouring lanes read side by side.

@@ -510,6 +510,44 @@ def test_trsv_premultiplied_tile_overflows(b2, ctx, dtype):
         assert np.array_equal(x.cpu().numpy(), expect), (flip, order, trans)
 
 
+# Geometries of the cluster trsv kernel: type, value of the knob that cuts float into block rows of 64, unknowns of a block row.
+TRSV_ROWS = [(np.float32, 0, 128), (np.float32, 1 << 30, 64), (np.float64, -1, 64)]
+
+
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
+@pytest.mark.parametrize("block,length", [(0, 0), (1, 0), (4, 0), (18, 30)])
+def test_trsv_infinite_right_hand_side(b2, ctx, dtype, rows, nb, block, length):
+    """An infinite element of the right-hand side in every place of a block row: that unknown is infinite, the block rows before it are
+    what they are without it, bit for bit, and what follows it is not finite.  In the first rows, in one with sums of rows further
+    back and in the ragged last one."""
+    n, length = 18 * nb + 30, length or nb
+    x = torch.from_numpy(synth.vector_np(9, n, n, dtype)).cuda()
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+    try:
+        for uplo, trans in itertools.product(UPLOS, TRANSES):
+            upper = (uplo == orc.UPPER) == (trans == orc.NO_TRANS)  # of op(A): solved from the last row on
+            a = tri_buf(24, n, n, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+            da, signs = torch.from_numpy(a).cuda(), np.sign(a.reshape(n, n).diagonal())
+
+            def solve(v):
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, da, n, v, 1)
+                assert ctx.device_status() == 0
+                return v.cpu().numpy()
+            whole = solve(x.clone())
+            before = slice(min(n, (block + 1) * nb), n) if upper else slice(0, block * nb)
+            for q in range(length):
+                i = block * nb + (length - 1 - q if upper else q)
+                v = x.clone()
+                v[i] = np.inf if q % 2 else -np.inf
+                want, got = float(v[i]) * signs[i], solve(v)
+                assert got[i] == want, (q, uplo, trans, got[i])
+                assert np.array_equal(got[before], whole[before]), (q, uplo, trans)
+                assert not np.any(np.isfinite(got[:i] if upper else got[i + 1:])), (q, uplo, trans)
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
