@@ -548,6 +548,47 @@ def test_trsv_infinite_right_hand_side(b2, ctx, dtype, rows, nb, block, length):
         b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
 
 
+def _solve_turned(b2, ctx, m, b, want):
+    """op(A) = m in blocks of 64 and one of 8, lower triangular, and turned round, in both orders and stored either way; the last block does
+    not count when it is turned, so that the blocks of 64 are whole from the other end."""
+    n = len(b)
+    for flip, order, trans in itertools.product((False, True), ORDERS, TRANSES):
+        op, rhs, expect = (v[::-1][8:] if flip else v for v in (m[:, ::-1] if flip else m, b, want))
+        if flip:
+            op = op[:, 8:]
+        stored = op if (order == orc.ROW_MAJOR) == (trans == orc.NO_TRANS) else op.T
+        uplo = orc.UPPER if flip != (trans == orc.TRANS) else orc.LOWER
+        length = len(rhs)
+        da = torch.from_numpy(np.ascontiguousarray(stored).ravel()).cuda()
+        x = torch.from_numpy(rhs.copy()).cuda()
+        b2.trsv(ctx, order, uplo, trans, orc.NON_UNIT, length, da, length, x, 1)
+        assert ctx.device_status() == 0
+        assert np.array_equal(x.cpu().numpy(), expect), (flip, order, trans)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("rest", [0.0, 2.0])
+def test_trsv_premultiplied_tile_underflows(b2, ctx, dtype, rest):
+    """Tiles beside the diagonal whose products with the block's inverse are below the type, times large unknowns, in the cluster's
+    first turn and after it; in double also products that vanish beside others that do not.  Powers of two: exact."""
+    diag, tile, size = (84, -66, 100) if dtype == np.float32 else (600, -500, 600)
+    n = 18 * 64 + 8
+    m, b = np.eye(n, dtype=dtype), np.ones(n, dtype=dtype)
+    want = b.copy()
+    for k in (1, 17):
+        here, before = slice(k * 64, (k + 1) * 64), slice((k - 1) * 64, k * 64)
+        m[here, here] *= dtype(2.0 ** diag)
+        m[here, before] = np.diag(np.full(64, 2.0 ** tile))
+        b[before] = want[before] = 2.0 ** size
+        b[here], want[here] = 0, -2.0 ** (tile + size - diag)
+        if rest:  # the first column beside them: a product of ordinary size with an unknown that is small
+            m[here, before][:, 0] = 2.0 ** diag * rest
+            b[(k - 1) * 64] = want[(k - 1) * 64] = 2.0 ** (tile + size - diag)
+            want[here] *= 3
+            want[k * 64] = -2.0 ** (tile + size - diag) * rest
+    _solve_turned(b2, ctx, m, b, want)
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
