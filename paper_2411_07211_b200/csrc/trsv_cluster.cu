@@ -553,7 +553,7 @@ __device__ __forceinline__ void stream_block(const Args<typename G::T>& p, Block
     Tile<G>::store(t, dst, b.tid);
     unsigned have = 0;
     if constexpr (G::PM) {
-      if (pm && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, b.tid)) {
+      if (pm && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, block_len<NB>(p, I), block_len<NB>(p, J), b.tid)) {
         have = 1;
         Tile<G>::from_rows(t, pad.N, Inv<G>::SP, b.tid);
         Tile<G>::store(t, dst + NB * NB, b.tid);
@@ -1088,7 +1088,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
   if (invert_block<G>(at, smem_off(b.red), p.unit, block_len<NB>(p, I0), b.tid)) invert_again<G, COLTYPE, AL>(p, at, I0, b.tid);
   bool have = true;  // (row 0: nothing to multiply)
   if constexpr (G::PM) {
-    if (rank > 0) have = p.pm > 0 && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, b.tid);
+    if (rank > 0) have = p.pm > 0 && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, block_len<NB>(p, I0), block_len<NB>(p, mem_block(p, rank - 1)), b.tid);
   }
   if (early) {
     if (const unsigned t = my_ticket()) {  // another cluster solves
