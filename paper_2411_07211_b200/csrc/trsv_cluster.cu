@@ -310,6 +310,13 @@ struct Tile {
 #pragma unroll
     for (int h = 0; h < CP; ++h) x[h] = *reinterpret_cast<const P*>(vec + h * H + (tid & 15) * V);
   }
+  // The row whose sum a thread ends up with (the first of every few lanes: its owner).
+  __device__ __forceinline__ static int row(int tid) { return (tid >> 4) * RS + (tid & 15) / (16 / RS); }
+  // Where the words of element i of x_(k-1) lie in a solving block's first slots: what neighbouring lanes read side by side.
+  __device__ __forceinline__ static unsigned x_word(unsigned slots, int i) {
+    constexpr int WPE = Words<T>::N;
+    return slots + (unsigned)(((i / H * 2 + i % V * WPE / 2) * 16 + i % H / V) * 16 + i % V * WPE % 2 * 8);
+  }
   // Sums of a thread's rows, in float of even and odd columns side by side (packed multiply-adds).
   struct Sums {
     typename std::conditional<sizeof(T) == 4, u64, T>::type v[RS];
@@ -439,6 +446,59 @@ __device__ __noinline__ void fetch_tile(const Args<typename G::T>& p, unsigned s
   stage_tile<G, COLTYPE, AL>(p.a, p.lda, I, J, block_len<G::NB>(p, I), block_len<G::NB>(p, J), pad.n, tid);
   cp_async_commit();
   cp_async_wait<0>();
+  bar_block();
+}
+
+// inv r and P x may be beyond the type where inv (r - A x) is not, and an infinite element of r must not take those before it along:
+// the unknown that this lane ends up with (Tile) once more, as inv(D_k) (r - A(k, k-1) x_(k-1)) without the zeros of the inverse, by
+// its warp alone, and where it is to go, if `out`.  Where x_(k-1) is not finite it stays what it is, x (what follows is not finite
+// either).  Cold path; offsets in shared memory, own: of the warp; inverse: in global memory, or null: in S.
+template <class G, bool COLTYPE>
+__device__ __noinline__ void solve_apart(const Args<typename G::T>& p, const typename G::T* inverse, unsigned s_off, unsigned slots, unsigned r_off,
+                                         unsigned own_off, int k, int tid, bool transposed, bool out, typename G::T x) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  using T = typename G::T;
+  using TL = Tile<G>;
+  constexpr int NB = G::NB, WPE = Words<T>::N;
+  T* const r = reinterpret_cast<T*>(smem_raw + r_off);
+  T* const own = reinterpret_cast<T*>(smem_raw + own_off);
+  const int I = mem_block(p, k), J = mem_block(p, max(k - 1, 0)), li = block_len<NB>(p, I), lj = k > 0 ? block_len<NB>(p, J) : 0, lane = tid & 31;
+  u64 wd[WPE];
+  double before[NB / 32];
+  bool finite = true;
+#pragma unroll
+  for (int c = 0; c < NB / 32; ++c) {
+    ld_slot(TL::x_word(slots, lane + 32 * c), wd);
+    before[c] = k > 0 ? (double)decode(wd, T(0)) : 0.;
+    finite = finite && isfinite(before[c]);
+  }
+  if (__all_sync(0xffffffffu, finite)) {
+#pragma unroll 8
+    for (int i = 0; i < NB; ++i) {
+      double s = 0.;
+#pragma unroll
+      for (int c = 0; c < NB / 32; ++c) {
+        const int j = lane + 32 * c;
+        const int64_t m = (int64_t)I * NB + i, q = (int64_t)J * NB + j;
+        if (i < li && j < lj) s += (double)__ldg(p.a + (COLTYPE ? q * p.lda + m : m * p.lda + q)) * before[c];
+      }
+      s = cross_group_sum<1>(s);
+      if (lane == 0) own[i] = (T)((double)r[i] - s);
+    }
+    __syncwarp();
+    typename TL::P inv[TL::NPK], v[TL::CP];
+    if (inverse) TL::load(inv, inverse, tid);
+    else TL::inverse(inv, reinterpret_cast<const typename G::Wide*>(smem_raw + s_off), transposed, tid);
+    TL::load_r(v, own, transposed, tid);
+    x = TL::triangle(inv, v, transposed, tid);
+  }
+  const int row = TL::row(tid);
+  encode(x, (unsigned)k + 2u, wd);
+  st_slot_if(out && k + 1 < p.K, map_remote(TL::x_word(slots, row), (unsigned)((k + 1) % kCS)), wd);
+  if (out) r[NB + row] = x;  // (x of the row)
+  encode(x, p.tag, wd);
+  st_gpu_if(out, p.xbuf + ((int64_t)k * NB + row) * WPE, wd);
+  st_val_if(out && row < li, p.x + ((int64_t)I * NB + min(row, li - 1)) * p.incx, x);
   bar_block();
 }
 
@@ -748,7 +808,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
   const Scratchpad<G> pad(b.big + Smem<G>::NEAR_ELEMS);  // behind the near-tile ring
   const unsigned at = smem_off(pad.S);
   const int rg = b.tid >> 4, cg = b.tid & 15;
-  const int row = rg * RS + cg / (16 / RS);        // the row whose sum this lane ends up with
+  const int row = TL::row(b.tid);
   const bool owner = cg % (16 / RS) == 0;
   const bool transposed = Diag<G, COLTYPE, AL>::transposed(p.backward);
 
@@ -918,8 +978,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
     const T r = (T)(isfinite(lo) ? hi + lo : hi);  // (with hi infinite the error is NaN)
     b.rs[b.tid] = k >= first ? r - sum_of(first) : r;
   };
-  // Where the words of element i of x_(k-1) lie: what neighbouring lanes read side by side.
-  auto x_word = [&](int i) { return slots + (unsigned)(((i / H * 2 + i % V * WPE / 2) * 16 + i % H / V) * 16 + i % V * WPE % 2 * 8); };
+  auto x_word = [&](int i) { return TL::x_word(slots, i); };
   // This thread's words of x_(k-1) as the neighbour stored them, and whether all are there.
   auto look_at_x = [&](u64 (&w)[CP][4], int k) {
     bool ok = true;
@@ -948,12 +1007,12 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
   // What lies between the arrival of u_1 (x_(k-1)) and the departure of the next block's runs twice, the first time
   // without its effects while the row still waits for its sums: code that has not run for microseconds is
   // fetched at a third of the speed at which it executes (u_1 to u_1 0.85 us -> 0.55 us in float).
-  // have: nxt is premultiplied; later: near tiles to ask for once x_k is out
-  auto solve_row = [&](int k, bool have, int later) {
+  // have: nxt is premultiplied; later: near tiles to ask for once x_k is out; inverse: where inv came from, null: from S
+  auto solve_row = [&](int k, bool have, int later, const T* inverse) {
     const int I = mem_block(p, k), li = block_len<NB>(p, I), wn = near_width(k);
     u64 wd[WPE];
     P cur[NPK], xv[CP];
-    bool pub = false;
+    bool pub = false, fine = true;
     T xk;
     // The first near tile is waited for least of all: in registers ahead of the chain.
     const unsigned next = map_remote(G::PM ? x_word(row) : slots + (unsigned)(row * WPE * 8), (unsigned)((k + 1) % kCS));
@@ -990,6 +1049,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
           TL::multiply(beside, nxt, xv);
           xk = TL::reduce(sums, beside, b.lane);
         }
+        fine = !have || is_finite(xk);
         encode(xk, (unsigned)k + 2u, wd);
       } else {
         TL::multiply(sums, inv, xv);
@@ -1003,13 +1063,19 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
         pub = go && !*b.wt.dead && k != p.debug_skip;
         encode(u1, (unsigned)k + 2u, wd);
       }
-      st_slot_if(pub && owner && k + 1 < p.K, next, wd);
+      // (what is not finite goes out after another look, below)
+      st_slot_if(pub && owner && fine && k + 1 < p.K, next, wd);
       if (G::PM && go && owner) b.xs[row] = xk;
       encode(xk, p.tag, wd);
-      st_gpu_if(pub && owner, p.xbuf + ((int64_t)k * NB + row) * WPE, wd);
-      st_val_if(pub && owner && row < li, p.x + ((int64_t)I * NB + min(row, li - 1)) * p.incx, xk);
+      st_gpu_if(pub && owner && fine, p.xbuf + ((int64_t)k * NB + row) * WPE, wd);
+      st_val_if(pub && owner && fine && row < li, p.x + ((int64_t)I * NB + min(row, li - 1)) * p.incx, xk);
     }
-    if (G::PM) bar_block();
+    if constexpr (G::PM) {
+      const bool again = pub && owner && !fine;
+      __syncwarp();
+      if (__builtin_expect(__syncthreads_or((int)again), 0))
+        solve_apart<G, COLTYPE>(p, inverse, at, slots, smem_off(b.rs), smem_off(b.red + b.warp * NB), k, b.tid, transposed, again, xk);
+    }
 #pragma unroll 1
     for (int i = 0; i < later; ++i) produce();
 #pragma unroll 1
@@ -1153,7 +1219,7 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
       st_gpu_if(!*b.wt.dead, p.far + ((int64_t)k * NB + b.warp * kStrip + b.lane) * WPE, wd);
     }
     if (k + kCS >= p.K) b.leave(p.ctl);
-    solve_row(k, have, rest - now);
+    solve_row(k, have, rest - now, formed ? nullptr : src);
   }
   cp_async_wait<0>();
   drain();

@@ -589,6 +589,73 @@ def test_trsv_premultiplied_tile_underflows(b2, ctx, dtype, rest):
     _solve_turned(b2, ctx, m, b, want)
 
 
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS[1:])
+@pytest.mark.parametrize("block,length", [(0, 64), (1, 64), (4, 64), (7, 30)])
+def test_trsv_infinite_element_and_its_block_row(b2, ctx, dtype, rows, nb, block, length):
+    """In rows of 64 the unknowns of the same block row that precede an infinite element of the right-hand side do not depend on it
+    either."""
+    n = 7 * nb + 30
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+    try:
+        for uplo, trans, q in itertools.product(UPLOS, TRANSES, (1, 18, length - 1)):
+            upper = (uplo == orc.UPPER) == (trans == orc.NO_TRANS)  # of op(A): solved from the last row on
+            a, hx = tri_buf(24, n, n, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT), synth.vector_np(9, n, n, dtype)
+            i = block * nb + (length - 1 - q if upper else q)
+            hx[i] = np.inf
+            ga, gx = Guarded(a), Guarded(hx)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n, gx.t, 1)
+            assert ctx.device_status() == 0
+            got = gx.host()
+            gx.check_guards()
+            assert got[i] == np.inf * np.sign(a.reshape(n, n)[i, i]), (q, uplo, trans, got[i])
+            resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n, hx, 1, got, 1)
+            before = slice(i + 1, n) if upper else slice(0, i)
+            assert np.all(resid[before] <= TOL[np.dtype(dtype)] * scale[before]), (q, uplo, trans)
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_trsv_product_beyond_the_type(b2, ctx, dtype):
+    """Right-hand sides and tiles whose products with the block's inverse are beyond the type, while the right-hand side less the tile's
+    product with the unknowns before is not.  Powers of two: exact."""
+    diag, size, rest = (-100, 33, 12) if dtype == np.float32 else (-750, 300, 250)
+    n = 18 * 64 + 8
+    m, b = np.eye(n, dtype=dtype), np.ones(n, dtype=dtype)
+    want = b.copy()
+    for k in (1, 17):
+        here, before = slice(k * 64, (k + 1) * 64), slice((k - 1) * 64, k * 64)
+        m[here, here] *= dtype(2.0 ** diag)
+        m[here, before] = np.eye(64)
+        b[before] = want[before] = 2.0 ** size
+        b[here], want[here] = 2.0 ** size + 2.0 ** rest, 2.0 ** (rest - diag)
+    _solve_turned(b2, ctx, m, b, want)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("at", [0, 70, 300])
+def test_trsv_solution_overflows(b2, ctx, dtype, at):
+    """A solution beyond the type from one unknown on, with a matrix and a right-hand side that make all later ones infinite of the same
+    sign by substitution: so they are in its block row and the next, and nowhere finite."""
+    n = 18 * 64 + 30
+    big = np.finfo(dtype).maxexp - 4
+    for pad in (0, 1):
+        m = np.full((n, n), -1.0 / n, dtype=dtype)
+        m[np.diag_indices(n)] = 1
+        b = np.ones(n, dtype=dtype)
+        m[at, at], b[at] = 2.0 ** -big, 2.0 ** 40
+        for uplo, trans in ((orc.LOWER, orc.NO_TRANS), (orc.UPPER, orc.TRANS)):
+            buf = np.zeros((n, n + pad), dtype=dtype)
+            buf[:, :n] = m if trans == orc.NO_TRANS else m.T
+            ga, gx = Guarded(buf), Guarded(b)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+            assert ctx.device_status() == 0
+            got = gx.host()
+            assert np.all(np.isfinite(got[:at])) and not np.any(np.isfinite(got[at:])), (pad, uplo, trans)
+            assert np.all(got[at:(at // 64 + 2) * 64] == np.inf), (pad, uplo, trans, np.flatnonzero(got[at:] != np.inf)[:4])
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
