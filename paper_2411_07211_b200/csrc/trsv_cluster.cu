@@ -1434,7 +1434,11 @@ int trsv_cluster_try(const Launch& l, bool coltype, bool backward, bool unit, in
   } else {
     const bool al = aligned_to(a, 16) && lda % 4 == 0;
     const int64_t k = knob(kKnobTrsvShortRows), most = k >= 0 ? k : al ? kShortRows : kShortRowsUnaligned;
-    return n <= most ? run_cluster<F64>(l, coltype, p, handled) : run_cluster<F128>(l, coltype, p, handled);
+    if (n <= most) {  // (rows of 128 need no inverses where rows of 64 need too many for the workspace)
+      const int st = run_cluster<F64>(l, coltype, p, handled);
+      if (st != B2_STATUS_OK || *handled) return st;
+    }
+    return run_cluster<F128>(l, coltype, p, handled);
   }
 }
 

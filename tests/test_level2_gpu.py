@@ -656,6 +656,28 @@ def test_trsv_solution_overflows(b2, ctx, dtype, at):
             assert np.all(got[at:(at // 64 + 2) * 64] == np.inf), (pad, uplo, trans, np.flatnonzero(got[at:] != np.inf)[:4])
 
 
+def test_trsv_small_workspace_takes_longer_rows(b2):
+    """Float with the smallest workspace, where the inverses of block rows of 64 do not fit and rows of 128 need none: these, bit for bit."""
+    small = b2.Context(workspace_bytes=b2.lib().b2_workspace_min_bytes())
+    small.reset()
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    for n, pad in [(1412, 0), (1601, 2), (2048, 0), (2047, 0)]:
+        for uplo, trans in itertools.product(UPLOS, TRANSES):
+            ga = Guarded(tri_buf(29, n, n + pad, np.float32, orc.ROW_MAJOR, uplo, orc.NON_UNIT))
+            hx, got = synth.vector_np(9, n, n, np.float32), []
+            for rows in (old, 0):
+                b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+                try:
+                    gx = Guarded(hx)
+                    b2.trsv(small, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                finally:
+                    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+                assert small.device_status() == 0
+                gx.check_guards()
+                got.append(gx.host())
+            assert np.array_equal(*got), (n, pad, uplo, trans)
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
