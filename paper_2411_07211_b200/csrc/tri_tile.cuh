@@ -463,7 +463,10 @@ static int tri_tile_run_cap(const Launch& l, const T* a, int64_t lda, int64_t n,
   // Longer units mean fewer partials, reductions and block-wide barriers per tile, and a coarser last round: of 1, 2 and 4 tiles the
   // one with which the busiest block gets the fewest tiles, the longest of several such.  (symv, upper and lower triangle in turn, us, with units
   // of 1 / 2: float n = 3000 (3 rounds of 1, 2 of 2) 20.1 / 21.1, 4096 (4, 2) 23.7 / 22.6; double 2000 (2, 1) 16.2 / 15.5, 3000 (4, 3) 24.8 / 26.0, 4096 (8, 4)
-  // 36.4 / 33.0.)
+  // 36.4 / 33.0.  trmv's float row sums with a strided x, of 1 / 2 / 4: n = 8192 52.5 / 54.2 / 53.3, 10240 76.6 / 78.6 / 77.9, 12800 115.7 / 118.4 / 117.3,
+  // 16384 187.0 / 187.9 / 185.3.)  Rows off 32-byte boundaries share sectors between neighbouring tiles, which two of them in one block
+  // read once: units of 2 from 8 tiles per block on (the same product: n = 6500 43.1 / 41.5 / 43.1, 8100 60.3 / 57.0 / 57.5, 12500
+  // 124.2 / 115.9 / 124.5, 14500 168.5 / 152.5 / 163.2, 16100 203.9 / 184.7 / 194.8).  Only units whose partials fit the workspace count.
   const int nmajor = WALK_ROWS ? args.nbr : args.nct;
   auto groups_of = [&](int i, int unit) {
     int lo, hi;
@@ -471,25 +474,25 @@ static int tri_tile_run_cap(const Launch& l, const T* a, int64_t lda, int64_t n,
     else col_range<TRI, TC>(i, n, args.nbr, &lo, &hi);
     return hi / unit - lo / unit + 1;
   };
-  const int64_t forced = knob(kKnobTriTileUnit);
+  const int64_t blocks = sm_count() * kBlocksPerSm, forced = knob(kKnobTriTileUnit);
+  const bool shared = forced == 0 && (lda * sizeof(T)) % 32 != 0 && nbr * nct / 2 >= 8 * blocks;
   int64_t least = INT64_MAX;
+  size_t row_bytes = 0, col_bytes = 0;
   for (int unit = 1; unit <= kUnitMax; unit *= 2) {
     int64_t units = 0;
-    for (int i = 0; i < nmajor; ++i) units += groups_of(i, unit);
-    const int64_t busiest = (units + sm_count() * kBlocksPerSm - 1) / (sm_count() * kBlocksPerSm) * unit;
-    if (forced == unit || (forced != 1 && forced != 2 && forced != 4 && busiest <= least)) least = busiest, args.unit = unit;
+    int most = 0;
+    for (int i = 0; i < nmajor; ++i) {
+      const int ng = groups_of(i, unit);
+      units += ng;
+      most = ng > most ? ng : most;
+    }
+    const size_t rb = ROW ? ((size_t)most * n * sizeof(T) + 255) / 256 * 256 : 0, cb = COL ? (size_t)(WALK_ROWS ? args.nbr : most) * n * sizeof(T) : 0;
+    if (rb + cb > l.scratch_bytes) continue;
+    const int64_t busiest = forced == unit || (shared && unit == 2) ? 0 : (units + blocks - 1) / blocks * unit;
+    if (busiest <= least) least = busiest, args.unit = unit, args.ngroups = most, row_bytes = rb, col_bytes = cb;
   }
-  if (args.unit == 0) args.unit = kUnitMax;
-  int ngroups = 0;
-  for (int i = 0; i < nmajor; ++i) {
-    const int ng = groups_of(i, args.unit);
-    args.prefix[i + 1] = args.prefix[i] + ng;
-    ngroups = ng > ngroups ? ng : ngroups;
-  }
-  args.ngroups = ngroups;
-  const size_t row_bytes = ROW ? ((size_t)ngroups * n * sizeof(T) + 255) / 256 * 256 : 0;
-  const size_t col_bytes = COL ? (size_t)(WALK_ROWS ? args.nbr : ngroups) * n * sizeof(T) : 0;
-  if (row_bytes + col_bytes > l.scratch_bytes) return B2_STATUS_OK;
+  if (args.unit == 0) return B2_STATUS_OK;
+  for (int i = 0; i < nmajor; ++i) args.prefix[i + 1] = args.prefix[i] + groups_of(i, args.unit);
   args.rowpart = reinterpret_cast<T*>(l.scratch);
   args.colpart = reinterpret_cast<T*>(l.scratch + row_bytes);
   args.alpha = alpha;

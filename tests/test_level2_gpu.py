@@ -678,6 +678,31 @@ def test_trsv_small_workspace_takes_longer_rows(b2):
             assert np.array_equal(*got), (n, pad, uplo, trans)
 
 
+@pytest.mark.parametrize("n,room,unit", [(6000, 320 << 10, 4), (2304, 230 << 10, 4), (6500, 0, 2)])
+def test_ring_units(b2, ctx, n, room, unit):
+    """trmv's float row sums with a strided x and symv on the ring kernel, bit for bit as with units of so many tiles: with a workspace that
+    holds the partials of units of four only, and on rows off 32-byte boundaries."""
+    c = b2.Context(workspace_bytes=4096 + room) if room else ctx
+    c.reset()
+    old = b2.get_tuning(b2.KNOB_TRI_TILE_UNIT)
+    for uplo in UPLOS:
+        ga = Guarded(tri_buf(26, n, n, np.float32, orc.ROW_MAJOR, uplo, orc.NON_UNIT))
+        x, y, got = place(synth.vector_np(7, n, n, np.float32), 2), synth.vector_np(8, n, n, np.float32), []
+        for where, asked in ((c, 0), (ctx, unit)):
+            b2.set_tuning(b2.KNOB_TRI_TILE_UNIT, asked)
+            try:
+                gx, gy = Guarded(x), Guarded(y)
+                if n == 2304:
+                    b2.symv(where, orc.ROW_MAJOR, uplo, n, 1.25, ga.t, n, gx.t, 2, 0.5, gy.t, 1)
+                else:
+                    b2.trmv(where, orc.ROW_MAJOR, uplo, orc.NO_TRANS, orc.NON_UNIT, n, ga.t, n, gx.t, 2)
+            finally:
+                b2.set_tuning(b2.KNOB_TRI_TILE_UNIT, old)
+            gx.check_guards(), gy.check_guards()
+            got += [gx.host(), gy.host()]
+        assert np.array_equal(got[0], got[2], equal_nan=True) and np.array_equal(got[1], got[3]), uplo
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
