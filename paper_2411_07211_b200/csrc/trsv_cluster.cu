@@ -76,7 +76,8 @@ struct Args {
   T* winv;           // [K - kCS][1 or 2][NB * NB] inverses of the diagonal blocks beyond the first kCS (and premultiplied tiles), as
                      // the solving blocks' threads hold them (Tile)
   u64* flags;        // [K] call tag once winv[k] is complete, below it whether there is a premultiplied tile
-  int pm;            // tiles are premultiplied: 1 in the first kCS rows, 2 in all
+  int pm;            // tiles are premultiplied: 1 in the first kCS rows, 2 also beyond them from row pm_from on
+  int pm_from;
   unsigned* ctl;
   int K;             // block rows
   int H;             // streaming blocks of the grid
@@ -591,7 +592,7 @@ __device__ __forceinline__ void stream_block(const Args<typename G::T>& p, Block
     const Scratchpad<G> pad(reinterpret_cast<unsigned char*>(b.big) + Smem<G>::STREAM - Smem<G>::SCRATCH);
     const unsigned at = smem_off(pad.S);
     const int I = mem_block(p, k), J = mem_block(p, k - 1);
-    const bool pm = G::PM && p.pm > 1;
+    const bool room = G::PM && p.pm > 1, pm = room && k >= p.pm_from;
     if constexpr (G::PM) {
       if (pm) stage_tile<G, COLTYPE, AL>(p.a, p.lda, I, J, block_len<NB>(p, I), block_len<NB>(p, J), pad.n, b.tid);
     }
@@ -607,7 +608,7 @@ __device__ __forceinline__ void stream_block(const Args<typename G::T>& p, Block
     bar_block();
     if (invert_block<G>(at, smem_off(b.red), p.unit, block_len<NB>(p, I), b.tid)) invert_again<G, COLTYPE, AL>(p, at, I, b.tid);
     const bool transposed = Diag<G, COLTYPE, AL>::transposed(p.backward);
-    T* dst = p.winv + (int64_t)(k - kCS) * NB * NB * (pm ? 2 : 1);
+    T* dst = p.winv + (int64_t)(k - kCS) * NB * NB * (room ? 2 : 1);
     typename Tile<G>::P t[Tile<G>::NPK];
     Tile<G>::inverse(t, pad.S, transposed, b.tid);
     Tile<G>::store(t, dst, b.tid);
@@ -1359,10 +1360,12 @@ struct Scratch {
   }
 };
 
-// Block rows up to which tiles beyond the first turn are premultiplied off 16-byte boundaries: further on the chain waits for the
-// streaming blocks, which have that to do first (us, without / with it: double n = 4001 146.9 / 140.9, 8001 321.0 / 321.1, 10001 434 / 440;
-// aligned 10000 286 / 276).
-constexpr int64_t kPremultiplyUnaligned = 144;
+// Last block rows whose tiles beyond the first turn are premultiplied off 16-byte boundaries.  There the streaming blocks, which have
+// that to do first, are the slower ones while many strips need each tile; the chain waits for them and has time for two products.
+// (Double, mean of four views, us a solve, all / none / the last 40 / 56 / 72 premultiplied: n = 7001 134.7 / 139.5 / 135.1 / 134.1 / 134.2, 8001 161.8 /
+// 166.7 / 159.3 / 158.7 / 161.4, 10001 222.9 / 225.3 / 219.9 / 219.4 / 220.2, 11519 287.3 / 287.9 / 284.5 / 283.2 / 283.6.  The first 72 rows of 110 premultiplied
+// instead of the last: 138.6.)
+constexpr int kPremultiplyLast = 56;
 
 // Block rows from which tiles are premultiplied: with fewer the chain is shorter than what that takes.  (A copy and both solves, us,
 // without / with it: float n = 100 17.1 / 20.0, 200 20.8 / 22.3, 380 24.3 / 24.3, 450 31.0 / 29.1, 600 31.4 / 28.5; double 100 16.9 / 18.3, 250
@@ -1379,7 +1382,8 @@ static int run_cluster(const Launch& l, bool coltype, Args<typename G::T>& p, bo
   const Scratch<G> w(K);
   if (w.inverses > l.scratch_bytes) return B2_STATUS_OK;
   const bool al = aligned_to(p.a, 16) && p.lda % G::V == 0;
-  p.pm = K < kPremultiplyFrom<typename G::T> ? 0 : w.total <= l.scratch_bytes && (al || K <= kPremultiplyUnaligned) ? 2 : 1;
+  p.pm = K < kPremultiplyFrom<typename G::T> ? 0 : w.total <= l.scratch_bytes ? 2 : 1;
+  p.pm_from = al ? 0 : (int)K - kPremultiplyLast;
   p.xbuf = reinterpret_cast<u64*>(l.scratch);
   p.far = reinterpret_cast<u64*>(l.scratch + w.words);
   p.flags = reinterpret_cast<u64*>(l.scratch + 2 * w.words);

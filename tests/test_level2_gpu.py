@@ -703,6 +703,26 @@ def test_ring_units(b2, ctx, n, room, unit):
         assert np.array_equal(got[0], got[2], equal_nan=True) and np.array_equal(got[1], got[3]), uplo
 
 
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS[1:])
+def test_trsv_premultiplied_last_rows(b2, ctx, dtype, rows, nb):
+    """Off 16-byte boundaries only the last block rows' tiles are premultiplied: one more block row than beyond the first turn and those,
+    and several; ragged, from either end."""
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+    try:
+        for n, uplo, trans in [(73 * nb - 1, orc.LOWER, orc.NO_TRANS), (76 * nb + 5, orc.LOWER, orc.TRANS)]:
+            a = tri_buf(30, n, n | 1, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+            hx = synth.vector_np(9, n, n, dtype)
+            ga, gx = Guarded(a), Guarded(hx)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n | 1, gx.t, 1)
+            assert ctx.device_status() == 0
+            resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n | 1, hx, 1, gx.host(), 1)
+            gx.check_guards()
+            assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("extra", [0, 400 << 10])
 def test_small_workspace_off_boundaries(b2, dtype, extra):
