@@ -1394,10 +1394,11 @@ static int run_cluster(const Launch& l, bool coltype, Args<typename G::T>& p, bo
 }
 
 // Unknowns up to which float takes the short block rows: the start costs half as much (an inverse 3300 cycles instead of
-// 10600) and a row 0.5 us instead of 0.8, but there are twice as many.  A copy and both solves, us, rows of 128 / 64: n = 500
-// 36.5 / 27.2, 1000 42.2 / 34.9, 2000 53.9 / 52.9, 2600 60.5 / 61.2, 3200 67.3 / 69.8; off 16-byte boundaries, where the longer
-// rows' tiles take long to copy, 1000 56.7 / 40.6, 4001 112 / 97, 6001 176 / 168, 7306 201 / 209, 8001 231 / 243.
-constexpr int64_t kShortRows = 2560, kShortRowsUnaligned = 6144;
+// 10600) and a row 0.5 us instead of 0.8, but there are twice as many.  A copy and both solves, us, rows of 128 / 64 (row-major; column-major):
+// n = 1024 37.4 / 35.6; 39.6 / 36.6, 1536 44.0 / 45.1; 46.3 / 46.0, 2048 51.5 / 54.1; 54.0 / 54.8, 2560 58.2 / 62.6; 60.4 / 63.4; off 16-byte boundaries, where the longer
+// rows' tiles take long to copy, 1001 47.2 / 38.3; 49.2 / 38.8, 4001 95.3 / 88.6; 98.7 / 89.4, 4601 105.5 / 103.5; 110.5 / 105.1, 4801 (72 rows of 64 have two strips
+// for some streaming blocks) 110.4 / 118.7; 114.7 / 118.9, 5301 122.8 / 129.1; 127.9 / 132.2.  (The error against a solve in double is 4 to 9 % smaller in rows of 128.)
+constexpr int64_t kShortRows = 1536, kShortRowsUnaligned = 4608;
 
 }  // namespace tc
 
