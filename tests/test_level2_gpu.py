@@ -373,57 +373,76 @@ def test_cut_longest_column_tile(b2, ctx, dtype, n, pad, rows):
         b2.set_tuning(b2.KNOB_TRI_ROWS, old[2])
 
 
-@pytest.mark.parametrize("dtype", DTYPES)
+# Geometries of the cluster trsv kernel: type, value of the knob that cuts float into block rows of 64, unknowns of a block row.
+TRSV_ROWS = [(np.float32, 0, 128), (np.float32, 1 << 30, 64), (np.float64, -1, 64)]
+
+
+def trsv_near(dtype, nb, aligned):
+    """Rows behind the front whose tiles the solving cluster multiplies itself (off 16-byte boundaries: of 15 block rows at most)."""
+    return (6 if nb == 128 else 8) if aligned else (3 if nb == 128 else 4)
+
+
+@pytest.fixture
+def trsv_rows(b2, rows):
+    """The knob that cuts float into block rows of 64 at the value of the test's parameter `rows`."""
+    old = b2.get_tuning(b2.KNOB_TRSV_SHORT_ROWS)
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, rows)
+    yield
+    b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
+
+
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1, 0])
-def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
-    """The cluster kernel at its edges: one unknown more and less than a block row, than the rows the solving
+def test_trsv_cluster_kernel(b2, ctx, dtype, rows, nb, streams, trsv_rows):
+    """The cluster kernel at its edges, in rows of 128 and of 64: one unknown more and less than a block row, than the rows the solving
     cluster multiplies itself, than one turn of the cluster; more strips than streaming blocks; with all
     streaming clusters, with one, and with none (the solving cluster then does their work)."""
-    nb, near, cs = (128, 4, 16) if dtype == np.float32 else (64, 6, 16)
-    sizes = [1, nb, nb + 1, (near + 1) * nb, (near + 1) * nb + 1, cs * nb - 1, cs * nb + 3]
-    if streams != 0:
-        sizes += [(cs + near + 2) * nb + 5] if streams == 1 else [(2 * cs + 7) * nb + 5, 70 * nb]
-    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    cs, old = 16, b2.get_tuning(b2.KNOB_TRSV_STREAMS)
     b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
     try:
-        for n, pad in itertools.product(sizes, (0, 1)):
-            for uplo, trans in itertools.product(UPLOS, TRANSES):
+        for aligned in (True, False):
+            near = trsv_near(dtype, nb, aligned)
+            sizes = [1, nb, nb + 1, (near + 1) * nb, (near + 1) * nb + 1, cs * nb - 1, cs * nb + 3]
+            if streams != 0:
+                sizes += [(cs + near + 2) * nb + 5] if streams == 1 else [(2 * cs + 7) * nb + 5, 70 * nb]
+            for n, uplo, trans in itertools.product(sizes, UPLOS, TRANSES):
+                lda, inc = ((n + 3) // 4 * 4, 1) if aligned else (n | 1, -2)
                 diag = orc.UNIT if n % 2 else orc.NON_UNIT
-                a = tri_buf(22, n, n + pad, dtype, orc.ROW_MAJOR, uplo, diag)
-                hx = place(synth.vector_np(9, n, n, dtype), -2 if pad else 1)
+                a = tri_buf(22, n, lda, dtype, orc.ROW_MAJOR, uplo, diag)
+                hx = place(synth.vector_np(9, n, n, dtype), inc)
                 ga, gx = Guarded(a), Guarded(hx)
-                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, diag, n, ga.t, n + pad, gx.t, -2 if pad else 1)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, diag, n, ga.t, lda, gx.t, inc)
                 assert ctx.device_status() == 0
                 rx = gx.host()
                 gx.check_guards()
-                inc = -2 if pad else 1
-                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, diag, n, a, n + pad, hx, inc, rx, inc)
-                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, diag, n, a, lda, hx, inc, rx, inc)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, aligned, uplo, trans, np.max(resid / scale))
     finally:
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
 
 
-@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1])
-def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
+def test_trsv_cluster_last_tiles(b2, ctx, dtype, rows, nb, streams, trsv_rows):
     """Solves whose strips end with the first and with the second tile of a pair (the streaming blocks take tiles in
-    pairs), whole and ragged, on and off 16-byte boundaries (one near row fewer in float); with one strip for each streaming
+    pairs), whole and ragged, on and off 16-byte boundaries (fewer near rows there); with one strip for each streaming
     block and, on one cluster of them, with several."""
-    nb, near = (128, 4) if dtype == np.float32 else (64, 6)
     old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
     b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
     try:
-        for n, pad in [((near + 2) * nb - 4, 0), ((near + 3) * nb, 0), ((near + 4) * nb + 4, 4), (near * nb + 1, 0), ((near + 3) * nb - 1, 2),
-                       ((near + 9) * nb, 0), ((near + 10) * nb + 4, 0)]:
-            for uplo, trans in itertools.product(UPLOS, TRANSES):
-                a = tri_buf(23, n, n + pad, dtype, orc.COL_MAJOR, uplo, orc.NON_UNIT)
+        for aligned in (True, False):
+            near = trsv_near(dtype, nb, aligned)
+            for n, uplo, trans in itertools.product([(near + 2) * nb - 4, (near + 3) * nb, (near + 4) * nb + 4, near * nb + 1, (near + 3) * nb - 1, (near + 9) * nb,
+                                                     (near + 10) * nb + 4], UPLOS, TRANSES):
+                lda = (n + 3) // 4 * 4 if aligned else n | 1
+                a = tri_buf(23, n, lda, dtype, orc.COL_MAJOR, uplo, orc.NON_UNIT)
                 hx = synth.vector_np(9, n, n, dtype)
                 ga, gx = Guarded(a), Guarded(hx)
-                b2.trsv(ctx, orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                b2.trsv(ctx, orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, lda, gx.t, 1)
                 assert ctx.device_status() == 0
-                resid, scale = orc.trsv_residual(orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n + pad, hx, 1, gx.host(), 1)
+                resid, scale = orc.trsv_residual(orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, a, lda, hx, 1, gx.host(), 1)
                 gx.check_guards()
-                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, aligned, uplo, trans, np.max(resid / scale))
     finally:
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
 
@@ -508,10 +527,6 @@ def test_trsv_premultiplied_tile_overflows(b2, ctx, dtype):
         assert ctx.device_status() == 0
         expect = want[::-1][8:] if flip else want
         assert np.array_equal(x.cpu().numpy(), expect), (flip, order, trans)
-
-
-# Geometries of the cluster trsv kernel: type, value of the knob that cuts float into block rows of 64, unknowns of a block row.
-TRSV_ROWS = [(np.float32, 0, 128), (np.float32, 1 << 30, 64), (np.float64, -1, 64)]
 
 
 @pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
@@ -779,13 +794,12 @@ def test_trsv_divides_by_the_diagonal(b2, ctx, dtype, n, power):
             assert np.array_equal(gx.host(), want), (lda, uplo, trans)
 
 
-@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
-def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, bad):
+def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, rows, nb, bad, trsv_rows):
     """An infinite or NaN element of the matrix in a diagonal block: the unknowns that the solve reaches before it do not depend
     on it.  The element lies beside the diagonal, on it, and in the lower left part of a block of every level of the
     inversion; in a whole block, in one that the streaming blocks invert and in the ragged last one."""
-    nb = 128 if dtype == np.float32 else 64
     n = 18 * nb + 44
     places = [(1, 0), (3, 1), (7, 0), (7, 6), (7, 7), (12, 3), (15, 2), (23, 16), (30, 9), (39, 37), (45, 45), (63, 1), (61, 35)]
     if nb == 128:
@@ -805,26 +819,27 @@ def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, bad):
             assert np.all(resid[before] <= TOL[np.dtype(dtype)] * scale[before]), (block, row, col, uplo, trans)
 
 
-@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1])
-def test_trsv_first_cluster_overtaken(b2, ctx, dtype, streams):
+def test_trsv_first_cluster_overtaken(b2, ctx, dtype, rows, nb, streams, trsv_rows):
     """The first cluster, whose blocks have staged their diagonal blocks by then, draws a ticket other than the first and
     streams: with fewer block rows than blocks in a cluster, with more, ragged, on and off 16-byte boundaries."""
-    nb, near = (128, 4) if dtype == np.float32 else (64, 6)
     old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
     b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
     b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 1 << 16)  # (polls; the other clusters draw their tickets within a hundred)
     try:
-        for n, pad in [((near + 3) * nb, 0), ((near + 4) * nb + 1, 0), (18 * nb + 4, 0), (21 * nb + 3, 2)]:
-            for uplo, trans in itertools.product(UPLOS, TRANSES):
-                a = tri_buf(25, n, n + pad, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+        for aligned in (True, False):
+            near = trsv_near(dtype, nb, aligned)
+            for n, uplo, trans in itertools.product([(near + 3) * nb, (near + 4) * nb + 1, 18 * nb + 4, 21 * nb + 3], UPLOS, TRANSES):
+                lda = (n + 3) // 4 * 4 if aligned else n | 1
+                a = tri_buf(25, n, lda, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
                 hx = synth.vector_np(9, n, n, dtype)
                 ga, gx = Guarded(a), Guarded(hx)
-                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, lda, gx.t, 1)
                 assert ctx.device_status() == 0
                 gx.check_guards()
-                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n + pad, hx, 1, gx.host(), 1)
-                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, lda, hx, 1, gx.host(), 1)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, aligned, uplo, trans, np.max(resid / scale))
     finally:
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
         b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 0)
