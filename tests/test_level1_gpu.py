@@ -127,6 +127,44 @@ def test_different_alignments(b2, ctx, dtype, n):
         gx.check_guards(), gy.check_guards()
 
 
+@pytest.mark.parametrize("n", [2999999, 3000000, 3001367])
+def test_different_alignments_of_long_vectors(b2, ctx, n):
+    """swap, rot and rotm in float around the length from which both vectors are written in shifted packs, every pair of places between
+    16-byte boundaries: the last packs end inside a block's, inside a warp's and where they may."""
+    x, y = _vecs(n, np.float32, 17)
+    param = [-1.0, 0.5, -0.25, 1.5, 2.0]
+    rx, ry, mx, my = x.copy(), y.copy(), x.copy(), y.copy()
+    ax, ay = orc.rot(n, rx, 1, ry, 1, np.float32(0.6), np.float32(0.8))
+    bx, by = orc.rotm(n, mx, 1, my, 1, np.array(param, dtype=np.float32))
+    for ox, oy in [(i, j) for i in range(4) for j in range(4) if i != j]:
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        b2.swap(ctx, n, gx.t, 1, gy.t, 1)
+        assert np.array_equal(gx.host(), y) and np.array_equal(gy.host(), x)
+        gx.check_guards(), gy.check_guards()
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        b2.rot(ctx, n, gx.t, 1, gy.t, 1, 0.6, 0.8)
+        assert_close(gx.host(), rx, ax, np.float32, "rot x"), assert_close(gy.host(), ry, ay, np.float32, "rot y")
+        gx.check_guards(), gy.check_guards()
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        b2.rotm(ctx, n, gx.t, 1, gy.t, 1, param)
+        assert_close(gx.host(), mx, bx, np.float32, "rotm x"), assert_close(gy.host(), my, by, np.float32, "rotm y")
+        gx.check_guards(), gy.check_guards()
+
+
+@pytest.mark.parametrize("n", [2500000, 2500001, 2500127])
+def test_different_alignments_of_long_vectors_double(b2, ctx, n):
+    """axpy in double on both sides of the length from which it goes by elements."""
+    x, y = _vecs(n, np.float64, 18)
+    want = y.copy()
+    absterms = orc.axpy(n, 1.5, x, 1, want, 1)
+    for ox, oy in ((0, 1), (1, 0)):
+        gx, gy = Guarded(x, ox), Guarded(y, oy)
+        b2.axpy(ctx, n, 1.5, gx.t, 1, gy.t, 1)
+        assert_close(gy.host(), want, absterms, np.float64, "axpy")
+        assert np.array_equal(gx.host(), x)
+        gx.check_guards(), gy.check_guards()
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("n", SIZES + [1 << 20, (1 << 22) + 5])
 @pytest.mark.parametrize("incx,incy", INCS)
