@@ -76,7 +76,7 @@ struct Args {
   T* winv;           // [K - kCS][1 or 2][NB * NB] inverses of the diagonal blocks beyond the first kCS (and premultiplied tiles), as
                      // the solving blocks' threads hold them (Tile)
   u64* flags;        // [K] call tag once winv[k] is complete, below it whether there is a premultiplied tile
-  int pm;            // tiles are premultiplied: 1 in the first kCS rows, 2 also beyond them from row pm_from on
+  int pm;            // tiles are premultiplied: 1 in the first kCS rows but the very first, 2 also beyond them from row pm_from on
   int pm_from;
   unsigned* ctl;
   int K;             // block rows
@@ -896,11 +896,14 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
     }
   };
 
+  // The chain is at the first rows before their tiles are premultiplied.  (A copy and two solves, us, from row 1 / 3 on: double n = 608 29.5 /
+  // 28.4, 1024 37.5 / 36.9, 2048 59.2 / 58.2; float 1000 35.3 / 34.1, 1500 45.4 / 43.7.)
+  const bool premultiplied = G::PM && p.pm > 0 && rank >= 3;
   P inv[NPK], nxt[NPK];  // inv(D_k), and beside it inv(D_k) A(k, k-1) -- or that tile, or A(k+1, k) where tiles are not premultiplied
   // The tile at positions (i, j) of the solve order -> nxt.
   auto load_tile = [&](int i, int j) {
     if constexpr (G::PM) {  // (where it is not premultiplied)
-      if (p.pm > 0 || i != rank) fetch_tile<G, COLTYPE, AL>(p, at, mem_block(p, i), mem_block(p, j), b.tid);
+      if (premultiplied || i != rank) fetch_tile<G, COLTYPE, AL>(p, at, mem_block(p, i), mem_block(p, j), b.tid);
       if constexpr (COLTYPE) TL::from_columns(nxt, pad.n, Inv<G>::SP, b.tid, [](const T* q) { return *reinterpret_cast<const P*>(q); });
       else TL::from_rows(nxt, pad.n, Inv<G>::SP, b.tid);
     } else {
@@ -1150,12 +1153,12 @@ __device__ __forceinline__ unsigned solve_block(const Args<typename G::T>& p, Bl
 #pragma unroll 1
   for (int i = 0; i < EARLY; ++i) produce();
   cp_async_wait<TMA ? 0 : EARLY>();
-  pad.arrived(rank > 0 && p.pm > 0, b.tid);
+  pad.arrived(premultiplied, b.tid);
   bar_block();
   if (invert_block<G>(at, smem_off(b.red), p.unit, block_len<NB>(p, I0), b.tid)) invert_again<G, COLTYPE, AL>(p, at, I0, b.tid);
   bool have = true;  // (row 0: nothing to multiply)
   if constexpr (G::PM) {
-    if (rank > 0) have = p.pm > 0 && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, block_len<NB>(p, I0), block_len<NB>(p, mem_block(p, rank - 1)), b.tid);
+    if (rank > 0) have = premultiplied && !premultiply<G, COLTYPE>(at, smem_off(pad.N), transposed, block_len<NB>(p, I0), block_len<NB>(p, mem_block(p, rank - 1)), b.tid);
   }
   if (early) {
     if (const unsigned t = my_ticket()) {  // another cluster solves

@@ -508,7 +508,7 @@ def test_trsv_premultiplied_tile_overflows(b2, ctx, dtype):
     n = 18 * 64 + 8
     m = np.diag(np.full(n, 2.0 ** small, dtype=dtype))
     b = synth.vector_np(3, 1, n, dtype)
-    for k in (1, 17):  # tile (k, k - 1), and zeros for the unknowns it meets
+    for k in (1, 4, 17):  # tile (k, k - 1), and zeros for the unknowns it meets
         m[k * 64:(k + 1) * 64, (k - 1) * 64:k * 64] = 2.0 ** big
         b[(k - 1) * 64:k * 64] = 0
     want = b / dtype(2.0 ** small)
@@ -590,7 +590,7 @@ def test_trsv_premultiplied_tile_underflows(b2, ctx, dtype, rest):
     n = 18 * 64 + 8
     m, b = np.eye(n, dtype=dtype), np.ones(n, dtype=dtype)
     want = b.copy()
-    for k in (1, 17):
+    for k in (1, 4, 17):
         here, before = slice(k * 64, (k + 1) * 64), slice((k - 1) * 64, k * 64)
         m[here, here] *= dtype(2.0 ** diag)
         m[here, before] = np.diag(np.full(64, 2.0 ** tile))
@@ -639,7 +639,7 @@ def test_trsv_product_beyond_the_type(b2, ctx, dtype):
     n = 18 * 64 + 8
     m, b = np.eye(n, dtype=dtype), np.ones(n, dtype=dtype)
     want = b.copy()
-    for k in (1, 17):
+    for k in (1, 4, 17):
         here, before = slice(k * 64, (k + 1) * 64), slice((k - 1) * 64, k * 64)
         m[here, here] *= dtype(2.0 ** diag)
         m[here, before] = np.eye(64)
