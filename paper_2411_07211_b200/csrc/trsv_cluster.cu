@@ -12,16 +12,20 @@
 //     x_k stored straight into the shared memory of the block that owns row k + 1, and then
 //     u   = A(k+w, k) x_k, w = 2 .. W          into those of the blocks that own rows k + w (the tiles through a
 //                                              ring that one tiled copy per tile fills; off 16-byte boundaries by elements)
-//     Between x_(k-1)'s arrival in row k and x_k's departure lie one register product and its reduction.  Block rows of 128
-//     have no registers for P_k: there u_1 travels, and two products and two block barriers stand in the chain.
+//     Between x_(k-1)'s arrival in row k and x_k's departure lie one register product and its reduction.  In block rows of 128 the
+//     solving blocks' shared memory has no room to premultiply beside the near tiles: there u_1 travels, and two products and two
+//     block barriers stand in the chain.
 //   streaming block: 32-row strips of op(A), dealt out cyclically; at each step it multiplies the tiles
 //     (strip, j), (strip, j + 1) of each of its strips that still needs them by x_j and x_(j+1) and keeps
 //     the sums in registers.  Tile data does not depend on the solve, so a ring of 192 KB is always in
 //     flight: every thread copies exactly the packs it later reads, so the ring needs no barrier.  A strip
 //     of row k is complete after x(k-W-1); its sums are published W steps before the chain needs them,
 //     which hides the two trips through L2.
-//   The streaming blocks first invert the diagonal blocks of the rows beyond the first kCS and premultiply the tiles beside them.
-//   Where P_k is not finite, or the workspace has no room for it, row k's block keeps A(k, k-1) itself and multiplies twice.
+//   The streaming blocks first invert the diagonal blocks of the rows beyond the first kCS and premultiply the tiles beside them
+//   (off 16-byte boundaries those of the last rows, where it pays).
+// Where P_k is not finite or has lost digits, where the workspace has no room for it and in rows 1 and 2, which the chain reaches
+// first, row k's block keeps A(k, k-1) itself and multiplies twice.  An unknown that comes out infinite or NaN is formed once more in
+// that way before it is sent on.
 // The blocks of the first cluster start as solving ones -- they request and invert their diagonal blocks -- before they know
 // their ticket; the others draw theirs a little later, and if the first cluster is late, one of them solves.
 //
@@ -32,14 +36,15 @@
 // the work of a streaming cluster that has not started yet itself, in the same order of additions.
 //
 // What bounds it: the chain, 0.6 us per block row of 64 in double and 0.5 in float (from x_k to the next: 0.2 us into the neighbour,
-// 0.1 us of multiply-adds, 0.1 us of shuffles; from x_k by way of u_2 to x_(k+2) 0.55 us and as much again), 0.8 to 0.95 us per row of 128, after 7
-// us until the second row is solved: 1.4 us until the diagonal block is there, 1.9 the inverse, 2.1 the premultiplication, 1 us of loads
+// 0.1 us of multiply-adds, 0.1 us of shuffles; from x_k by way of u_2 to x_(k+2) 0.55 us and as much again), 0.8 to 0.95 us per row of 128, after
+// the start: 1.4 us until the diagonal block is there, 1.9 the inverse, 1 us of loads, and from row 3 on 2.1 the premultiplication
 // (block rows of 128: 5.5 us the inverse).  From n = 11520 on in double, and off 16-byte boundaries from 8000 on, the streaming blocks
 // (112 of them, the clusters leave 20 SMs idle), 5 TB/s.
 // A copy and both solves, us, before the block rows of 64 in float, the premultiplied tiles, the tiled copies and the plain
-// shared-memory polls / now: float n = 64 24.2 / 15.4, 192 32.0 / 19.5, 731 (unaligned) 49.0 / 34.2, 1000 44.5 / 34.9, 2322 (unaligned) 71.0 / 62.2,
-// 4784 101.8 / 94.6, 11520 208.7 / 205.2, 13296 265.9 / 249.7; double 112 19.0 / 16.2, 608 32.9 / 28.8, 1024 42.5 / 36.7, 4224 123.6 / 108.6, 8512 231 / 202, 10752 293 / 268.
-// Slower: double off 16-byte boundaries from 8000 on, 473 / 486 at 10416.
+// shared-memory polls / now: float n = 64 24.4 / 17.1, 192 29.9 / 19.0, 731 (unaligned) 45.9 / 31.9, 1000 45.1 / 34.6, 2048 53.7 / 50.8, 2322 (unaligned) 69.3 / 61.1,
+// 4784 94.9 / 88.1, 11520 207.9 / 204.3, 13296 265 / 249; double 112 19.4 / 16.9, 608 32.7 / 28.7, 1024 42.2 / 36.7, 4224 118.8 / 104.2, 8512 229 / 206, 10417
+// (unaligned) 479 / 474, 10752 291 / 271.  Slower: double off 16-byte boundaries, n = 4873 165.6 / 167.8, 8801 377 / 388; a first pass in double, whose matrix and code
+// are not in L2, n = 300 39.1 / 42.4, 608 41 / 45, 1024 51.3 / 53.3, 1601 71.5 / 78 (but 2048 79.2 / 74.6; float 1000 55.2 / 49.5).
 // Tried: clusters of 8 (column-type views 40 % slower in float: a block's pass over its near tiles takes
 // longer than its turn), the near tiles on the receiving side (0.8 us more per row: the last of them then
 // stands in the chain), one tile per ring slot (streaming alone 84 us instead of 51 us at n = 11520), the start's code run once on
