@@ -391,9 +391,39 @@ def trsv_rows(b2, rows):
     b2.set_tuning(b2.KNOB_TRSV_SHORT_ROWS, old)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("streams", [-1, 1, 0])
+def test_trsv_cluster_kernel(b2, ctx, dtype, streams):
+    """The cluster kernel at its edges: one unknown more and less than a block row, than the rows the solving
+    cluster multiplies itself, than one turn of the cluster; more strips than streaming blocks; with all
+    streaming clusters, with one, and with none (the solving cluster then does their work)."""
+    nb, near, cs = (128, 4, 16) if dtype == np.float32 else (64, 6, 16)
+    sizes = [1, nb, nb + 1, (near + 1) * nb, (near + 1) * nb + 1, cs * nb - 1, cs * nb + 3]
+    if streams != 0:
+        sizes += [(cs + near + 2) * nb + 5] if streams == 1 else [(2 * cs + 7) * nb + 5, 70 * nb]
+    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
+    try:
+        for n, pad in itertools.product(sizes, (0, 1)):
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                diag = orc.UNIT if n % 2 else orc.NON_UNIT
+                a = tri_buf(22, n, n + pad, dtype, orc.ROW_MAJOR, uplo, diag)
+                hx = place(synth.vector_np(9, n, n, dtype), -2 if pad else 1)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, diag, n, ga.t, n + pad, gx.t, -2 if pad else 1)
+                assert ctx.device_status() == 0
+                rx = gx.host()
+                gx.check_guards()
+                inc = -2 if pad else 1
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, diag, n, a, n + pad, hx, inc, rx, inc)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
+
+
 @pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1, 0])
-def test_trsv_cluster_kernel(b2, ctx, dtype, rows, nb, streams, trsv_rows):
+def test_trsv_cluster_kernel_in_rows(b2, ctx, dtype, rows, nb, streams, trsv_rows):
     """The cluster kernel at its edges, in rows of 128 and of 64: one unknown more and less than a block row, than the rows the solving
     cluster multiplies itself, than one turn of the cluster; more strips than streaming blocks; with all
     streaming clusters, with one, and with none (the solving cluster then does their work)."""
@@ -421,9 +451,34 @@ def test_trsv_cluster_kernel(b2, ctx, dtype, rows, nb, streams, trsv_rows):
         b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("streams", [-1, 1])
+def test_trsv_cluster_last_tiles(b2, ctx, dtype, streams):
+    """Solves whose strips end with the first and with the second tile of a pair (the streaming blocks take tiles in
+    pairs), whole and ragged, on and off 16-byte boundaries (one near row fewer in float); with one strip for each streaming
+    block and, on one cluster of them, with several."""
+    nb, near = (128, 4) if dtype == np.float32 else (64, 6)
+    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
+    try:
+        for n, pad in [((near + 2) * nb - 4, 0), ((near + 3) * nb, 0), ((near + 4) * nb + 4, 4), (near * nb + 1, 0), ((near + 3) * nb - 1, 2),
+                       ((near + 9) * nb, 0), ((near + 10) * nb + 4, 0)]:
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                a = tri_buf(23, n, n + pad, dtype, orc.COL_MAJOR, uplo, orc.NON_UNIT)
+                hx = synth.vector_np(9, n, n, dtype)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trsv(ctx, orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                assert ctx.device_status() == 0
+                resid, scale = orc.trsv_residual(orc.COL_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n + pad, hx, 1, gx.host(), 1)
+                gx.check_guards()
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
+
+
 @pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1])
-def test_trsv_cluster_last_tiles(b2, ctx, dtype, rows, nb, streams, trsv_rows):
+def test_trsv_cluster_last_tiles_in_rows(b2, ctx, dtype, rows, nb, streams, trsv_rows):
     """Solves whose strips end with the first and with the second tile of a pair (the streaming blocks take tiles in
     pairs), whole and ragged, on and off 16-byte boundaries (fewer near rows there); with one strip for each streaming
     block and, on one cluster of them, with several."""
@@ -508,7 +563,7 @@ def test_trsv_premultiplied_tile_overflows(b2, ctx, dtype):
     n = 18 * 64 + 8
     m = np.diag(np.full(n, 2.0 ** small, dtype=dtype))
     b = synth.vector_np(3, 1, n, dtype)
-    for k in (1, 4, 17):  # tile (k, k - 1), and zeros for the unknowns it meets
+    for k in (1, 17):  # tile (k, k - 1), and zeros for the unknowns it meets
         m[k * 64:(k + 1) * 64, (k - 1) * 64:k * 64] = 2.0 ** big
         b[(k - 1) * 64:k * 64] = 0
     want = b / dtype(2.0 ** small)
@@ -579,6 +634,16 @@ def _solve_turned(b2, ctx, m, b, want):
         b2.trsv(ctx, order, uplo, trans, orc.NON_UNIT, length, da, length, x, 1)
         assert ctx.device_status() == 0
         assert np.array_equal(x.cpu().numpy(), expect), (flip, order, trans)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_trsv_premultiplied_tile_overflows_in_row_4(b2, ctx, dtype):
+    """The same in a row of the cluster's first turn whose tile is premultiplied (those of rows 1 and 2 are not)."""
+    small, big = (-60, 90) if dtype == np.float32 else (-600, 500)
+    n = 18 * 64 + 8
+    m, b = np.diag(np.full(n, 2.0 ** small, dtype=dtype)), synth.vector_np(3, 1, n, dtype)
+    m[256:320, 192:256], b[192:256] = 2.0 ** big, 0
+    _solve_turned(b2, ctx, m, b, b / dtype(2.0 ** small))
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
@@ -794,9 +859,35 @@ def test_trsv_divides_by_the_diagonal(b2, ctx, dtype, n, power):
             assert np.array_equal(gx.host(), want), (lda, uplo, trans)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, bad):
+    """An infinite or NaN element of the matrix in a diagonal block: the unknowns that the solve reaches before it do not depend
+    on it.  The element lies beside the diagonal, on it, and in the lower left part of a block of every level of the
+    inversion; in a whole block, in one that the streaming blocks invert and in the ragged last one."""
+    nb = 128 if dtype == np.float32 else 64
+    n = 18 * nb + 44
+    places = [(1, 0), (3, 1), (7, 0), (7, 6), (7, 7), (12, 3), (15, 2), (23, 16), (30, 9), (39, 37), (45, 45), (63, 1), (61, 35)]
+    if nb == 128:
+        places += [(76, 65), (99, 10), (100, 63), (127, 64), (127, 127)]
+    for block, length, where in ((1, nb, places), (17, nb, places[3::4]), (18, 44, [(43, 40), (20, 3), (43, 43)])):
+        for (row, col), uplo, trans in itertools.product(where, UPLOS, TRANSES):
+            upper = (uplo == orc.UPPER) == (trans == orc.NO_TRANS)  # of op(A): solved from the last row on
+            i, j = (block * nb + (length - 1 - q if upper else q) for q in (row, col))
+            a = tri_buf(24, n, n, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+            a.reshape(n, n)[(i, j) if trans == orc.NO_TRANS else (j, i)] = bad
+            hx = synth.vector_np(9, n, n, dtype)
+            ga, gx = Guarded(a), Guarded(hx)
+            b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n, gx.t, 1)
+            assert ctx.device_status() == 0
+            resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n, hx, 1, gx.host(), 1)
+            before = slice(i + 1, n) if upper else slice(0, i)
+            assert np.all(resid[before] <= TOL[np.dtype(dtype)] * scale[before]), (block, row, col, uplo, trans)
+
+
 @pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
-def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, rows, nb, bad, trsv_rows):
+def test_trsv_keeps_what_precedes_a_bad_element_in_rows(b2, ctx, dtype, rows, nb, bad, trsv_rows):
     """An infinite or NaN element of the matrix in a diagonal block: the unknowns that the solve reaches before it do not depend
     on it.  The element lies beside the diagonal, on it, and in the lower left part of a block of every level of the
     inversion; in a whole block, in one that the streaming blocks invert and in the ragged last one."""
@@ -819,9 +910,34 @@ def test_trsv_keeps_what_precedes_a_bad_element(b2, ctx, dtype, rows, nb, bad, t
             assert np.all(resid[before] <= TOL[np.dtype(dtype)] * scale[before]), (block, row, col, uplo, trans)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("streams", [-1, 1])
+def test_trsv_first_cluster_overtaken(b2, ctx, dtype, streams):
+    """The first cluster, whose blocks have staged their diagonal blocks by then, draws a ticket other than the first and
+    streams: with fewer block rows than blocks in a cluster, with more, ragged, on and off 16-byte boundaries."""
+    nb, near = (128, 4) if dtype == np.float32 else (64, 6)
+    old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
+    b2.set_tuning(b2.KNOB_TRSV_STREAMS, streams)
+    b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 1 << 16)  # (polls; the other clusters draw their tickets within a hundred)
+    try:
+        for n, pad in [((near + 3) * nb, 0), ((near + 4) * nb + 1, 0), (18 * nb + 4, 0), (21 * nb + 3, 2)]:
+            for uplo, trans in itertools.product(UPLOS, TRANSES):
+                a = tri_buf(25, n, n + pad, dtype, orc.ROW_MAJOR, uplo, orc.NON_UNIT)
+                hx = synth.vector_np(9, n, n, dtype)
+                ga, gx = Guarded(a), Guarded(hx)
+                b2.trsv(ctx, orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, ga.t, n + pad, gx.t, 1)
+                assert ctx.device_status() == 0
+                gx.check_guards()
+                resid, scale = orc.trsv_residual(orc.ROW_MAJOR, uplo, trans, orc.NON_UNIT, n, a, n + pad, hx, 1, gx.host(), 1)
+                assert np.all(resid <= TOL[np.dtype(dtype)] * scale), (n, pad, uplo, trans, np.max(resid / scale))
+    finally:
+        b2.set_tuning(b2.KNOB_TRSV_STREAMS, old)
+        b2.set_tuning(b2.KNOB_TRSV_DEBUG_LATE, 0)
+
+
 @pytest.mark.parametrize("dtype,rows,nb", TRSV_ROWS)
 @pytest.mark.parametrize("streams", [-1, 1])
-def test_trsv_first_cluster_overtaken(b2, ctx, dtype, rows, nb, streams, trsv_rows):
+def test_trsv_first_cluster_overtaken_in_rows(b2, ctx, dtype, rows, nb, streams, trsv_rows):
     """The first cluster, whose blocks have staged their diagonal blocks by then, draws a ticket other than the first and
     streams: with fewer block rows than blocks in a cluster, with more, ragged, on and off 16-byte boundaries."""
     old = b2.get_tuning(b2.KNOB_TRSV_STREAMS)
