@@ -434,7 +434,7 @@ def test_trsv_cluster_kernel_in_rows(b2, ctx, dtype, rows, nb, streams, trsv_row
             near = trsv_near(dtype, nb, aligned)
             sizes = [1, nb, nb + 1, (near + 1) * nb, (near + 1) * nb + 1, cs * nb - 1, cs * nb + 3]
             if streams != 0:
-                sizes += [(cs + near + 2) * nb + 5] if streams == 1 else [(2 * cs + 7) * nb + 5, 70 * nb]
+                sizes += [(cs + near + 2) * nb + 5]
             for n, uplo, trans in itertools.product(sizes, UPLOS, TRANSES):
                 lda, inc = ((n + 3) // 4 * 4, 1) if aligned else (n | 1, -2)
                 diag = orc.UNIT if n % 2 else orc.NON_UNIT
